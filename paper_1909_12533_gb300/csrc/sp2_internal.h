@@ -179,7 +179,7 @@ struct TcLaunch {
   int64_t n;
   int nb, nsr, k, words;
   int32_t* err;
-  void* scratch;             // nsuper * tc_tile_slots() * 128 * 128 int64 (epilogue staging per CTA)
+  void* scratch;             // nsuper * 128 * 128 int64 (epilogue staging per CTA)
   int seg_min;               // K loops of at least this many steps are accumulated in segments (0: never)
   int seg_ksteps = 16;       // K steps per segment (8 or 16)
   unsigned long long wait_ns = 2000000000ull;   // limit of every bounded wait in the kernel
@@ -195,7 +195,6 @@ size_t panel_record_bytes(int k);
 // operand's panel records (spos: the operand's record offsets, nsr x words + 1)
 cudaError_t launch_row_sq_sum(const int32_t* spos, int nsr, int words, const double* rsq, int64_t n, double* dsq,
                               cudaStream_t st);
-int tc_tile_slots();   // tiles in flight between the producer and the epilogue of k_square_tc
 // report_range: also report an out-of-range element (error bit 4) without one
 // being present (self-test of the error path); rsq (nullptr: skipped): 128
 // squared row sums per record, FP64, unscaled

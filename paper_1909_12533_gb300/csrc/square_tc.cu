@@ -165,24 +165,29 @@ __device__ __forceinline__ long long f32_int_to_ll(float x) {
   return (long long)ih * 2048 + il;
 }
 
-// The per-CTA fixed-point staging (two 128 KB slots per CTA, 38 MB in all) is
-// written and read back by the same CTA within one tile: an L2 evict_last
-// policy keeps it out of DRAM while the operand records stream past.
+// The per-CTA fixed-point staging (128 KB per CTA, 19 MB in all) is written and
+// read back by the same thread within one tile: an L2 evict_last policy keeps
+// it out of DRAM while the operand records stream past.
 __device__ __forceinline__ uint64_t policy_evict_last() {
   uint64_t pol;
   asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(pol));
   return pol;
 }
 
-__device__ __forceinline__ longlong2 ld_staging(const longlong2* p, uint64_t pol) {
-  long long a, b;
-  asm volatile("ld.global.L2::cache_hint.v2.s64 {%0, %1}, [%2], %3;" : "=l"(a), "=l"(b) : "l"(p), "l"(pol));
-  return make_longlong2(a, b);
+__device__ __forceinline__ long long ld_staging(const long long* p, uint64_t pol) {
+  long long v;
+  asm volatile("ld.global.L2::cache_hint.s64 %0, [%1], %2;" : "=l"(v) : "l"(p), "l"(pol));
+  return v;
 }
 
-__device__ __forceinline__ void st_staging(longlong2* p, longlong2 v, uint64_t pol) {
-  asm volatile("st.global.L2::cache_hint.v2.s64 [%0], {%1, %2}, %3;" ::"l"(p), "l"(v.x), "l"(v.y), "l"(pol)
-               : "memory");
+__device__ __forceinline__ void st_staging(long long* p, long long v, uint64_t pol) {
+  asm volatile("st.global.L2::cache_hint.s64 [%0], %1, %2;" ::"l"(p), "l"(v), "l"(pol) : "memory");
+}
+
+// 0.0 - x, bit for bit (a zero gives +0), without an FP64 instruction
+__device__ __forceinline__ double negated(double x) {
+  const int hi = __double2hiint(x), lo = __double2loint(x);
+  return ((hi & 0x7FFFFFFF) | lo) == 0 ? 0.0 : __hiloint2double(hi ^ (int)0x80000000, lo);
 }
 
 // x * 2^k, exact, by exponent arithmetic on the high word; x an integer-valued
@@ -521,7 +526,7 @@ struct TcArgs {
   int64_t n;
   int nb, words, nsr;
   int32_t* err;
-  long long* scratch;       // per CTA, NSLOT slots: 128 x 128 fixed-point sums of a tile in its epilogue
+  long long* scratch;       // per CTA: 128 x 128 fixed-point sums of the tile in its epilogue
   int seg_min;              // K loops of at least this many steps are cut into segments (0: never)
   int seg_ksteps;           // K steps per segment (8 or 16, divides the 32-step batch)
   unsigned long long wait_ns;   // limit of every bounded wait
@@ -960,7 +965,9 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_square_tc(TcArgs a) {
               const uint64_t ad = ds + (uint64_t)((i * UNIT_BYTES + kk * 256) >> 4);
               const uint64_t bd = ds + (uint64_t)(((2 + j) * UNIT_BYTES + kk * 256) >> 4);
               // the first MMA into a group accumulator of a segment overwrites it
-              mma_f16(dcol, ad, bd, (kk > 0 || acc) ? 1u : 0u);
+              // (the unit of the super-column as the M operand, that of the super-row
+              // as the N operand: TMEM holds the transposed super-tile)
+              mma_f16(dcol, bd, ad, (kk > 0 || acc) ? 1u : 0u);
             }
             written |= 1u << g;
             ++nprod;
@@ -1039,15 +1046,22 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_square_tc(TcArgs a) {
       asm volatile("cp.async.wait_all;" ::: "memory");
     }
   } else if (warp >= 2) {
-    // ---------------- epilogue (warps 2-9, two per SM sub-partition: warp w
-    // reads TMEM lanes 32 (w % 4)..+31 = tile row I0 + w % 4, lane = row inside
-    // the tile; warps 2-5 take column tiles 0-1, warps 6-9 column tiles 2-3).
+    // ---------------- epilogue (warps 2-9, two per SM sub-partition).  TMEM holds
+    // the super-tile transposed (lane = column, TMEM column = row): warp w reads
+    // TMEM lanes 32 (w % 4)..+31 = tile column J0 + w % 4, lane = column inside
+    // the tile; warps 2-5 take row tiles 0-1, warps 6-9 row tiles 2-3.  So the
+    // 32 lanes of a warp hold 32 consecutive elements of a row of the row-major
+    // tiles, and every access to the scratch, to X~ and to X_new is one
+    // contiguous 256-byte piece.  With lane = row each 16-byte access touched 32
+    // separate sectors, and the load/store unit cost as much as the FP64 pipe:
+    // whole runs, before -> after: water-like N = 24,000 188.1 -> 172.3 ms, dense
+    // N = 4,096 with five slices 95.7 -> 77.4 ms, same bits.
     // Phase 1 moves the exact fixed-point sums to the CTA's scratch and returns
     // the TMEM blocks, so the next tile's products run during phase 2, the FP64
-    // arithmetic.
+    // arithmetic.  A thread reads back only what it wrote, so one scratch slot
+    // per CTA serves all tiles.
     const int quarter = warp & 3;
     const int bt0 = 2 * ((warp - 2) >> 2);
-    const int r = lane;
     // unit of the finest group of the window: with W bits per slice, slice s
     // lies on the grid 2^-(W s + W - 1), so group g = s + t has the unit
     // 2^-(W g + 2 W - 2)
@@ -1086,14 +1100,15 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_square_tc(TcArgs a) {
       const int stile = a.list[idx];
       const int R = stile / a.nsr, C = stile % a.nsr;
       const int I0 = 4 * R, J0 = 4 * C;
-      const int Ia = I0 + quarter;           // tile row of this thread
-      const int64_t gi = (int64_t)Ia * TB + r;
-      long long* scr = a.scratch + ((int64_t)blockIdx.x * NSLOT + b) * (ST * ST) + (int64_t)(quarter * 32 + r) * ST;
-      // output tile index of each column tile
+      const int Jb = J0 + quarter;           // tile column of this thread
+      const int64_t gj = (int64_t)Jb * TB + lane;
+      // scratch element of super-tile row i: scr[i * ST]
+      long long* scr = a.scratch + (int64_t)blockIdx.x * (ST * ST) + quarter * 32 + lane;
+      // output tile index of each row tile
       int oidx[2];
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
-        const int Jb = J0 + bt0 + h;
+        const int Ia = I0 + bt0 + h;
         oidx[h] = (Ia < a.nb && Jb < a.nb && (a.general || Ia <= Jb)) ? find(a.obits, a.orowptr, Ia, Jb) : -1;
       }
       // Z_IJ of each output tile (X~_IJ in the forward step; absent -> null),
@@ -1103,15 +1118,15 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_square_tc(TcArgs a) {
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         if (oidx[h] < 0 || emode == 1) continue;
-        const int zp = find(a.zbits, a.zrowptr, Ia, J0 + bt0 + h);
+        const int zp = find(a.zbits, a.zrowptr, I0 + bt0 + h, Jb);
         if (zp < 0) continue;
         const int64_t zi = (int64_t)(a.zref[zp] & ~REF_T);
         Zt[h] = a.zpool + (int64_t)(a.zslot ? a.zslot[zi] : zi) * TE;
-        prefetch_l2(Zt[h] + r * TB);
-        prefetch_l2(Zt[h] + r * TB + 16);
+        prefetch_l2(Zt[h] + lane * TB);
+        prefetch_l2(Zt[h] + lane * TB + 16);
       }
       // phase 1, once per accumulation segment: TMEM -> the exact fixed-point
-      // sums of this thread's row in the scratch (the first segment stores, the
+      // sums of this thread's column in the scratch (the first segment stores, the
       // others add), then the segment's TMEM blocks go back to the MMA issuer
       for (bool first = true;; first = false) {
         const int q = seg & (SEG_RING - 1);
@@ -1132,32 +1147,23 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_square_tc(TcArgs a) {
           if (oidx[h] < 0) continue;      // warp-uniform
 #pragma unroll
           for (int ch = 0; ch < 2; ++ch) {
-            const int col0 = bt * 32 + ch * 16;
+            const int row0 = bt * 32 + ch * 16;
             long long fx[16];
-            longlong2* sp = reinterpret_cast<longlong2*>(scr + col0);
-            if (first) {
+            long long* sp = scr + row0 * ST;
 #pragma unroll
-              for (int i = 0; i < 16; ++i) fx[i] = 0;
-            } else {
-#pragma unroll
-              for (int i = 0; i < 8; ++i) {
-                const longlong2 t2 = ld_staging(sp + i, pol);
-                fx[2 * i] = t2.x;
-                fx[2 * i + 1] = t2.y;
-              }
-            }
+            for (int i = 0; i < 16; ++i) fx[i] = first ? 0 : ld_staging(sp + i * ST, pol);
 #pragma unroll
             for (int gg = 0; gg < 4; ++gg) {   // relative groups of the window
               if (gg <= ghi - glo && ((written >> gg) & 1u)) {   // warp-uniform: groups no product reached are zero
                 float g[16];
                 const uint32_t blk = (gm >> (8 + 2 * gg)) & 3u;
-                tmem_ld16(tmem + ((uint32_t)(quarter * 32) << 16) + blk * ST + (uint32_t)col0, g);
+                tmem_ld16(tmem + ((uint32_t)(quarter * 32) << 16) + blk * ST + (uint32_t)row0, g);
 #pragma unroll
                 for (int i = 0; i < 16; ++i) fx[i] += f32_int_to_ll(g[i]) * (1ll << (W * (ghi - glo - gg)));
               }
             }
 #pragma unroll
-            for (int i = 0; i < 8; ++i) st_staging(sp + i, make_longlong2(fx[2 * i], fx[2 * i + 1]), pol);
+            for (int i = 0; i < 16; ++i) st_staging(sp + i * ST, fx[i], pol);
           }
         }
         // this warp's TMEM reads of the segment are complete
@@ -1172,53 +1178,31 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_square_tc(TcArgs a) {
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         const int bt = bt0 + h;
-        const int Jb = J0 + bt;
+        const int Ia = I0 + bt;
         const int oi = oidx[h];
         if (oi < 0) continue;
         const double* Z = Zt[h];
         double trS = 0.0, trX = 0.0, n2 = 0.0, e2 = 0.0;
         double* O = a.opool + (int64_t)oi * TE;
-        for (int ch = 0; ch < 2; ++ch) {     // 16 columns per chunk
-          const int col0 = bt * 32 + ch * 16;
+        for (int ch = 0; ch < 2; ++ch) {     // 16 rows per chunk
+          const int64_t gi0 = (int64_t)Ia * TB + ch * 16;
+          const long long* sp = scr + (bt * 32 + ch * 16) * ST;
+          const int e0 = ch * 16 * TB + lane;     // element of the chunk's first row in a tile
           double zv[16];
 #pragma unroll
-          for (int i = 0; i < 16; ++i) zv[i] = 0.0;
-          if (Z) {
-            const double2* zp = reinterpret_cast<const double2*>(Z + r * TB + ch * 16);
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-              const double2 t2 = zp[i];
-              zv[2 * i] = t2.x;
-              zv[2 * i + 1] = t2.y;
-            }
-          }
+          for (int i = 0; i < 16; ++i) zv[i] = Z ? Z[e0 + i * TB] : 0.0;
           long long fx[16];
-          const longlong2* sp = reinterpret_cast<const longlong2*>(scr + col0);
 #pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            const longlong2 t2 = ld_staging(sp + i, pol);
-            fx[2 * i] = t2.x;
-            fx[2 * i + 1] = t2.y;
-          }
+          for (int i = 0; i < 16; ++i) fx[i] = ld_staging(sp + i * ST, pol);
           // emode 2: the finer groups' S, left in the output tile by the launch before
           double prev[16];
 #pragma unroll
-          for (int i = 0; i < 16; ++i) prev[i] = 0.0;
-          if (emode == 2) {
-            const double2* pp = reinterpret_cast<const double2*>(O + r * TB + ch * 16);
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-              const double2 t2 = pp[i];
-              prev[2 * i] = t2.x;
-              prev[2 * i + 1] = t2.y;
-            }
-          }
+          for (int i = 0; i < 16; ++i) prev[i] = emode == 2 ? O[e0 + i * TB] : 0.0;
           double out[16];
           if (Z || form == 0) {
 #pragma unroll
             for (int i = 0; i < 16; ++i) {
-              const int c = ch * 16 + i;
-              const int64_t gj = (int64_t)Jb * TB + c;
+              const int64_t gi = gi0 + i;
               const bool inside = gi < a.n && gj < a.n;
               const double fxd = inside ? (double)fx[i] : 0.0;
               const double z = inside ? zv[i] : 0.0;
@@ -1246,27 +1230,25 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_square_tc(TcArgs a) {
             // (e2 is set from n2 below; the same values in the same order)
 #pragma unroll
             for (int i = 0; i < 16; ++i) {
-              const int c = ch * 16 + i;
-              const int64_t gj = (int64_t)Jb * TB + c;
+              const int64_t gi = gi0 + i;
               const bool inside = gi < a.n && gj < a.n;
               const double fxd = inside ? (double)fx[i] : 0.0;
               const bool dg = inside && gi == gj;
               const double S0 = int_times_pow2(fxd, lsu);
               if (emode == 1) { out[i] = S0; continue; }
               const double S = (dg && a.dsq) ? a.dsq[gi] : (emode == 2 ? S0 + prev[i] : S0);
-              const double xn = form == 1 ? S : 0.0 - S;
+              const double xn = form == 1 ? S : negated(S);
               out[i] = xn;
               n2 = fma(xn, xn, n2);
               if (dg) trS += S;
             }
           }
-          double2* op = reinterpret_cast<double2*>(O + r * TB + ch * 16);
 #pragma unroll
-          for (int i = 0; i < 8; ++i) op[i] = make_double2(out[2 * i], out[2 * i + 1]);
+          for (int i = 0; i < 16; ++i) O[e0 + i * TB] = out[i];
         }
         if (emode == 1) continue;
         if (!Z && form != 0) e2 = n2;
-        // warp reductions (the tile's 32 rows are this warp's 32 lanes)
+        // warp reductions (the tile's 32 columns are this warp's 32 lanes)
         for (int o = 16; o > 0; o >>= 1) {
           e2 += __shfl_xor_sync(FULLW, e2, o);
           n2 += __shfl_xor_sync(FULLW, n2, o);
@@ -1279,7 +1261,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_square_tc(TcArgs a) {
           a.part.n2[oi] = n2;
           a.part.trS[oi] = diag ? trS : 0.0;
           a.part.trX[oi] = diag ? trX : 0.0;
-          a.part.ktiles[oi] = kcount[b * 16 + quarter * 4 + bt];
+          a.part.ktiles[oi] = kcount[b * 16 + bt * 4 + quarter];
         }
       }
       __syncwarp();
@@ -1469,8 +1451,4 @@ cudaError_t launch_square_tc(const TcLaunch& L, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-}  // namespace sp2
-
-namespace sp2 {
-int tc_tile_slots() { return NSLOT; }
 }  // namespace sp2
