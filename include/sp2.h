@@ -275,7 +275,8 @@ int sp2_backward(sp2_ctx* ctx, const sp2_bsr* W, sp2_bsr* dF_view);
  * Budget sums are exact integers in units of budget * 2^-36 (shares rounded
  * up).  keep[nnzb] (same residency as X) receives 1 = kept, 0 = dropped.
  * MIXED mode (the mixed norm of Section 3) uses the threshold rule described
- * at sp2_trunc.  Allocates its scratch with cudaMallocAsync on cuda_stream and
+ * at sp2_trunc.  Its scratch comes from the library's memory pool (copies of
+ * host tiles from the device's default pool), stream-ordered on cuda_stream;
  * synchronises that stream before returning.  Errors: INVALID_ARG, OOM, CUDA. */
 int sp2_truncate(const sp2_bsr* X, double tau, int32_t mode, int64_t frobinf_part, int32_t* keep,
                  void* cuda_stream);

@@ -1653,8 +1653,15 @@ int sp2_truncate(const sp2_bsr* X, double tau, int32_t mode, int64_t frobinf_par
   const int64_t part_tiles = std::max<int64_t>(1, frobinf_part / TB);
   void *dbrow = nullptr, *dbcol = nullptr, *dval = nullptr, *dn2 = nullptr, *work = nullptr, *dkeep = nullptr;
   int rc = SP2_OK;
-  auto get = [&](void** p, size_t bytes) {
-    if (cudaMallocAsync(p, std::max<size_t>(bytes, 256), st) != cudaSuccess) {
+  // the selection's scratch (28 bytes a tile) comes from the library's pool,
+  // which keeps it for the next call: the device's default pool gives its memory
+  // back at every synchronisation, and mapping it anew cost more than the
+  // kernels.  Copies of host tiles stay with the default pool.
+  cudaMemPool_t pool = device_pool();
+  auto get = [&](void** p, size_t bytes, bool scratch) {
+    bytes = std::max<size_t>(bytes, 256);
+    const cudaError_t e = scratch && pool ? cudaMallocFromPoolAsync(p, bytes, pool, st) : cudaMallocAsync(p, bytes, st);
+    if (e != cudaSuccess) {
       cudaGetLastError();
       rc = SP2_ERR_OOM;
       return false;
@@ -1667,7 +1674,8 @@ int sp2_truncate(const sp2_bsr* X, double tau, int32_t mode, int64_t frobinf_par
   const double* val = X->val;
   do {
     if (!dev) {
-      if (!get(&dbrow, nnzb * 4) || !get(&dbcol, nnzb * 4) || !get(&dval, (size_t)nnzb * TE * 8)) break;
+      if (!get(&dbrow, nnzb * 4, false) || !get(&dbcol, nnzb * 4, false) || !get(&dval, (size_t)nnzb * TE * 8, false))
+        break;
       if (cudaMemcpyAsync(dbrow, X->brow, nnzb * 4, cudaMemcpyHostToDevice, st) != cudaSuccess ||
           cudaMemcpyAsync(dbcol, X->bcol, nnzb * 4, cudaMemcpyHostToDevice, st) != cudaSuccess ||
           cudaMemcpyAsync(dval, X->val, (size_t)nnzb * TE * 8, cudaMemcpyHostToDevice, st) != cudaSuccess) {
@@ -1680,10 +1688,10 @@ int sp2_truncate(const sp2_bsr* X, double tau, int32_t mode, int64_t frobinf_par
     }
     const int nsb = (int)((nb + part_tiles - 1) / part_tiles);
     const size_t wbytes = mode == SP2_TRUNC_MIXED ? mixed_work_bytes(nnzb, nsb) : trunc_work_bytes(nnzb, nb, part_tiles);
-    if (!get(&dn2, nnzb * 8) || !get(&work, wbytes)) break;
+    if (!get(&dn2, nnzb * 8, true) || !get(&work, wbytes, true)) break;
     int32_t* kout = keep;
     if (!dev) {
-      if (!get(&dkeep, nnzb * 4)) break;
+      if (!get(&dkeep, nnzb * 4, true)) break;
       kout = static_cast<int32_t*>(dkeep);
     }
     TileSet ts;

@@ -14,15 +14,25 @@
 //    understate ||E||_F^2.
 //
 // GPU form: a segmented most-significant-digit radix select over the 96-bit key
-// (63 bits of the squared norm's IEEE pattern -- non-negative doubles order like
-// their bit patterns -- then the 32-bit linear tile index).  Twelve passes of
-// 8 bits; each pass histograms the budget units of the remaining candidates and
-// one thread per segment walks its 256 buckets.  No sort, no host round trip.
-// A single segment of at most 2048 tiles runs the same passes in one CTA.
+// (the squared norm's IEEE pattern -- non-negative doubles order like their bit
+// patterns -- then the 32-bit linear tile index), one cluster of CL_CTAS CTAs
+// per segment.  Each pass histograms the budget units of the remaining
+// candidates in shared memory, the CTAs sum the bins through distributed shared
+// memory and find the bucket in which the budget ends.  The cluster's hardware
+// barrier orders the passes, so a selection is one launch; it ends as soon as
+// one candidate is left, usually after three of the nine passes.  (A memset, a
+// histogram and a one-thread-per-segment bucket walk for each of twelve 8-bit
+// passes were 36 launches; one truncation of 180,300 device tiles, norms
+// included, took 1.46 ms and takes 0.58 ms.)
+// A single segment of at most 2048 tiles runs in one CTA.
 #include <cmath>
 #include <vector>
 
+#include <cooperative_groups.h>
+
 #include "sp2_internal.h"
+
+namespace cg = cooperative_groups;
 
 namespace sp2 {
 namespace {
@@ -33,15 +43,8 @@ constexpr unsigned long long Q_CAP = 1ull << 37;
 constexpr int MIXED_POWER_ITERS = 100;        // power steps of the mixed-norm bound
 
 struct Work {
-  unsigned long long* q;
-  int32_t* seg;
-  double* scale;
-  unsigned long long* rem;
-  unsigned long long* pref_hi;
-  uint32_t* pref_lo;
-  int32_t* state;
-  int32_t* depth;
-  unsigned long long* hist;
+  unsigned long long* q;   // budget units of each tile
+  double* scale;           // Frob-Inf: units per squared norm of each segment
   int32_t* nz;
   int32_t* m;
   int64_t nseg;
@@ -54,14 +57,7 @@ Work carve(void* base, int64_t nnzb, int64_t nseg, int nsb) {
   char* p = static_cast<char*>(base);
   Work w;
   w.q = reinterpret_cast<unsigned long long*>(p); p += align_up(nnzb * 8);
-  w.seg = reinterpret_cast<int32_t*>(p); p += align_up(nnzb * 4);
   w.scale = reinterpret_cast<double*>(p); p += align_up(nseg * 8);
-  w.rem = reinterpret_cast<unsigned long long*>(p); p += align_up(nseg * 8);
-  w.pref_hi = reinterpret_cast<unsigned long long*>(p); p += align_up(nseg * 8);
-  w.pref_lo = reinterpret_cast<uint32_t*>(p); p += align_up(nseg * 4);
-  w.state = reinterpret_cast<int32_t*>(p); p += align_up(nseg * 4);
-  w.depth = reinterpret_cast<int32_t*>(p); p += align_up(nseg * 4);
-  w.hist = reinterpret_cast<unsigned long long*>(p); p += align_up(nseg * 256 * 8);
   w.nz = reinterpret_cast<int32_t*>(p); p += align_up((size_t)nsb * nsb * 4);
   w.m = reinterpret_cast<int32_t*>(p); p += align_up((size_t)nsb * 4);
   w.nseg = nseg;
@@ -86,51 +82,40 @@ __global__ void k_m(const int32_t* __restrict__ nz, int nsb, int32_t* m) {
   m[R] = c;
 }
 
-// mode 0: one segment, budget tau^2.  mode 1: segment R * nsb + C.
-__global__ void k_seg_init(Work w, int mode, double tau) {
+// Frob-Inf: units per squared norm of segment R * nsb + C
+__global__ void k_seg_scale(Work w, double tau) {
   const int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (s >= w.nseg) return;
-  double budget;
-  if (mode == 0) {
-    budget = tau * tau;
-  } else {
-    const int R = (int)(s / w.nsb), C = (int)(s % w.nsb);
-    const int mm = max(w.m[R], w.m[C]);
-    const double beta = mm > 0 ? tau / (double)mm : 0.0;
-    budget = beta * beta;
-  }
+  const int R = (int)(s / w.nsb), C = (int)(s % w.nsb);
+  const int mm = max(w.m[R], w.m[C]);
+  const double beta = mm > 0 ? tau / (double)mm : 0.0;
+  const double budget = beta * beta;
   w.scale[s] = budget > 0.0 ? Q_SCALE / budget : 0.0;
-  w.rem[s] = Q_BUDGET;
-  w.pref_hi[s] = 0ull;
-  w.pref_lo[s] = 0u;
-  w.state[s] = 0;
-  w.depth[s] = 0;
 }
 
+// budget units of a tile of squared norm v and weight wt (1: stored once, 2: mirrored)
+__device__ __forceinline__ unsigned long long budget_units(double v, double wt, double sc) {
+  if (sc == 0.0) return (v == 0.0) ? 0ull : Q_CAP;
+  const double x = (wt * v) * sc;
+  return (x >= (double)Q_CAP) ? Q_CAP : (unsigned long long)ceil(x);
+}
+
+// mode 0: one segment, scale sc; mode 1: the segment's scale.  Its own launch
+// over all SMs: the FP64 pipe (2 lanes per SM cycle) is too slow for it to sit
+// in the few CTAs of the selection.
 __global__ void k_q(const int32_t* __restrict__ brow, const int32_t* __restrict__ bcol,
                     const int32_t* __restrict__ slot, const double* __restrict__ n2, int64_t nnzb, int mode, int pt,
-                    Work w) {
+                    double sc, Work w) {
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (t >= nnzb) return;
   const int I = brow[t], J = bcol[t];
-  int s = 0;
   double wt = (I == J) ? 1.0 : 2.0;
   if (mode == 1) {
     const int R = I / pt, C = J / pt;
-    s = R * w.nsb + C;
+    sc = w.scale[R * w.nsb + C];
     if (R != C) wt = 1.0;
   }
-  w.seg[t] = s;
-  const double v = n2[slot ? slot[t] : t];
-  const double sc = w.scale[s];
-  unsigned long long q;
-  if (sc == 0.0) {
-    q = (v == 0.0) ? 0ull : Q_CAP;
-  } else {
-    const double x = (wt * v) * sc;
-    q = (x >= (double)Q_CAP) ? Q_CAP : (unsigned long long)ceil(x);
-  }
-  w.q[t] = q;
+  w.q[t] = budget_units(n2[slot ? slot[t] : t], wt, sc);
 }
 
 __device__ __forceinline__ bool is_candidate(unsigned long long hi, uint32_t lo, int p, unsigned long long ph,
@@ -145,86 +130,187 @@ __device__ __forceinline__ int digit_of(unsigned long long hi, uint32_t lo, int 
   return (int)((lo >> (24 - 8 * (p - 8))) & 0xFFu);
 }
 
-template <bool ONE_SEG>
-__global__ void k_hist(const int32_t* __restrict__ brow, const int32_t* __restrict__ bcol,
-                       const int32_t* __restrict__ slot, const double* __restrict__ n2, int64_t nnzb, int nb, int p,
-                       Work w) {
-  __shared__ unsigned long long sh[256];
-  if (ONE_SEG) {
-    for (int k = threadIdx.x; k < 256; k += blockDim.x) sh[k] = 0ull;
-    __syncthreads();
+// Radix select of one segment per cluster (mode 1: grid (nsb clusters, nsb),
+// segment (R, C), R <= C, of the upper triangle of nsb x nsb super-blocks).
+// The tiles are sorted by row, so the segment's tiles lie in the range of its
+// super-row (all of them in mode 0); the CTAs of the cluster split that range.
+// Digits: the 12 bits of sign and exponent first (a tile set spans some 100
+// octaves, so the shared-memory atomics of a warp rarely meet in one bin),
+// 11 bits at a time after that.
+// Two sizes: CL_CTAS x 1024 threads for segments of many tiles, one CTA of 256
+// threads for small ones (Frob-Inf with a small partition has thousands).
+constexpr int CL_CTAS = 8;
+constexpr int64_t CL_MANY = 4096;   // tiles of a segment (mean) from which the cluster is taken
+constexpr int CL_BINS = 4096;
+constexpr int CL_PASSES = 9;      // 6 over the norm (52, 41, 30, 19, 8, 0), 3 over the index (21, 10, 0)
+constexpr size_t CL_SMEM = (size_t)CL_BINS * 12;
+
+__device__ __forceinline__ int cl_shift(int p) {
+  return p < 5 ? 52 - 11 * p : p == 5 ? 0 : p == 6 ? 21 : p == 7 ? 10 : 0;
+}
+
+__device__ __forceinline__ int64_t first_row_ge(const int32_t* __restrict__ brow, int64_t n, int row) {
+  int64_t lo = 0, hi = n;
+  while (lo < hi) {
+    const int64_t mid = (lo + hi) >> 1;
+    if (brow[mid] < row) lo = mid + 1; else hi = mid;
   }
-  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (t < nnzb) {
-    const int s = w.seg[t];
-    if (w.state[s] == 0) {
+  return lo;
+}
+
+template <int CTAS, int THREADS>
+__global__ void __cluster_dims__(CTAS, 1, 1) __launch_bounds__(THREADS)
+    k_trunc_cluster(const int32_t* __restrict__ brow, const int32_t* __restrict__ bcol,
+                    const int32_t* __restrict__ slot, const double* __restrict__ n2,
+                    const unsigned long long* __restrict__ q, int64_t nnzb, int nb, int mode, int pt, int nsb,
+                    int32_t* keep) {
+  extern __shared__ __align__(16) unsigned char cl_smem[];
+  unsigned long long* hist = reinterpret_cast<unsigned long long*>(cl_smem);   // [CL_BINS] units
+  uint32_t* cnt = reinterpret_cast<uint32_t*>(hist + CL_BINS);                 // [CL_BINS] candidates
+  __shared__ unsigned long long tot[CTAS];     // units in the bins of each CTA's share
+  __shared__ unsigned long long wsum[32];
+  __shared__ unsigned long long s_rem;            // budget left below the cut bucket
+  __shared__ int s_cut, s_cnt;
+  __shared__ int64_t range[2];
+  cg::cluster_group cl = cg::this_cluster();
+  const int rank = (int)cl.block_rank();
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  int C = 0;
+  if (mode == 1) {
+    const int R = (int)blockIdx.y;
+    C = (int)(blockIdx.x / CTAS);
+    if (C < R) return;     // the whole cluster
+    if (tid < 2) range[tid] = first_row_ge(brow, nnzb, (R + tid) * pt);
+  } else if (tid == 0) {
+    range[0] = 0;
+    range[1] = nnzb;
+  }
+  __syncthreads();
+  const int64_t len = (range[1] - range[0] + CTAS - 1) / CTAS;
+  const int64_t c0 = range[0] + rank * len, c1 = min(range[1], c0 + len);
+  constexpr int SHARE = CL_BINS / CTAS;        // bins a CTA sums over the cluster
+  constexpr int PER = SHARE > THREADS ? SHARE / THREADS : 1;
+  unsigned long long ph = 0ull, rem = Q_BUDGET;
+  uint32_t pl = 0u;
+  int depth = 0;       // digits fixed in (ph, pl)
+  bool all = false;    // every remaining candidate fits
+  for (int p = 0; p < CL_PASSES; ++p) {
+    for (int k = tid; k < CL_BINS; k += THREADS) {
+      hist[k] = 0ull;
+      cnt[k] = 0u;
+    }
+    __syncthreads();
+    const int sh = cl_shift(p), psh = p > 0 ? cl_shift(p - 1) : 0;
+    const uint32_t dm = p == 0 ? 0xFFFu : p == 5 ? 0xFFu : p == 8 ? 0x3FFu : 0x7FFu;
+    for (int64_t t = c0 + tid; t < c1; t += THREADS) {
       const unsigned long long hi = __double_as_longlong(n2[slot ? slot[t] : t]);
-      const uint32_t lo = (uint32_t)brow[t] * (uint32_t)nb + (uint32_t)bcol[t];
-      if (is_candidate(hi, lo, p, w.pref_hi[s], w.pref_lo[s])) {
-        const int d = digit_of(hi, lo, p);
-        if (ONE_SEG) atomicAdd(&sh[d], w.q[t]);
-        else atomicAdd(&w.hist[(int64_t)s * 256 + d], w.q[t]);
+      uint32_t lo = 0u;
+      bool in = true;
+      if (p > 0 && p <= 6) in = (hi >> psh) == ph;
+      if (p > 6) in = hi == ph;
+      if (in && p >= 6) {
+        lo = (uint32_t)brow[t] * (uint32_t)nb + (uint32_t)bcol[t];
+        if (p > 6) in = (lo >> psh) == pl;
+      }
+      if (in && mode == 1) in = bcol[t] / pt == C;
+      if (in) {
+        const uint32_t d = (p < 6 ? (uint32_t)(hi >> sh) : lo >> sh) & dm;
+        atomicAdd(&hist[d], q[t]);
+        atomicAdd(&cnt[d], 1u);
       }
     }
-  }
-  if (ONE_SEG) {
-    __syncthreads();
-    for (int k = threadIdx.x; k < 256; k += blockDim.x)
-      if (sh[k]) atomicAdd(&w.hist[k], sh[k]);
-  }
-}
-
-__global__ void k_select(Work w, int p) {
-  const int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (s >= w.nseg || w.state[s] != 0) return;
-  unsigned long long rem = w.rem[s];
-  const unsigned long long* h = w.hist + s * 256;
-  int cut = -1;
-  for (int d = 0; d < 256; ++d) {
-    const unsigned long long v = h[d];
-    if (v <= rem) rem -= v;
-    else { cut = d; break; }
-  }
-  w.rem[s] = rem;
-  if (cut < 0) {
-    w.state[s] = 1;      // every candidate fits: drop all keys whose top 8p bits <= prefix
-    w.depth[s] = p;
-  } else if (p < 8) {
-    w.pref_hi[s] = (w.pref_hi[s] << 8) | (unsigned long long)cut;
-  } else {
-    w.pref_lo[s] = (w.pref_lo[s] << 8) | (uint32_t)cut;
-  }
-}
-
-__global__ void k_mark(const int32_t* __restrict__ brow, const int32_t* __restrict__ bcol,
-                       const int32_t* __restrict__ slot, const double* __restrict__ n2, int64_t nnzb, int nb, Work w,
-                       int32_t* keep) {
-  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (t >= nnzb) return;
-  const int s = w.seg[t];
-  const unsigned long long hi = __double_as_longlong(n2[slot ? slot[t] : t]);
-  const uint32_t lo = (uint32_t)brow[t] * (uint32_t)nb + (uint32_t)bcol[t];
-  const unsigned long long ph = w.pref_hi[s];
-  const uint32_t pl = w.pref_lo[s];
-  bool drop;
-  if (w.state[s] == 1) {
-    const int dep = w.depth[s];
-    if (dep == 0) drop = true;
-    else if (dep <= 8) drop = (hi >> (64 - 8 * dep)) <= ph;
-    else {
-      const uint32_t top = lo >> (32 - 8 * (dep - 8));
-      drop = hi < ph || (hi == ph && top <= pl);
+    cl.sync();
+    // this CTA's share of the bins, summed over the cluster (PER bins a thread),
+    // and its prefix sums
+    unsigned long long v = 0ull, bv[PER];
+    uint32_t bc[PER];
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+      bv[j] = 0ull;
+      bc[j] = 0u;
+      if (tid * PER < SHARE) {
+        for (int r = 0; r < CTAS; ++r) {
+          bv[j] += cl.map_shared_rank(hist, r)[rank * SHARE + tid * PER + j];
+          bc[j] += cl.map_shared_rank(cnt, r)[rank * SHARE + tid * PER + j];
+        }
+      }
+      v += bv[j];
     }
-  } else {
-    drop = hi < ph || (hi == ph && lo < pl);
+    unsigned long long inc = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned long long y = __shfl_up_sync(0xffffffffu, inc, o);
+      if (lane >= o) inc += y;
+    }
+    if (lane == 31) wsum[wid] = inc;
+    __syncthreads();
+    unsigned long long below = 0ull, mine = 0ull;
+    for (int k = 0; k < THREADS / 32; ++k) {
+      if (k < wid) below += wsum[k];
+      mine += wsum[k];
+    }
+    if (tid < CTAS) cl.map_shared_rank(tot, tid)[rank] = mine;
+    cl.sync();
+    unsigned long long before = below + inc - v, grand = 0ull;
+    for (int r = 0; r < CTAS; ++r) {
+      if (r < rank) before += tot[r];
+      grand += tot[r];
+    }
+    if (grand <= rem) {      // the same in every thread of the cluster
+      all = true;
+      break;
+    }
+    // the one bucket in which the budget ends
+    if (before <= rem && before + v > rem) {
+      bool open = true;
+#pragma unroll
+      for (int j = 0; j < PER; ++j) {
+        if (open && before + bv[j] > rem) {
+          for (int r = 0; r < CTAS; ++r) {
+            *cl.map_shared_rank(&s_rem, r) = rem - before;
+            *cl.map_shared_rank(&s_cut, r) = rank * SHARE + tid * PER + j;
+            *cl.map_shared_rank(&s_cnt, r) = (int)bc[j];
+          }
+          open = false;
+        }
+        before += bv[j];
+      }
+    }
+    cl.sync();
+    rem = s_rem;
+    if (p == 0) ph = (unsigned long long)s_cut;
+    else if (p < 5) ph = (ph << 11) | (unsigned long long)s_cut;
+    else if (p == 5) ph = (ph << 8) | (unsigned long long)s_cut;
+    else if (p == 6) pl = (uint32_t)s_cut;
+    else if (p == 7) pl = (pl << 11) | (uint32_t)s_cut;
+    else pl = (pl << 10) | (uint32_t)s_cut;
+    depth = p + 1;
+    if (s_cnt == 1) break;   // the bucket's only candidate is the first tile that does not fit
   }
-  keep[t] = drop ? 0 : 1;
+  // dropped: keys below the prefix; the prefix's own bucket only when everything fits
+  const int dsh = depth > 0 ? cl_shift(depth - 1) : 0;
+  for (int64_t t = c0 + tid; t < c1; t += THREADS) {
+    if (mode == 1 && bcol[t] / pt != C) continue;
+    const unsigned long long hi = __double_as_longlong(n2[slot ? slot[t] : t]);
+    bool less, equal;
+    if (depth == 0) {
+      less = false;
+      equal = true;
+    } else if (depth <= 6) {
+      less = (hi >> dsh) < ph;
+      equal = (hi >> dsh) == ph;
+    } else {
+      const uint32_t lo = ((uint32_t)brow[t] * (uint32_t)nb + (uint32_t)bcol[t]) >> dsh;
+      less = hi < ph || (hi == ph && lo < pl);
+      equal = hi == ph && lo == pl;
+    }
+    keep[t] = (less || (equal && all)) ? 0 : 1;
+  }
 }
 
-// One CTA for a single segment of at most SMALL_MAX tiles: the same twelve
-// passes as k_hist + k_select + k_mark, keys held in shared memory, so a small
-// truncation is one launch instead of about forty.  All sums are the same exact
-// integers, so the keep flags equal the multi-launch path's.
+// One CTA for a single segment of at most SMALL_MAX tiles: twelve 8-bit passes
+// with keys and units held in shared memory, one launch.  All sums are the same
+// exact integers, so the keep flags equal the cluster's.
 constexpr int SMALL_MAX = 2048;
 constexpr int SMALL_THREADS = 1024;
 
@@ -243,17 +329,9 @@ __global__ void __launch_bounds__(SMALL_THREADS)
   for (int t = threadIdx.x; t < n; t += blockDim.x) {
     const int I = brow[t], J = bcol[t];
     const double v = n2[slot ? slot[t] : t];
-    const double wt = (I == J) ? 1.0 : 2.0;
-    unsigned long long q;
-    if (sc == 0.0) {
-      q = (v == 0.0) ? 0ull : Q_CAP;
-    } else {
-      const double x = (wt * v) * sc;
-      q = (x >= (double)Q_CAP) ? Q_CAP : (unsigned long long)ceil(x);
-    }
     s_hi[t] = __double_as_longlong(v);
     s_lo[t] = (uint32_t)I * (uint32_t)nb + (uint32_t)J;
-    s_q[t] = q;
+    s_q[t] = budget_units(v, (I == J) ? 1.0 : 2.0, sc);
   }
   if (threadIdx.x == 0) {
     s_rem = Q_BUDGET;
@@ -275,7 +353,7 @@ __global__ void __launch_bounds__(SMALL_THREADS)
     }
     __syncthreads();
     if (threadIdx.x < 32) {
-      // bucket walk of k_select: lane l owns buckets 8l..8l+7, an inclusive
+      // bucket walk: lane l owns buckets 8l..8l+7, an inclusive
       // scan over the lanes finds the lane holding the cut
       const int lane = threadIdx.x;
       unsigned long long loc[8], sum = 0ull;
@@ -335,21 +413,34 @@ __global__ void __launch_bounds__(SMALL_THREADS)
   }
 }
 
-// ||tile||_F^2 of contiguous tiles (fixed order: 4 strided partial sums per
-// thread, then a fixed tree), one CTA of 256 threads per tile.
-__global__ void __launch_bounds__(256) k_tile_norms(const double* __restrict__ val, double* n2) {
-  const int64_t t = blockIdx.x;
-  const double* x = val + t * TE;
-  double a = 0.0;
-  for (int q = threadIdx.x; q < TE; q += 256) a += x[q] * x[q];
-  __shared__ double red[256];
-  red[threadIdx.x] = a;
-  __syncthreads();
-  for (int h = 128; h > 0; h >>= 1) {
-    if ((int)threadIdx.x < h) red[threadIdx.x] += red[threadIdx.x + h];
-    __syncthreads();
+// ||tile||_F^2 of contiguous tiles, one warp per tile: lane l, j = 0..7, sums the
+// elements l + 32 j + 256 k over k in order, then a fixed tree over j and the
+// lanes.  All 32 loads of a lane are in flight at once; the FP64 pipe (1,408
+// lane operations a tile at 2 per SM cycle, 0.42 ms for 180,300 tiles) bounds it, not
+// HBM (0.22 ms).
+constexpr int NORM_WARPS = 8;
+__global__ void __launch_bounds__(32 * NORM_WARPS) k_tile_norms(const double* __restrict__ val, int64_t nnzb, double* n2) {
+  const int64_t t = (int64_t)blockIdx.x * NORM_WARPS + (threadIdx.x >> 5);
+  const int lane = threadIdx.x & 31;
+  if (t >= nnzb) return;
+  const double* x = val + t * TE + lane;
+  double v[32];
+#pragma unroll
+  for (int i = 0; i < 32; ++i) v[i] = x[32 * i];
+  double a[8];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    a[j] = v[j] * v[j];
+#pragma unroll
+    for (int k = 1; k < 4; ++k) a[j] = fma(v[j + 8 * k], v[j + 8 * k], a[j]);
   }
-  if (threadIdx.x == 0) n2[t] = red[0];
+#pragma unroll
+  for (int h = 4; h > 0; h >>= 1)
+#pragma unroll
+    for (int j = 0; j < h; ++j) a[j] += a[j + h];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) a[0] += __shfl_down_sync(0xffffffffu, a[0], o);
+  if (lane == 0) n2[t] = a[0];
 }
 
 inline unsigned grid_for(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
@@ -407,15 +498,14 @@ __global__ void k_mixed_keep(const long long* __restrict__ bits, int64_t nnzb, l
 
 cudaError_t launch_tile_norms(const double* val, int64_t nnzb, double* n2, cudaStream_t st) {
   if (nnzb == 0) return cudaSuccess;
-  { ++g_launches; k_tile_norms<<<(unsigned)nnzb, 256, 0, st>>>(val, n2); }
+  { ++g_launches; k_tile_norms<<<grid_for(nnzb, NORM_WARPS), 32 * NORM_WARPS, 0, st>>>(val, nnzb, n2); }
   return cudaGetLastError();
 }
 
 size_t trunc_work_bytes(int64_t nnzb, int nb, int64_t part_tiles) {
   const int nsb = (int)((nb + part_tiles - 1) / part_tiles);
   const int64_t nseg = (int64_t)nsb * nsb;
-  return align_up(nnzb * 8) + align_up(nnzb * 4) + 5 * align_up(nseg * 8) + 3 * align_up(nseg * 4) +
-         align_up(nseg * 256 * 8) + align_up((size_t)nsb * nsb * 4) + align_up((size_t)nsb * 4) + 1024;
+  return align_up(nnzb * 8) + align_up(nseg * 8) + align_up((size_t)nsb * nsb * 4) + align_up((size_t)nsb * 4) + 1024;
 }
 
 // x: the tiles of X_i (slot indexes n2); n2[slot] = ||X_i tile||_F^2; keep[t] out.
@@ -431,24 +521,31 @@ cudaError_t launch_truncate(const TileSet& x, const double* n2, int nb, double t
     return cudaGetLastError();
   }
   Work w = carve(work, nnzb, nseg, nsb);
-  cudaError_t e;
-  if (mode == 1) {
-    e = cudaMemsetAsync(w.nz, 0, (size_t)nsb * nsb * 4, st);
+  const int md = nseg == 1 ? 0 : 1;   // mode 1 with a single super-block has m = 1: budget tau^2 as in mode 0
+  double sc = 0.0;
+  if (md == 1) {
+    const cudaError_t e = cudaMemsetAsync(w.nz, 0, (size_t)nsb * nsb * 4, st);
     if (e != cudaSuccess) return e;
     { ++g_launches; k_nz<<<grid_for(nnzb, 256), 256, 0, st>>>(x.brow, x.bcol, nnzb, (int)part_tiles, nsb, w.nz); }
     { ++g_launches; k_m<<<grid_for(nsb, 128), 128, 0, st>>>(w.nz, nsb, w.m); }
+    { ++g_launches; k_seg_scale<<<grid_for(nseg, 256), 256, 0, st>>>(w, tau); }
+  } else {
+    const double budget = tau * tau;
+    sc = budget > 0.0 ? Q_SCALE / budget : 0.0;
   }
-  { ++g_launches; k_seg_init<<<grid_for(nseg, 256), 256, 0, st>>>(w, mode, tau); }
-  { ++g_launches; k_q<<<grid_for(nnzb, 256), 256, 0, st>>>(x.brow, x.bcol, x.slot, n2, nnzb, mode, (int)part_tiles, w); }
-  for (int p = 0; p < 12; ++p) {
-    e = cudaMemsetAsync(w.hist, 0, (size_t)nseg * 256 * 8, st);
+  { ++g_launches; k_q<<<grid_for(nnzb, 256), 256, 0, st>>>(x.brow, x.bcol, x.slot, n2, nnzb, md, (int)part_tiles, sc, w); }
+  const int64_t nclus = md == 1 ? (int64_t)nsb * (nsb + 1) / 2 : 1;
+  const unsigned side = md == 1 ? (unsigned)nsb : 1u;
+  auto launch = [&](auto kernel, int ctas, int threads) -> cudaError_t {
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CL_SMEM);
     if (e != cudaSuccess) return e;
-    if (nseg == 1) { ++g_launches; k_hist<true><<<grid_for(nnzb, 256), 256, 0, st>>>(x.brow, x.bcol, x.slot, n2, nnzb, nb, p, w); }
-    else { ++g_launches; k_hist<false><<<grid_for(nnzb, 256), 256, 0, st>>>(x.brow, x.bcol, x.slot, n2, nnzb, nb, p, w); }
-    { ++g_launches; k_select<<<grid_for(nseg, 128), 128, 0, st>>>(w, p); }
-  }
-  { ++g_launches; k_mark<<<grid_for(nnzb, 256), 256, 0, st>>>(x.brow, x.bcol, x.slot, n2, nnzb, nb, w, keep); }
-  return cudaGetLastError();
+    ++g_launches;
+    kernel<<<dim3(side * ctas, side), threads, CL_SMEM, st>>>(x.brow, x.bcol, x.slot, n2, w.q, nnzb, nb, md,
+                                                               (int)part_tiles, nsb, keep);
+    return cudaGetLastError();
+  };
+  return nnzb >= CL_MANY * nclus || nclus == 1 ? launch(k_trunc_cluster<CL_CTAS, 1024>, CL_CTAS, 1024)
+                                               : launch(k_trunc_cluster<1, 256>, 1, 256);
 }
 
 }  // namespace sp2

@@ -80,12 +80,25 @@ def test_device_input_matches_host_input():
 @pytest.mark.parametrize("tau", [0.0, 1e-4, 0.3])
 def test_keep_flags_around_one_cta_limit(n, mode, tau):
     """2016 upper tiles (nb = 63) take the one-CTA select, 2080 (nb = 64, also
-    with a ragged tail) the multi-launch passes; both match the oracle bit for bit."""
+    with a ragged tail) the cluster's passes; both match the oracle bit for bit."""
     import paper_1909_12533_gb300 as sp2
     X = _decaying(n, 5, ties=True)
     X.val[11] = 0.0
     g = sp2.sp2_truncate(X, tau, mode, 4096)
     o = _oracle_keep(X, tau, mode, 4096)
+    assert np.array_equal(g, o), np.nonzero(g != o)
+
+
+@pytest.mark.parametrize("n,part", [(331, 32), (5900, 3008)])
+@pytest.mark.parametrize("tau", [0.0, 1e-3, 1e3])
+def test_keep_flags_of_both_segment_selects(n, part, tau):
+    """Frob-Inf with 66 one-tile segments (one CTA each) and with three segments
+    of 5,735 tiles on average (a cluster each), equal norms among them."""
+    import paper_1909_12533_gb300 as sp2
+    X = _decaying(n, 23, ties=True)
+    X.val[11] = 0.0
+    g = sp2.sp2_truncate(X, tau, "frobinf", part)
+    o = _oracle_keep(X, tau, "frobinf", part)
     assert np.array_equal(g, o), np.nonzero(g != o)
 
 

@@ -54,8 +54,8 @@ def _oracle_keep(X, tau, mode, part):
 
 
 # Frobenius: 3000 and 2600 rows give 4465 and 3403 upper tiles, above the
-# 2048-tile limit of the one-CTA select, so both calls run the multi-launch
-# select in the shared scratch array.  Frob-Inf with 128-row super-blocks:
+# 2048-tile limit of the one-CTA select, so both calls run the cluster's
+# select with its units in the shared scratch array.  Frob-Inf with 128-row super-blocks:
 # 64 and 49 segments.
 @pytest.mark.parametrize("mode,part,sizes", [("frobenius", 4096, (3000, 2600)), ("frobinf", 128, (1000, 700))])
 def test_noalloc_matches_allocating_entry_point_twice(mode, part, sizes):
