@@ -764,7 +764,6 @@ void run_tc(sp2_ctx* c, TcLaunch& L, const uint32_t* obits, const int32_t* orowp
   L.scratch = c->tcscratch.p;
   L.seg_min = c->prm.acc_flush_min;
   L.wait_ns = (unsigned long long)c->prm.wait_limit_ms * 1000000ull;
-  L.split_supply = c->prm.split_supply != 0;
   L.selftest = c->selftest_pending == 1;
   if (c->selftest_pending == 1) c->selftest_pending = 0;
   L.err = c->errflag.as<int32_t>();

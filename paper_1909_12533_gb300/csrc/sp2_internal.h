@@ -185,7 +185,6 @@ struct TcLaunch {
   unsigned long long wait_ns = 2000000000ull;   // limit of every bounded wait in the kernel
   bool selftest = false;     // wait first on a barrier nothing arrives at (tests the timeout path)
   bool general = false;      // general storage: every output tile of the square, weight 1 in e^2
-  bool split_supply = false; // B operand units through copy warps (cp.async) beside the bulk copies of A
   const double* dsq = nullptr;   // S_ii per global row in FP64 (symmetric square: the squared row norms)
   int glo = 0, ghi = -1;     // slice-pair groups s + t of the launch (ghi < 0: all, k - 1; at most 4 groups)
   int emode = 0;             // 0 full epilogue, 1 store S only, 2 full epilogue on S + the stored S

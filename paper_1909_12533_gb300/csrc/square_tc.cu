@@ -34,16 +34,17 @@
 // Pairs left out multiply zeros, so the result is the same bit for bit.
 //
 // Data path per CTA (one 128 x 128 output super-tile = 4 x 4 tiles of 32):
-//   warp 0: producer -- for every K tile in the union of the super-rows'
+//   warp 0: planner -- for every K tile in the union of the super-rows'
 //     patterns (32 at a time, found from the super-row bitmaps, their record
-//     headers fetched one batch ahead), emits sub-steps of at most two A
-//     slices x two B slices: each sub-step is one pipeline stage filled by up
-//     to four 8 KB cp.async.bulk copies (completion tracked by an mbarrier
-//     transaction count), described by a small stage record.
-//   warp 1 lane 0: issues tcgen05.mma kind::f16 (M = 128, N = 128, K = 16) for
-//     every slice pair of the record into the TMEM accumulator of its group,
-//     then tcgen05.commit frees the stage.
-//   all 8 warps: epilogue -- tcgen05.ld of the accumulators that were written,
+//     headers fetched one batch ahead), lists sub-steps of at most two A
+//     slices x two B slices.
+//   warps 18 and 19: issuers -- copy the A and the B units of every sub-step
+//     into shared-memory rings (cp.async.bulk of 8 or 16 KB, completion tracked
+//     by an mbarrier transaction count).
+//   warp 1: issues tcgen05.mma kind::f16 (M = 128, N = 128, K = 16) for every
+//     slice pair of the record into the TMEM accumulator of its group, then
+//     tcgen05.commit frees the units.
+//   warps 2-17: epilogue -- tcgen05.ld of the accumulators that were written,
 //     exact fixed-point combination, X_new = c0 I + c1 X~ + c2 S in FP64,
 //     per-tile ||X~ - S||^2, traces and ||X_new||^2, FP64 stores of the
 //     output tiles present.
@@ -115,8 +116,8 @@ __device__ __forceinline__ bool mbar_try_wait_sleep(uint64_t* bar, uint32_t pari
 }
 
 // Timeout sites of a launch, for the error message (err[1], bit 0 self-test
-// probe, 8 copy warps, 9 copies still in flight at an error exit, 1 producer
-// stage, 2 producer tile slot, 3 MMA data, 4 MMA TMEM or segment slot, 5 MMA
+// probe, 1 planner batch or tile slot, 2 issuer ring, 8 issuer batch, 9 copies
+// still in flight at the exit, 3 MMA data, 4 MMA TMEM or segment slot, 5 MMA
 // drain, 6 epilogue tile, 7 epilogue segment).
 __device__ __forceinline__ void note_timeout(int32_t* err, int where) {
   if (err) atomicOr(err + 1, 1 << where);
@@ -146,10 +147,10 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
   return true;
 }
 
-__device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
+__device__ __forceinline__ void bulk_g2s(uint32_t dst, const void* src, uint32_t bytes, uint64_t* bar) {
   asm volatile(
       "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-          smem_u32(dst)),
+          dst),
       "l"(src), "r"(bytes), "r"(smem_u32(bar))
       : "memory");
 }
@@ -235,6 +236,13 @@ __device__ __forceinline__ void mma_f16(uint32_t tmem_d, uint64_t adesc, uint64_
 __device__ __forceinline__ void mma_commit(uint64_t* bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
                : "memory");
+}
+
+// true in one lane of the (converged) warp, the same lane every time
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\tselp.u32 %0, 1, 0, q;\n\t}" : "=r"(p));
+  return p != 0;
 }
 
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
@@ -532,36 +540,61 @@ struct TcArgs {
   unsigned long long wait_ns;   // limit of every bounded wait
   int selftest;             // 1: the producer first waits on a barrier nothing arrives at (timeout path test)
   int general;              // general storage: output tiles on both sides of the diagonal, weight 1 in e^2
-  int split_supply;         // 1: the B units come through the copy warps (cp.async), the A units by bulk copy
   const double* dsq;        // S_ii = sum_k x_ik^2 in FP64 per global row (nullptr: from the tensor cores)
   int glo, ghi;             // slice-pair groups s + t of this launch (ghi - glo <= 3)
   int emode;                // 0: full epilogue; 1: write S (this launch's groups) into the output tiles only;
                             // 2: full epilogue on S + the S already in the output tiles
 };
 
-// A pipeline stage holds one sub-step: two A units and two B units, a unit
-// being one slice of a 4-tile panel (128 rows x 32, 8 KB, 8-row groups 512 B
-// apart).  A sub-step record (32 bits) tells the MMA issuer what it holds:
-//   bits 3u..3u+2: slice of unit u (u = 0, 1: A units, u = 2, 3: B units),
-//   bits 12-15: product mask, bit (2 i + j) for A unit i x B unit j,
-//   bit 16: end of the super-tile, bit 17: no more super-tiles, bit 18: end of an
-//   accumulation segment (no data).  A super-tile whose K loop has at least
+// Shared memory holds two rings of RING operand units, one for each side of the
+// product, a unit being one slice of a 4-tile panel (128 rows x 32, 8 KB, 8-row
+// groups 512 B apart).  A sub-step takes the next one or two units of each ring:
+// up to two adjacent slices of the A record and up to two of the B record, each
+// side one bulk copy of 8 or 16 KB (two where the ring wraps).  A sub-step
+// record (32 bits; the MMA issuer sees the lower 16) tells the issuers what to
+// copy and the MMA issuer what to multiply:
+//   bits 0-2: 1 + the group (s + t - glo) of the first A x first B slice,
+//   bits 4-7: product mask, bit (2 i + j) for A slice a0 + i x B slice b0 + j,
+//   bits 8-11: groups its products write,
+//   bit 12: end of the super-tile, bit 13: no more super-tiles, bit 14: end of an
+//   accumulation segment (no data),
+//   bits 20-21, 22-24: A slices to copy and the first of them, bits 25-26, 27-29:
+//   the same for B.  A super-tile whose K loop has at least
 //   seg_min K steps closes a segment after every 16 K steps: the epilogue adds
 //   the segment's exact fixed-point sums into the scratch and frees the TMEM,
 //   so no FP32 accumulator sums more than 16 K steps (512 products per
 //   element) and the groups stay exact for dense operands.
+//
+// What bounds the kernel is how fast its single-thread loops run, not the copy
+// path (a lone thread that issues 16 KB bulk copies fills 72 B per SM cycle out
+// of L2; a K step needs 27 KB and has 210 cycles of MMAs) and not the tensor
+// pipe (25%).  So the producer side is three warps: the planner finds the K
+// steps of a tile, reads their record headers and writes batches of sub-steps
+// (at most 32 K steps each) into NPLAN buffers; two issuers copy the units, one
+// the A side, one the B side.  The loops of the issuers and of the MMA issuer
+// are run by whole warps on warp-uniform values, with one elected lane acting:
+// tcgen05.mma and cp.async.bulk take their operands from uniform registers, and
+// in code that only one lane enters each operand is moved there at every use
+// (240 cycles a product and 130 a copy; 110 and about 60 with uniform loops).
+// Cycles per super-tile, water-like N = 24,000 and 96,000: one producer warp
+// 126,000 and 96,000; planner and one issuer 120,000 and 81,000 (with the
+// shorter epilogue loops); two issuers, uniform loops and 16 epilogue warps
+// 103,000 and 67,000.  Whole runs 172 -> 145 ms and 1,250 -> 855 ms.
 constexpr int UNIT_BYTES = 4 * SLICE_BYTES;
-constexpr int STAGE_BYTES = 4 * UNIT_BYTES;
-constexpr int STAGES = 6;
-constexpr uint32_t REC_END = 1u << 16;
-constexpr int EPI_WARPS = 8;                       // epilogue warps 2..9
-constexpr int COPY_WARPS = 2;                      // copy warps 10..11 (B units by 16-byte cp.async)
-constexpr int TC_THREADS = 32 * (2 + EPI_WARPS + COPY_WARPS);   // + producer warp 0, MMA warp 1
-constexpr uint32_t REC_LAST = 1u << 17;   // no more super-tiles (no data)
-constexpr uint32_t REC_SEG = 1u << 18;    // end of an accumulation segment of the super-tile (no data)
+constexpr int RING = 12;                           // units of one side's ring (96 KB; 192 KB in all)
+constexpr int STEPS = 16;                          // sub-steps in flight
+constexpr int NPLAN = 4;                           // batches between the planner and the issuer
+constexpr int PLAN = 104;                          // entries of a batch: 32 K steps x 3 + segment ends
+constexpr uint32_t REC_END = 1u << 12;
+constexpr int EPI_WARPS = 16;                      // epilogue warps 2..17
+constexpr int ISSUE_WARP = 2 + EPI_WARPS;          // issuer warps 18 (A units) and 19 (B units)
+constexpr int TC_THREADS = 32 * (2 + EPI_WARPS + 2);   // + planner warp 0, MMA warp 1
+constexpr uint32_t REC_LAST = 1u << 13;   // no more super-tiles (no data)
+constexpr uint32_t REC_SEG = 1u << 14;    // end of an accumulation segment of the super-tile (no data)
+constexpr uint32_t REC_CTL = REC_END | REC_LAST | REC_SEG;
 constexpr uint32_t SEG_LAST = 1u << 31;   // segment record flag: last segment of its super-tile
 constexpr int SEG_RING = 4;               // accumulation segments in flight between MMA and epilogue
-constexpr int NSLOT = 3;                  // tiles in flight between the producer and the epilogue (2: 3% slower, 4: same)
+constexpr int NSLOT = 3;                  // tiles in flight between the planner and the epilogue
 constexpr int SEG_KSTEPS = 16;            // K steps per accumulation segment of a segmented tile (default)
 
 // record header byte: first nonzero slice (bits 0-2), tiles present (bits 4-7)
@@ -569,7 +602,7 @@ constexpr uint32_t HEAD_NONE = 0x07u;   // header of a K index outside the step 
 
 template <int K>
 struct TcCfg {
-  static constexpr int SMEM = STAGES * STAGE_BYTES + 1024 + 128 * 16;
+  static constexpr int SMEM = 2 * RING * UNIT_BYTES + 2048 + NPLAN * PLAN * 16;
 };
 
 template <int K>
@@ -580,32 +613,36 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_square_tc(TcArgs a) {
   // slices take every group in one launch (compile-time constants)
   const int glo = K == 5 ? a.glo : 0, ghi = K == 5 ? a.ghi : K - 1, emode = K == 5 ? a.emode : 0;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
-  unsigned char* stage_base = smem_raw;
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem_raw + STAGES * STAGE_BYTES);
-  uint64_t* empty = full + STAGES;
-  uint64_t* acc_full = empty + STAGES;     // [SEG_RING] MMAs of a segment done (commit) + its record written
-  uint64_t* tile_full = acc_full + SEG_RING;   // [NSLOT] tile slot written by the producer
+  unsigned char* ring = smem_raw;
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem_raw + 2 * RING * UNIT_BYTES);   // [STEPS] the sub-step's units are in
+  uint64_t* empty = full + STEPS;          // [STEPS] its products are done
+  uint64_t* acc_full = empty + STEPS;      // [SEG_RING] MMAs of a segment done (commit) + its record written
+  uint64_t* tile_full = acc_full + SEG_RING;   // [NSLOT] tile slot written by the planner
   uint64_t* tile_empty = tile_full + NSLOT;    // [NSLOT] epilogue done with the tile slot (one arrive per warp)
   uint64_t* drain = tile_empty + NSLOT;    // MMAs issued before the exit are complete
   uint64_t* tmem_empty = drain + 1;        // [SEG_RING] every epilogue warp has read the segment's TMEM
   uint64_t* probe = tmem_empty + SEG_RING; // self-test: a barrier that nothing arrives at
-  uint64_t* fill = probe + 1;              // [STAGES] stage record written: the copy warps may fill B
-  const __half** srcb = reinterpret_cast<const __half**>(fill + STAGES);   // [STAGES] B record of the stage
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(srcb + STAGES);
+  uint64_t* plan_full = probe + 1;         // [NPLAN] batch written by the planner
+  uint64_t* plan_empty = plan_full + NPLAN;    // [NPLAN] batch taken by the issuer
+  uint32_t* rec = reinterpret_cast<uint32_t*>(plan_empty + NPLAN);   // [STEPS] bits 0-15 of the sub-step's record, ring places of A0, A1, B0, B1
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(rec + STEPS);
   int32_t* tslot = reinterpret_cast<int32_t*>(tmem_slot + 2);      // [NSLOT] super-tile list index, -1: none
   int32_t* kcount = tslot + NSLOT;                                  // [NSLOT][16] triplets per output tile
   uint32_t* gmap = reinterpret_cast<uint32_t*>(kcount + 16 * NSLOT);   // [SEG_RING] groups written, block of each, last flag
-  uint32_t* rec = gmap + SEG_RING;                                  // [STAGES] sub-step records
-  int32_t* status = reinterpret_cast<int32_t*>(rec + STAGES);      // [0] a wait timed out
-  uint4* ulist = reinterpret_cast<uint4*>(smem_raw + STAGES * STAGE_BYTES + 1024);   // [128] sub-steps of a batch
+  int32_t* bcnt = reinterpret_cast<int32_t*>(gmap + SEG_RING);     // [NPLAN] entries of a batch
+  int32_t* status = bcnt + NPLAN;                                   // [0] a wait timed out
+  uint4* steps = reinterpret_cast<uint4*>(smem_raw + 2 * RING * UNIT_BYTES + 1024);   // [8][8] sub-steps of (first A, first B slice)
+  uint4* plan = steps + 64;                                         // [NPLAN][PLAN] record, A unit, B unit, pass
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
-    for (int s = 0; s < STAGES; ++s) {
-      // the producer's arrival (with the bulk bytes), plus one per copy-warp thread
-      mbar_init(&full[s], 1 + (a.split_supply ? 32 * COPY_WARPS : 0));
+    for (int s = 0; s < STEPS; ++s) {
+      mbar_init(&full[s], 2);     // each issuer's arrival, with its bulk bytes
       mbar_init(&empty[s], 1);
-      mbar_init(&fill[s], 1);
+    }
+    for (int b = 0; b < NPLAN; ++b) {
+      mbar_init(&plan_full[b], 1);
+      mbar_init(&plan_empty[b], 2);   // both issuers
     }
     for (int b = 0; b < SEG_RING; ++b) {
       mbar_init(&acc_full[b], 2);
@@ -632,63 +669,74 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_square_tc(TcArgs a) {
   const uint32_t tmem = *tmem_slot;
   const int total = *a.count;
 
-  // Persistent and warp-specialised: the producer (warp 0) takes super-tiles
-  // from the work counter and streams their operand slices; the MMA issuer
+  // Persistent and warp-specialised: the planner (warp 0) takes super-tiles from
+  // the work counter, the issuers (warps 18, 19) stream their operand slices; the MMA issuer
   // (warp 1) accumulates each tile in TMEM blocks of 128 columns taken on
-  // first use; the epilogue (warps 2-9) finishes tile i while tiles i + 1 and
+  // first use; the epilogue (warps 2-17) finishes tile i while tiles i + 1 and
   // i + 2 are being loaded and multiplied.  Tiles pass through NSLOT slots.
   if (warp == 0) {
-    // ---------------- producer warp.  The record headers of 32 K steps are
+    // ---------------- planner warp.  The record headers of 32 K steps are
     // fetched at a time (lane j: step j), one batch ahead of their use; the
-    // lanes turn them into the batch's list of sub-steps in shared memory, and
-    // lanes 0-3 issue the sub-steps, lane u copying unit u (A0, A1, B0, B1) and
-    // lane 0 writing the stage record and arming its barrier.  Every lane keeps
-    // its own copy of the stage counter; no warp votes per sub-step.
-    int step = 0;
-    int emitted = 0;   // stages whose copies were issued (lane 0's view)
-    bool ok = true;
-    // lanes 0-3: one sub-step (srcA / srcB: the K step's A and B panel records).
-    // Lane 0 waits for the stage and the others take its result, so the four
-    // lanes stay on the same stage phase.
-    auto emit = [&](uint32_t rv, const __half* srcA, const __half* srcB) -> bool {
-      const int s = step % STAGES;
-      const uint32_t par = ((step / STAGES) & 1) ^ 1;
-      ++step;
-      int good = 1;
-      if (lane == 0) good = mbar_wait(&empty[s], par) ? 1 : 0;
-      good = __shfl_sync(0xFu, good, 0);
-      if (!good) {
-        if (lane == 0) {
-          status[0] = 1;
-          note_timeout(a.err, 1);
+    // lanes turn them into the batch's list of sub-steps.
+    // steps[8 fa + fb]: the sub-steps of a K step whose A record starts at slice
+    // fa and whose B record at fb -- the pairs s >= fa, t >= fb with
+    // glo <= s + t <= ghi (the launch's group window), two A and two B slices
+    // each; the B pair starts where A slice a0 + 1 meets glo.  At most three for
+    // every window used (x, y, z: records; w: their number).
+    for (int e = lane; e < 64; e += 32) {
+      const int fa = e >> 3, fb = e & 7;
+      uint32_t rv[3] = {0u, 0u, 0u};
+      int ns = 0;
+      for (int a0 = fa; a0 <= K - 1 && a0 + fb <= ghi; a0 += 2) {
+        for (int b0 = max(fb, glo - a0 - 1); b0 <= K - 1 && a0 + b0 <= ghi; b0 += 2) {
+          uint32_t mask = 0;
+          for (int i = 0; i < 2; ++i)
+            for (int j = 0; j < 2; ++j) {
+              const int si = a0 + i, tj = b0 + j;
+              if (si <= K - 1 && tj <= K - 1 && si + tj >= glo && si + tj <= ghi) mask |= 1u << (2 * i + j);
+            }
+          if (!mask) continue;
+          const int base = a0 + b0 - glo;     // >= -1
+          const uint32_t need = ((((mask & 1u) | ((mask & 6u) ? 2u : 0u) | ((mask & 8u) ? 4u : 0u)) << (base + 1)) >> 1) & 0xFu;
+          const int uA0 = (mask & 3u) ? 1 : 0, uA1 = (mask & 12u) ? 1 : 0;
+          const int uB0 = (mask & 5u) ? 1 : 0, uB1 = (mask & 10u) ? 1 : 0;
+          const uint32_t v = (uint32_t)(base + 1) | (mask << 4) | (need << 8) | ((uint32_t)(uA0 + uA1) << 20) |
+                             ((uint32_t)(a0 + 1 - uA0) << 22) | ((uint32_t)(uB0 + uB1) << 25) |
+                             ((uint32_t)(b0 + 1 - uB0) << 27);
+          if (ns == 0) rv[0] = v;
+          else if (ns == 1) rv[1] = v;
+          else rv[2] = v;
+          ++ns;
         }
-        return false;
       }
-      const uint32_t mask = (rv & (REC_END | REC_LAST | REC_SEG)) ? 0u : (rv >> 12) & 0xFu;
-      // units A0, A1, B0, B1 read by a product of the mask; with the split
-      // supply the B units go to the copy warps
-      uint32_t use = ((mask & 0x3u) ? 1u : 0u) | ((mask & 0xCu) ? 2u : 0u) | ((mask & 0x5u) ? 4u : 0u) |
-                     ((mask & 0xAu) ? 8u : 0u);
-      if (a.split_supply) use &= 0x3u;
-      if (lane == 0) {
-        rec[s] = rv;
-        srcb[s] = srcB;
-        mbar_expect_tx(&full[s], (uint32_t)__popc(use) * UNIT_BYTES);
-      }
-      if ((use >> lane) & 1u)
-        bulk_g2s(stage_base + s * STAGE_BYTES + lane * UNIT_BYTES,
-                 (lane < 2 ? srcA : srcB) + (int64_t)((rv >> (3 * lane)) & 7u) * (UNIT_BYTES / 2), UNIT_BYTES,
-                 &full[s]);
-      if (a.split_supply && lane == 0) mbar_arrive(&fill[s]);   // release: record and B source visible
-      emitted = step;
-      return true;
+      steps[e] = make_uint4(rv[0], rv[1], rv[2], (uint32_t)ns);
+    }
+    __syncwarp();
+    bool ok = true;
+    int nbat = 0;      // batches handed to the issuer
+    // all lanes: wait for the next batch buffer; false on timeout
+    auto batch_open = [&]() -> bool {
+      int good = 1;
+      if (lane == 0) good = mbar_wait_sleep(&plan_empty[nbat % NPLAN], (((uint32_t)(nbat / NPLAN)) & 1u) ^ 1u) ? 1 : 0;
+      good = __shfl_sync(FULLW, good, 0);
+      if (!good && lane == 0) { status[0] = 1; note_timeout(a.err, 1); }
+      return good != 0;
     };
-    // all lanes: a control sub-step (no data) through lanes 0-3
-    auto emit_ctl = [&](uint32_t rv) -> bool {
-      bool r = true;
-      if (lane < 4) r = emit(rv, nullptr, nullptr);
-      else ++step;
-      return __shfl_sync(FULLW, r ? 1 : 0, 0) != 0;
+    // all lanes: hand the batch's n entries to the issuer
+    auto batch_close = [&](int n) {
+      __syncwarp();
+      if (lane == 0) {
+        bcnt[nbat % NPLAN] = n;
+        mbar_arrive(&plan_full[nbat % NPLAN]);   // release: the entries are visible
+      }
+      ++nbat;
+    };
+    // all lanes: a batch of one control entry
+    auto batch_ctl = [&](uint32_t rv) -> bool {
+      if (!batch_open()) return false;
+      if (lane == 0) plan[(nbat % NPLAN) * PLAN] = make_uint4(rv, 0u, 0u, 0u);
+      batch_close(1);
+      return true;
     };
     // self-test of the timeout path: before any copy is issued, wait on a
     // barrier that nothing arrives at; the wait gives up after the wait limit,
@@ -703,6 +751,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_square_tc(TcArgs a) {
       }
       __syncwarp();
     }
+    int nidx = 0;      // next super-tile, taken from the work counter one tile ahead
+    if (lane == 0) nidx = atomicAdd(a.work, 1);
     for (int it = 0; ok; ++it) {
       const int b = it % NSLOT;
       // the slot's previous tile (it - NSLOT) has left the epilogue
@@ -710,21 +760,20 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_square_tc(TcArgs a) {
       if (lane == 0) good = mbar_wait_sleep(&tile_empty[b], (((uint32_t)(it / NSLOT)) & 1u) ^ 1u) ? 1 : 0;
       good = __shfl_sync(FULLW, good, 0);
       if (!good) {
-        if (lane == 0) { status[0] = 1; note_timeout(a.err, 2); }
+        if (lane == 0) { status[0] = 1; note_timeout(a.err, 1); }
         break;
       }
-      int idx = 0;
-      if (lane == 0) idx = atomicAdd(a.work, 1);
-      idx = __shfl_sync(FULLW, idx, 0);
+      const int idx = __shfl_sync(FULLW, nidx, 0);
       if (idx >= total || *(volatile int32_t*)status != 0) {
         // no more tiles: tell the epilogue (slot) and the MMA issuer (record)
         if (lane == 0) {
           tslot[b] = -1;
           mbar_arrive(&tile_full[b]);
         }
-        emit_ctl(REC_LAST);
+        batch_ctl(REC_LAST);
         break;
       }
+      if (lane == 0) nidx = atomicAdd(a.work, 1);
       const int stile = a.list[idx];
       const int R = stile / a.nsr, C = stile % a.nsr;
       // the epilogue learns the tile now (it drains segments while the tile is produced)
@@ -734,7 +783,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_square_tc(TcArgs a) {
       }
       // K steps of the tile (both passes): long K loops are cut into segments
       int ktot = 0;
-      if (a.seg_min > 0) {
+      if (a.seg_min > 0 && a.nb * (1 + a.two_pass) >= a.seg_min) {
         for (int pass = 0; pass < 1 + a.two_pass; ++pass) {
           const TcOperand& oa = pass == 0 ? a.P : a.Q;
           const TcOperand& ob = pass == 0 ? a.Q : a.P;
@@ -745,7 +794,20 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_square_tc(TcArgs a) {
       }
       const bool segmented = a.seg_min > 0 && ktot >= a.seg_min;
       int kdone = 0;
-      int kc = 0;   // lane t < 16: K steps with A tile t / 4 and B tile t % 4 both present
+      // triplet counts: K steps with A tile q and B tile y both present, byte y of
+      // acc[q] in every lane, moved to kc (lane 4 q + y) before a byte overflows
+      int kc = 0, nacc = 0;
+      uint32_t acc[4] = {0u, 0u, 0u, 0u};
+      auto flush_counts = [&]() {
+#pragma unroll
+        for (int t = 0; t < 16; ++t) {
+          const int s = __reduce_add_sync(FULLW, (int)((acc[t >> 2] >> (8 * (t & 3))) & 0xFFu));
+          if (lane == t) kc += s;
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[q] = 0u;
+        nacc = 0;
+      };
       for (int pass = 0; pass < 1 + a.two_pass && ok; ++pass) {
         // pass 0: A = P (rows I), B = Q (rows J); pass 1: A = Q, B = P
         const TcOperand& opA = pass == 0 ? a.P : a.Q;
@@ -789,9 +851,19 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_square_tc(TcArgs a) {
             const int pbL = __shfl_sync(FULLW, pb, Lc);
             const int exL = __shfl_sync(FULLW, excl, Lc);
             if (j < total) {
+              // position of the set bit number j - exL
               uint32_t m = mL;
-              for (int r = j - exL; r > 0; --r) m &= m - 1;
-              const uint32_t below = (1u << (__ffs(m) - 1)) - 1u;
+              int r = j - exL, pos = 0;
+#pragma unroll
+              for (int h = 16; h > 0; h >>= 1) {
+                const int c = __popc(m & ((1u << h) - 1u));
+                if (r >= c) {
+                  r -= c;
+                  m >>= h;
+                  pos += h;
+                }
+              }
+              const uint32_t below = (1u << pos) - 1u;
               ea = paL + __popc(maL & below);
               eb = pbL + __popc(mbL & below);
               ha = opA.head[ea];
@@ -805,38 +877,13 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_square_tc(TcArgs a) {
             int ea_n, eb_n;
             uint32_t ha_n, hb_n;
             fetch(jb + 32 + lane, ea_n, eb_n, ha_n, hb_n);   // next batch, in flight during this one
-            // triplet counts: K steps of this batch with A tile x and B tile y present
-            const uint32_t pa4 = (ha >> 4) & 0xFu, pb4 = (hb >> 4) & 0xFu;
+            const uint32_t pa4 = (ha >> 4) & 0xFu;
+            const uint32_t eb4 = (((hb >> 4) & 0xFu) * 0x00204081u) & 0x01010101u;   // one byte per B tile
 #pragma unroll
-            for (int t = 0; t < 16; ++t) {
-              const int c16 = __popc(__ballot_sync(FULLW, (pa4 >> (t >> 2)) & (pb4 >> (t & 3)) & 1u));
-              if (lane == t) kc += c16;
-            }
-            // sub-steps of this lane's K step: pairs s >= fa, t >= fb with
-            // glo <= s + t <= ghi (the launch's group window), two A and two B
-            // slices each; the B pair starts where A slice a0 + 1 meets glo
-            // (at most three sub-steps for every window used)
-            const int fa = (int)(ha & 7u), fb = (int)(hb & 7u);
-            uint32_t rv0 = 0u, rv1 = 0u, rv2 = 0u;
-            int ns = 0;
-            for (int a0 = fa; a0 <= K - 1 && a0 + fb <= ghi; a0 += 2) {
-              for (int b0 = max(fb, glo - a0 - 1); b0 <= K - 1 && a0 + b0 <= ghi; b0 += 2) {
-                uint32_t mask = 0;
-                for (int i = 0; i < 2; ++i)
-                  for (int jj = 0; jj < 2; ++jj) {
-                    const int si = a0 + i, tj = b0 + jj;
-                    if (si <= K - 1 && tj <= K - 1 && si + tj >= glo && si + tj <= ghi)
-                      mask |= 1u << (2 * i + jj);
-                  }
-                if (!mask) continue;
-                const uint32_t rv = (uint32_t)a0 | ((uint32_t)min(a0 + 1, K - 1) << 3) | ((uint32_t)b0 << 6) |
-                                    ((uint32_t)min(b0 + 1, K - 1) << 9) | (mask << 12);
-                if (ns == 0) rv0 = rv;
-                else if (ns == 1) rv1 = rv;
-                else rv2 = rv;
-                ++ns;
-              }
-            }
+            for (int q = 0; q < 4; ++q) acc[q] += ((pa4 >> q) & 1u) ? eb4 : 0u;
+            if (++nacc == 255) flush_counts();
+            const uint4 sv = steps[(ha & 7u) * 8u + (hb & 7u)];   // HEAD_NONE: no sub-steps
+            const int ns = (int)sv.w;
             // a segmented tile also closes a segment before every seg_ksteps-th K
             // step inside the batch (the batch end closes one too)
             const int lead = (segmented && lane > 0 && (lane % a.seg_ksteps) == 0 && jb + lane < total) ? 1 : 0;
@@ -846,30 +893,25 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_square_tc(TcArgs a) {
               const int v = __shfl_up_sync(FULLW, soff, o);
               if (lane >= o) soff += v;
             }
-            const int nsub = __shfl_sync(FULLW, soff, 31);
+            int nsub = __shfl_sync(FULLW, soff, 31);
             soff -= ns;
-            if (lead) ulist[soff - 1] = make_uint4(REC_SEG, 0u, 0u, 0u);
-            if (ns > 0) ulist[soff] = make_uint4(rv0, (uint32_t)ea, (uint32_t)eb, 0u);
-            if (ns > 1) ulist[soff + 1] = make_uint4(rv1, (uint32_t)ea, (uint32_t)eb, 0u);
-            if (ns > 2) ulist[soff + 2] = make_uint4(rv2, (uint32_t)ea, (uint32_t)eb, 0u);
-            __syncwarp();
-            bool lok = true;
-            if (lane < 4) {
-              for (int u = 0; u < nsub; ++u) {
-                const uint4 en = ulist[u];
-                if (!emit(en.x, opA.data + (int64_t)en.y * (K * UNIT_BYTES / 2),
-                          opB.data + (int64_t)en.z * (K * UNIT_BYTES / 2))) {
-                  lok = false;
-                  break;
-                }
-              }
-            } else {
-              step += nsub;
-            }
-            ok = __all_sync(FULLW, lok);
-            __syncwarp();   // the list is rebuilt for the next batch
+            ok = batch_open();
+            if (!ok) break;
+            uint4* ul = plan + (nbat % NPLAN) * PLAN;
+            const uint32_t ua = (uint32_t)ea * K, ub = (uint32_t)eb * K;
+            auto entry = [&](uint32_t rv) {
+              return make_uint4(rv, ua + ((rv >> 22) & 7u), ub + ((rv >> 27) & 7u), (uint32_t)pass);
+            };
+            if (lead) ul[soff - 1] = make_uint4(REC_SEG, 0u, 0u, 0u);
+            if (ns > 0) ul[soff] = entry(sv.x);
+            if (ns > 1) ul[soff + 1] = entry(sv.y);
+            if (ns > 2) ul[soff + 2] = entry(sv.z);
             kdone += min(32, total - jb);
-            if (segmented && ok && kdone < ktot) ok = emit_ctl(REC_SEG);
+            if (segmented && kdone < ktot) {
+              if (lane == 0) ul[nsub] = make_uint4(REC_SEG, 0u, 0u, 0u);
+              ++nsub;
+            }
+            batch_close(nsub);
             ea = ea_n;
             eb = eb_n;
             ha = ha_n;
@@ -877,21 +919,100 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_square_tc(TcArgs a) {
           }
         }
       }
-      // counts before the end record: the record's barrier, then the segment's,
-      // order them before the epilogue's reads
+      // counts before the end record: the barriers of its batch, its sub-step and
+      // its segment order them before the epilogue's reads
+      flush_counts();
       if (lane < 16) kcount[b * 16 + lane] = kc;
       __syncwarp();
-      if (ok) ok = emit_ctl(REC_END);
+      if (ok) ok = batch_ctl(REC_END);
     }
-    // after a timeout anywhere in the CTA: wait (bounded) until the copies of
-    // the last STAGES emitted stages have landed, so that no bulk copy into
-    // this CTA's shared memory is in flight when the CTA exits
-    if (lane == 0 && *(volatile int32_t*)status != 0) {
-      for (int j = max(0, emitted - STAGES); j < emitted; ++j)
-        if (!mbar_wait(&full[j % STAGES], (uint32_t)(j / STAGES) & 1u)) note_timeout(a.err, 9);
+  } else if (warp >= ISSUE_WARP) {
+    // ---------------- issuers: one thread copies the A units of every planned
+    // sub-step into A's ring, the other the B units into B's, in order, once
+    // the sub-steps before it have left enough units free.
+    // As in the MMA issuer the whole warp runs the loop and an elected lane acts.
+    const bool leader = elect_one();
+    const int lead = __ffs(__ballot_sync(FULLW, leader)) - 1;
+    const int side = __shfl_sync(FULLW, warp, 0) - ISSUE_WARP;      // 0: A, 1: B
+    const uint32_t first_used = side ? 0x50u : 0x30u;       // products that read the side's first slice
+    const uint32_t mine = smem_u32(ring) + (uint32_t)side * (RING * UNIT_BYTES);
+    int s = 0, q = 0;              // next sub-step slot to issue, next to be released
+    uint32_t qpar = 0;             // phase of slot q
+    int busy = 0;                  // slots issued and not released
+    int pos = 0, nfree = RING;     // next unit of the ring, free units
+    uint32_t held = 0u;            // units of sub-step slot s: bits 2 s, 2 s + 1
+    int head = 0;                  // sub-steps issued
+    bool done = false;
+    for (int bat = 0; !done; ++bat) {
+      if (!__shfl_sync(FULLW, mbar_wait_sleep(&plan_full[bat % NPLAN], (uint32_t)(bat / NPLAN) & 1u) ? 1 : 0, lead)) {
+        if (leader) {
+          status[0] = 1;
+          note_timeout(a.err, 8);
+        }
+        break;
+      }
+      const uint4* ul = plan + (bat % NPLAN) * PLAN;
+      const int n = __shfl_sync(FULLW, bcnt[bat % NPLAN], 0);
+      uint4 nx = ul[0];
+      for (int u = 0; u < n && !done; ++u) {
+        const uint32_t rv = __shfl_sync(FULLW, nx.x, 0);
+        const uint32_t unit = __shfl_sync(FULLW, side ? nx.z : nx.y, 0);
+        const bool swap = __shfl_sync(FULLW, nx.w, 0) != 0u;
+        nx = ul[min(u + 1, n - 1)];
+        const int m = (int)((rv >> (side ? 25 : 20)) & 3u);
+        while (nfree < m || busy == STEPS) {
+          if (!__shfl_sync(FULLW, mbar_wait(&empty[q], qpar) ? 1 : 0, lead)) {
+            if (leader) {
+              status[0] = 1;
+              note_timeout(a.err, 2);
+            }
+            done = true;
+            break;
+          }
+          nfree += (int)((held >> (2 * q)) & 3u);
+          --busy;
+          if (++q == STEPS) { q = 0; qpar ^= 1u; }
+        }
+        if (done) break;
+        held = (held & ~(3u << (2 * s))) | ((uint32_t)m << (2 * s));
+        nfree -= m;
+        ++busy;
+        // ring places of the side's two slices (an unused first slice takes none)
+        const int p0 = pos;
+        int p1 = pos + ((rv & first_used) ? 1 : 0);
+        if (p1 == RING) p1 = 0;
+        pos += m;
+        if (pos >= RING) pos -= RING;
+        const __half* base = swap == (side != 0) ? a.P.data : a.Q.data;
+        const unsigned char* src = reinterpret_cast<const unsigned char*>(base) + (uint64_t)unit * UNIT_BYTES;
+        const uint32_t bytes = (uint32_t)m * UNIT_BYTES, part = m == 2 && p0 == RING - 1 ? UNIT_BYTES : bytes;
+        if (leader) {
+          uint8_t* rb = reinterpret_cast<uint8_t*>(rec + s);
+          if (side == 0) *reinterpret_cast<uint16_t*>(rb) = (uint16_t)rv;
+          rb[2 + side] = (uint8_t)(p0 | (p1 << 4));
+          mbar_expect_tx(&full[s], bytes);
+          if (m > 0) bulk_g2s(mine + p0 * UNIT_BYTES, src, part, &full[s]);
+          if (part != bytes) bulk_g2s(mine, src + UNIT_BYTES, UNIT_BYTES, &full[s]);
+        }
+        __syncwarp();
+        ++head;
+        if (++s == STEPS) s = 0;
+        if (rv & REC_LAST) done = true;
+      }
+      if (leader) mbar_arrive(&plan_empty[bat % NPLAN]);
+      __syncwarp();
     }
-  } else if (warp == 1 && lane == 0) {
-    // ---------------- MMA issuer.  TMEM is four blocks of 128 columns; a group
+    // no bulk copy into this CTA's shared memory may be in flight when the CTA
+    // exits: wait (bounded) for those of the last STEPS sub-steps
+    if (leader)
+      for (int j = max(0, head - STEPS); j < head; ++j)
+        if (!mbar_wait(&full[j % STEPS], (uint32_t)(j / STEPS) & 1u)) {
+          status[0] = 1;
+          note_timeout(a.err, 9);
+        }
+  } else if (warp == 1) {
+    // ---------------- MMA issuer: the whole warp runs the loop, so that its values
+    // are warp-uniform; one elected lane issues.  TMEM is four blocks of 128 columns; a group
     // accumulator of a segment (a whole super-tile, or 32 of its K steps) takes
     // a free block on its first product, and the blocks of a segment return to
     // the pool once every epilogue warp has read them (one arrival per warp on
@@ -903,10 +1024,22 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_square_tc(TcArgs a) {
     int seg = 0;                   // segments published
     unsigned long long nprod = 0;
     bool ok = true, done = false;
+    // the shared-memory descriptor of a unit is that of the ring's start plus
+    // a constant (the start-address field holds address / 16 in 14 bits; every
+    // address here is below 2^18)
+    const uint64_t dring = make_desc(smem_u32(ring), 128, 512);
+    const uint32_t dlo = (uint32_t)dring & 0xFFFFu;              // start address / 16 (below 2^14 for every unit)
+    const uint64_t dhi = dring & ~0xFFFFull;
+    const bool leader = elect_one();
+    const int lead = __ffs(__ballot_sync(FULLW, leader)) - 1;
+    // bounded wait of the whole warp: the leader's result in every lane
+    auto wait = [&](uint64_t* bar, uint32_t parity) -> bool {
+      return __shfl_sync(FULLW, mbar_wait(bar, parity) ? 1 : 0, lead) != 0;
+    };
     // take back the blocks of the oldest segment that still holds some; false on timeout
     auto reclaim = [&]() -> bool {
-      if (!mbar_wait(&tmem_empty[released & (SEG_RING - 1)], ((uint32_t)released >> 2) & 1u)) {
-        note_timeout(a.err, 4);
+      if (!wait(&tmem_empty[released & (SEG_RING - 1)], ((uint32_t)released >> 2) & 1u)) {
+        if (leader) note_timeout(a.err, 4);
         return false;
       }
       tc_fence_after();
@@ -919,63 +1052,63 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_square_tc(TcArgs a) {
       ++released;
       return true;
     };
-    // stage counter and phase kept incrementally; the shared-memory descriptor
-    // of a unit is the stage's descriptor plus a constant (the start-address
-    // field holds address / 16 in 14 bits; every address here is below 2^18)
-    int s = 0;
+    int s = 0;      // next sub-step slot and its phase
     uint32_t par = 0;
-    const uint64_t d0 = make_desc(smem_u32(stage_base), 128, 512);
     while (ok && !done) {
       uint32_t written = 0, gblk = 0, used = 0;
       uint32_t kind = 0;
       for (;;) {
         const int cs = s;
         const uint32_t cpar = par;
-        if (++s == STAGES) { s = 0; par ^= 1u; }
-        if (!mbar_wait(&full[cs], cpar)) { ok = false; note_timeout(a.err, 3); break; }
-        tc_fence_after();
-        // units written by cp.async (generic proxy) are read by the MMAs (async proxy)
-        if (a.split_supply) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        const uint32_t rv = rec[cs];
-        if (rv & (REC_END | REC_LAST | REC_SEG)) {
-          mma_commit(&empty[cs]);
-          kind = rv & (REC_END | REC_LAST | REC_SEG);
+        if (++s == STEPS) { s = 0; par ^= 1u; }
+        if (!wait(&full[cs], cpar)) {
+          ok = false;
+          if (leader) note_timeout(a.err, 3);
           break;
         }
-        const uint64_t ds = d0 + (uint64_t)(cs * (STAGE_BYTES >> 4));
-#pragma unroll
-        for (int i = 0; i < 2; ++i) {
-#pragma unroll
-          for (int j = 0; j < 2; ++j) {
-            if (!((rv >> (12 + 2 * i + j)) & 1u)) continue;
-            // group relative to the launch's window (at most four groups live)
-            const int g = (int)((rv >> (3 * i)) & 7u) + (int)((rv >> (6 + 3 * j)) & 7u) - glo;
-            if (!((written >> g) & 1u)) {
-              while (free_mask == 0u && ok) ok = reclaim();
-              if (!ok) break;
-              const uint32_t blk = (uint32_t)(__ffs(free_mask) - 1);
-              free_mask &= ~(1u << blk);
-              used |= 1u << blk;
-              gblk |= blk << (2 * g);
-            }
-            const uint32_t dcol = tmem + ((gblk >> (2 * g)) & 3u) * ST;
-            const uint32_t acc = (written >> g) & 1u;
-#pragma unroll
-            for (int kk = 0; kk < 2; ++kk) {
-              const uint64_t ad = ds + (uint64_t)((i * UNIT_BYTES + kk * 256) >> 4);
-              const uint64_t bd = ds + (uint64_t)(((2 + j) * UNIT_BYTES + kk * 256) >> 4);
-              // the first MMA into a group accumulator of a segment overwrites it
-              // (the unit of the super-column as the M operand, that of the super-row
-              // as the N operand: TMEM holds the transposed super-tile)
-              mma_f16(dcol, bd, ad, (kk > 0 || acc) ? 1u : 0u);
-            }
-            written |= 1u << g;
-            ++nprod;
-          }
-          if (!ok) break;
+        tc_fence_after();
+        const uint32_t rv = __shfl_sync(FULLW, rec[cs], 0);
+        if (rv & REC_CTL) {
+          if (leader) mma_commit(&empty[cs]);
+          kind = rv & REC_CTL;
+          break;
         }
-        mma_commit(&empty[cs]);
+        // groups (relative to the launch's window, at most four live) that this
+        // segment has not written yet: take a TMEM block; their first MMA overwrites it
+        uint32_t fresh = (rv >> 8) & ~written & 0xFu;
+        for (uint32_t f = fresh; f != 0u; f &= f - 1u) {
+          const int g = __ffs(f) - 1;
+          while (free_mask == 0u && ok) ok = reclaim();
+          if (!ok) break;
+          const uint32_t blk = (uint32_t)(__ffs(free_mask) - 1);
+          free_mask &= ~(1u << blk);
+          used |= 1u << blk;
+          gblk |= blk << (2 * g);
+          written |= 1u << g;
+        }
         if (!ok) break;
+        const int base = (int)(rv & 7u) - 1;     // group of A0 x B0
+        const uint32_t a0 = dlo + ((rv >> 16) & 15u) * (UNIT_BYTES >> 4), a1 = dlo + ((rv >> 20) & 15u) * (UNIT_BYTES >> 4);
+        const uint32_t b0 = dlo + (((rv >> 24) & 15u) + RING) * (UNIT_BYTES >> 4);
+        const uint32_t b1 = dlo + ((rv >> 28) + RING) * (UNIT_BYTES >> 4);
+        const uint32_t gb = base >= 0 ? gblk >> (2 * base) : gblk << 2;    // blocks of groups base, base + 1, base + 2
+        uint32_t fr = base >= 0 ? fresh >> base : fresh << 1;
+        if (leader) {
+          // the unit of the super-column as the M operand, that of the super-row
+          // as the N operand: TMEM holds the transposed super-tile
+          auto product = [&](uint32_t ua, uint32_t ub, int k) {
+            const uint32_t dcol = tmem + ((gb >> (2 * k)) & 3u) * ST;
+            mma_f16(dcol, dhi | ub, dhi | ua, ((fr >> k) & 1u) ^ 1u);
+            mma_f16(dcol, dhi | (ub + 16u), dhi | (ua + 16u), 1u);
+          };
+          if (rv & (1u << 4)) { product(a0, b0, 0); }
+          if (rv & (1u << 5)) { product(a0, b1, 1); fr &= ~2u; }
+          if (rv & (1u << 6)) { product(a1, b0, 1); }
+          if (rv & (1u << 7)) { product(a1, b1, 2); }
+          mma_commit(&empty[cs]);
+        }
+        __syncwarp();
+        nprod += (unsigned)__popc((rv >> 4) & 0xFu);
       }
       if (!ok) break;
       if (kind & REC_LAST) { done = true; break; }
@@ -990,66 +1123,28 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_square_tc(TcArgs a) {
         case 2: pend2 = used; break;
         default: pend3 = used; break;
       }
-      gmap[q] = written | (gblk << 8) | ((kind & REC_END) ? SEG_LAST : 0u);
-      mma_commit(&acc_full[q]);    // arrives once every MMA of the segment has completed
-      mbar_arrive(&acc_full[q]);   // release: segment record visible to the epilogue
+      if (leader) gmap[q] = written | (gblk << 8) | ((kind & REC_END) ? SEG_LAST : 0u);
+      if (leader) {
+        mma_commit(&acc_full[q]);    // arrives once every MMA of the segment has completed
+        mbar_arrive(&acc_full[q]);   // release: segment record visible to the epilogue
+      }
+      __syncwarp();
       ++seg;
     }
     if (!ok) status[0] = 1;
     // slice-pair products issued (each 2 MMAs of 128 x 128 x 16)
-    if (a.err && nprod) atomicAdd(reinterpret_cast<unsigned long long*>(a.err + 2), nprod);
-    mma_commit(drain);
-    if (!mbar_wait(drain, 0)) { status[0] = 1; note_timeout(a.err, 5); }
-  } else if (warp >= 2 + EPI_WARPS) {
-    // ---------------- copy warps (split supply only).  Stage by stage, in the
-    // producer's order: wait until the producer has written the stage record
-    // (fill), copy the B units the record uses as 16-byte cp.async pieces (the
-    // 64 threads take every 64th piece of an 8 KB unit), then arrive on the
-    // stage's full barrier when this thread's copies have landed.  Control
-    // records carry no data but are arrived at all the same.
-    if (a.split_supply) {
-      const int t = threadIdx.x - 32 * (2 + EPI_WARPS);   // 0 .. 63
-      int ns = 0;
-      uint32_t npar = 0;
-      for (;;) {
-        const int s = ns;
-        const uint32_t par = npar;
-        if (++ns == STAGES) { ns = 0; npar ^= 1u; }
-        bool good = true;
-        if (lane == 0) good = mbar_wait_sleep(&fill[s], par);
-        good = __shfl_sync(FULLW, good ? 1 : 0, 0) != 0;
-        if (!good) {
-          if (lane == 0) {
-            status[0] = 1;
-            note_timeout(a.err, 8);
-          }
-          break;
-        }
-        const uint32_t rv = rec[s];
-        if (!(rv & (REC_END | REC_LAST | REC_SEG))) {
-          const uint32_t mask = (rv >> 12) & 0xFu;
-          const __half* srcB = srcb[s];
-#pragma unroll
-          for (int j = 0; j < 2; ++j) {
-            if (!(mask & (j == 0 ? 0x5u : 0xAu))) continue;
-            const char* src = reinterpret_cast<const char*>(srcB + (int64_t)((rv >> (6 + 3 * j)) & 7u) * (UNIT_BYTES / 2));
-            const uint32_t dst = smem_u32(stage_base + s * STAGE_BYTES + (2 + j) * UNIT_BYTES);
-#pragma unroll
-            for (int c = t; c < UNIT_BYTES / 16; c += 32 * COPY_WARPS)
-              asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + 16 * c), "l"(src + 16 * c)
-                           : "memory");
-          }
-        }
-        asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(&full[s])) : "memory");
-        if (rv & REC_LAST) break;
-      }
-      asm volatile("cp.async.wait_all;" ::: "memory");
+    if (leader && a.err && nprod) atomicAdd(reinterpret_cast<unsigned long long*>(a.err + 2), nprod);
+    if (leader) mma_commit(drain);
+    __syncwarp();
+    if (!wait(drain, 0)) {
+      status[0] = 1;
+      if (leader) note_timeout(a.err, 5);
     }
   } else if (warp >= 2) {
-    // ---------------- epilogue (warps 2-9, two per SM sub-partition).  TMEM holds
+    // ---------------- epilogue (warps 2-17, four per SM sub-partition).  TMEM holds
     // the super-tile transposed (lane = column, TMEM column = row): warp w reads
     // TMEM lanes 32 (w % 4)..+31 = tile column J0 + w % 4, lane = column inside
-    // the tile; warps 2-5 take row tiles 0-1, warps 6-9 row tiles 2-3.  So the
+    // the tile; four warps share each tile column, one per row tile.  So the
     // 32 lanes of a warp hold 32 consecutive elements of a row of the row-major
     // tiles, and every access to the scratch, to X~ and to X_new is one
     // contiguous 256-byte piece.  With lane = row each 16-byte access touched 32
@@ -1060,8 +1155,15 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_square_tc(TcArgs a) {
     // the TMEM blocks, so the next tile's products run during phase 2, the FP64
     // arithmetic.  A thread reads back only what it wrote, so one scratch slot
     // per CTA serves all tiles.
+    // Sixteen warps, one tile each, keep the FP64 pipe busier than eight with two
+    // tiles each (phase 2 of a super-tile 63,000 -> 51,000 cycles at N = 24,000;
+    // 1.7 to 2 FP64 lane operations per SM cycle are its floor).  The loops are
+    // rolled over row chunks and groups, which keeps the code short (the
+    // sub-partition's instruction cache is shared with the issuers) and the
+    // registers below the 102 that 640 threads leave.
+    constexpr int CH = 8;       // rows of a tile in one chunk of phase 2
     const int quarter = warp & 3;
-    const int bt0 = 2 * ((warp - 2) >> 2);
+    const int bt = (warp - 2) >> 2;
     // unit of the finest group of the window: with W bits per slice, slice s
     // lies on the grid 2^-(W s + W - 1), so group g = s + t has the unit
     // 2^-(W g + 2 W - 2)
@@ -1104,26 +1206,21 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_square_tc(TcArgs a) {
       const int64_t gj = (int64_t)Jb * TB + lane;
       // scratch element of super-tile row i: scr[i * ST]
       long long* scr = a.scratch + (int64_t)blockIdx.x * (ST * ST) + quarter * 32 + lane;
-      // output tile index of each row tile
-      int oidx[2];
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int Ia = I0 + bt0 + h;
-        oidx[h] = (Ia < a.nb && Jb < a.nb && (a.general || Ia <= Jb)) ? find(a.obits, a.orowptr, Ia, Jb) : -1;
-      }
-      // Z_IJ of each output tile (X~_IJ in the forward step; absent -> null),
-      // looked up and its row requested into L2 before the accumulators are
+      const int Ia = I0 + bt;                // tile row of this warp
+      // output tile index
+      const int oi = (Ia < a.nb && Jb < a.nb && (a.general || Ia <= Jb)) ? find(a.obits, a.orowptr, Ia, Jb) : -1;
+      // Z_IJ of the output tile (X~_IJ in the forward step; absent -> null),
+      // looked up and its rows requested into L2 before the accumulators are
       // waited for, so that the chain of dependent loads overlaps the wait
-      const double* Zt[2] = {nullptr, nullptr};
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        if (oidx[h] < 0 || emode == 1) continue;
-        const int zp = find(a.zbits, a.zrowptr, I0 + bt0 + h, Jb);
-        if (zp < 0) continue;
-        const int64_t zi = (int64_t)(a.zref[zp] & ~REF_T);
-        Zt[h] = a.zpool + (int64_t)(a.zslot ? a.zslot[zi] : zi) * TE;
-        prefetch_l2(Zt[h] + lane * TB);
-        prefetch_l2(Zt[h] + lane * TB + 16);
+      const double* Z = nullptr;
+      if (oi >= 0 && emode != 1) {
+        const int zp = find(a.zbits, a.zrowptr, Ia, Jb);
+        if (zp >= 0) {
+          const int64_t zi = (int64_t)(a.zref[zp] & ~REF_T);
+          Z = a.zpool + (int64_t)(a.zslot ? a.zslot[zi] : zi) * TE;
+          prefetch_l2(Z + lane * TB);
+          prefetch_l2(Z + lane * TB + 16);
+        }
       }
       // phase 1, once per accumulation segment: TMEM -> the exact fixed-point
       // sums of this thread's column in the scratch (the first segment stores, the
@@ -1141,30 +1238,31 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_square_tc(TcArgs a) {
         tc_fence_after();
         const uint32_t gm = gmap[q];
         const uint32_t written = gm & 0xFu;
+#pragma unroll 1
+        for (int hc = 0; hc < 2 && oi >= 0; ++hc) {       // 16 rows at a time
+          const int row0 = bt * 32 + hc * 16;
+          long long fx[16];
+          long long* sp = scr + row0 * ST;
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const int bt = bt0 + h;
-          if (oidx[h] < 0) continue;      // warp-uniform
+          for (int i = 0; i < 16; ++i) fx[i] = 0;
+          const uint32_t trow = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)row0;
+#pragma unroll 1
+          for (int gg = 0; gg <= ghi - glo; ++gg) {   // relative groups of the window, coarsest first
 #pragma unroll
-          for (int ch = 0; ch < 2; ++ch) {
-            const int row0 = bt * 32 + ch * 16;
-            long long fx[16];
-            long long* sp = scr + row0 * ST;
+            for (int i = 0; i < 16; ++i) fx[i] *= 1ll << W;
+            if ((written >> gg) & 1u) {        // warp-uniform: groups no product reached are zero
+              float g[16];
+              tmem_ld16(trow + ((gm >> (8 + 2 * gg)) & 3u) * ST, g);
 #pragma unroll
-            for (int i = 0; i < 16; ++i) fx[i] = first ? 0 : ld_staging(sp + i * ST, pol);
-#pragma unroll
-            for (int gg = 0; gg < 4; ++gg) {   // relative groups of the window
-              if (gg <= ghi - glo && ((written >> gg) & 1u)) {   // warp-uniform: groups no product reached are zero
-                float g[16];
-                const uint32_t blk = (gm >> (8 + 2 * gg)) & 3u;
-                tmem_ld16(tmem + ((uint32_t)(quarter * 32) << 16) + blk * ST + (uint32_t)row0, g);
-#pragma unroll
-                for (int i = 0; i < 16; ++i) fx[i] += f32_int_to_ll(g[i]) * (1ll << (W * (ghi - glo - gg)));
-              }
+              for (int i = 0; i < 16; ++i) fx[i] += f32_int_to_ll(g[i]);
             }
-#pragma unroll
-            for (int i = 0; i < 16; ++i) st_staging(sp + i * ST, fx[i], pol);
           }
+          if (!first) {
+#pragma unroll
+            for (int i = 0; i < 16; ++i) fx[i] += ld_staging(sp + i * ST, pol);
+          }
+#pragma unroll
+          for (int i = 0; i < 16; ++i) st_staging(sp + i * ST, fx[i], pol);
         }
         // this warp's TMEM reads of the segment are complete
         tc_fence_before();
@@ -1175,33 +1273,28 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_square_tc(TcArgs a) {
       }
       if (!good) { if (lane == 0) status[0] = 1; break; }
       // phase 2: X_new, per-tile ||X~ - S||^2, ||X_new||^2 and traces
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int bt = bt0 + h;
-        const int Ia = I0 + bt;
-        const int oi = oidx[h];
-        if (oi < 0) continue;
-        const double* Z = Zt[h];
+      if (oi >= 0) {
         double trS = 0.0, trX = 0.0, n2 = 0.0, e2 = 0.0;
         double* O = a.opool + (int64_t)oi * TE;
-        for (int ch = 0; ch < 2; ++ch) {     // 16 rows per chunk
-          const int64_t gi0 = (int64_t)Ia * TB + ch * 16;
-          const long long* sp = scr + (bt * 32 + ch * 16) * ST;
-          const int e0 = ch * 16 * TB + lane;     // element of the chunk's first row in a tile
-          double zv[16];
+#pragma unroll 1
+        for (int ch = 0; ch < TB / CH; ++ch) {     // CH rows per chunk
+          const int64_t gi0 = (int64_t)Ia * TB + ch * CH;
+          const long long* sp = scr + (bt * 32 + ch * CH) * ST;
+          const int e0 = ch * CH * TB + lane;     // element of the chunk's first row in a tile
+          double zv[CH];
 #pragma unroll
-          for (int i = 0; i < 16; ++i) zv[i] = Z ? Z[e0 + i * TB] : 0.0;
-          long long fx[16];
+          for (int i = 0; i < CH; ++i) zv[i] = Z ? Z[e0 + i * TB] : 0.0;
+          long long fx[CH];
 #pragma unroll
-          for (int i = 0; i < 16; ++i) fx[i] = ld_staging(sp + i * ST, pol);
+          for (int i = 0; i < CH; ++i) fx[i] = ld_staging(sp + i * ST, pol);
           // emode 2: the finer groups' S, left in the output tile by the launch before
-          double prev[16];
+          double prev[CH];
 #pragma unroll
-          for (int i = 0; i < 16; ++i) prev[i] = emode == 2 ? O[e0 + i * TB] : 0.0;
-          double out[16];
-          if (Z || form == 0) {
+          for (int i = 0; i < CH; ++i) prev[i] = emode == 2 ? O[e0 + i * TB] : 0.0;
+          double out[CH];
+          if (Z) {
 #pragma unroll
-            for (int i = 0; i < 16; ++i) {
+            for (int i = 0; i < CH; ++i) {
               const int64_t gi = gi0 + i;
               const bool inside = gi < a.n && gj < a.n;
               const double fxd = inside ? (double)fx[i] : 0.0;
@@ -1225,11 +1318,11 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_square_tc(TcArgs a) {
               if (dg) { trS += S; trX += z; }
             }
           } else {
-            // no X~ tile here (z = 0) and X_new = S or 2 z - S = -S: every
-            // (z - S)^2 equals xn^2, so one FMA per element gives both sums
+            // no X~ tile here: z = 0.  X_new = S or 2 z - S = -S (forms 1 and 2):
+            // every (z - S)^2 equals xn^2, so one FMA per element gives both sums
             // (e2 is set from n2 below; the same values in the same order)
 #pragma unroll
-            for (int i = 0; i < 16; ++i) {
+            for (int i = 0; i < CH; ++i) {
               const int64_t gi = gi0 + i;
               const bool inside = gi < a.n && gj < a.n;
               const double fxd = inside ? (double)fx[i] : 0.0;
@@ -1237,16 +1330,21 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_square_tc(TcArgs a) {
               const double S0 = int_times_pow2(fxd, lsu);
               if (emode == 1) { out[i] = S0; continue; }
               const double S = (dg && a.dsq) ? a.dsq[gi] : (emode == 2 ? S0 + prev[i] : S0);
-              const double xn = form == 1 ? S : negated(S);
+              double xn;
+              if (form == 0) {
+                xn = fma(a.c2, S, dg ? a.c0 : 0.0);
+                e2 = fma(S, S, e2);
+              } else {
+                xn = form == 1 ? S : negated(S);
+              }
               out[i] = xn;
               n2 = fma(xn, xn, n2);
               if (dg) trS += S;
             }
           }
 #pragma unroll
-          for (int i = 0; i < 16; ++i) O[e0 + i * TB] = out[i];
+          for (int i = 0; i < CH; ++i) O[e0 + i * TB] = out[i];
         }
-        if (emode == 1) continue;
         if (!Z && form != 0) e2 = n2;
         // warp reductions (the tile's 32 columns are this warp's 32 lanes)
         for (int o = 16; o > 0; o >>= 1) {
@@ -1255,7 +1353,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_square_tc(TcArgs a) {
           trS += __shfl_xor_sync(FULLW, trS, o);
           trX += __shfl_xor_sync(FULLW, trX, o);
         }
-        if (lane == 0) {
+        if (lane == 0 && emode != 1) {
           const bool diag = Ia == Jb;
           a.part.e2[oi] = (diag || a.general ? 1.0 : 2.0) * e2;
           a.part.n2[oi] = n2;
@@ -1423,7 +1521,6 @@ cudaError_t launch_square_tc(const TcLaunch& L, cudaStream_t st) {
   a.wait_ns = L.wait_ns;
   a.selftest = L.selftest ? 1 : 0;
   a.general = L.general ? 1 : 0;
-  a.split_supply = L.split_supply ? 1 : 0;
   a.dsq = L.dsq;
   a.glo = L.glo;
   a.ghi = L.ghi < 0 ? L.k - 1 : L.ghi;
