@@ -39,11 +39,11 @@
 //     headers fetched one batch ahead), lists sub-steps of at most two A
 //     slices x two B slices.
 //   warps 18 and 19: issuers -- copy the A and the B units of every sub-step
-//     into shared-memory rings (cp.async.bulk of 8 or 16 KB, completion tracked
-//     by an mbarrier transaction count).
+//     into the stages (cp.async.bulk of 8 or 16 KB, completion tracked by an
+//     mbarrier transaction count).
 //   warp 1: issues tcgen05.mma kind::f16 (M = 128, N = 128, K = 16) for every
 //     slice pair of the record into the TMEM accumulator of its group, then
-//     tcgen05.commit frees the units.
+//     tcgen05.commit frees the stage.
 //   warps 2-17: epilogue -- tcgen05.ld of the accumulators that were written,
 //     exact fixed-point combination, X_new = c0 I + c1 X~ + c2 S in FP64,
 //     per-tile ||X~ - S||^2, traces and ||X_new||^2, FP64 stores of the
@@ -87,6 +87,19 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
   asm volatile(
       "{\n\t.reg .pred p;\n\t"
       "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(smem_u32(bar)), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
+
+// whether the phase has completed, without waiting
+__device__ __forceinline__ bool mbar_test(uint64_t* bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
       "selp.u32 %0, 1, 0, p;\n\t}"
       : "=r"(ok)
       : "r"(smem_u32(bar)), "r"(parity)
@@ -196,6 +209,17 @@ __device__ __forceinline__ double negated(double x) {
 __device__ __forceinline__ double int_times_pow2(double x, int k) {
   const int hi = __double2hiint(x);
   return (hi & 0x7FFFFFFF) == 0 ? x : __hiloint2double(hi + (k << 20), __double2loint(x));
+}
+
+// v * 2^k for |v| < 2^53 (exact; a normal result) with no FP64 instruction: the
+// leading bit is shifted to bit 52 and the exponent added.
+__device__ __forceinline__ double small_ll_times_pow2(long long v, int k) {
+  const unsigned long long m = (unsigned long long)(v < 0 ? -v : v);
+  const int c = __clzll((long long)m);                       // >= 11; 64 for zero
+  const unsigned long long f = m << ((c - 11) & 63);         // bit 52 set
+  const int hi = (int)(f >> 32) + ((1085 - c + k) << 20);    // 1085: bit 52 adds one
+  const int sgn = (int)((unsigned long long)v >> 32) & (int)0x80000000;
+  return m == 0ull ? 0.0 : __hiloint2double(hi | sgn, (int)(uint32_t)f);
 }
 
 __device__ __forceinline__ void prefetch_l2(const void* p) {
@@ -546,18 +570,20 @@ struct TcArgs {
                             // 2: full epilogue on S + the S already in the output tiles
 };
 
-// Shared memory holds two rings of RING operand units, one for each side of the
-// product, a unit being one slice of a 4-tile panel (128 rows x 32, 8 KB, 8-row
-// groups 512 B apart).  A sub-step takes the next one or two units of each ring:
+// A pipeline stage holds one sub-step: two A units and two B units, a unit being
+// one slice of a 4-tile panel (128 rows x 32, 8 KB, 8-row groups 512 B apart):
 // up to two adjacent slices of the A record and up to two of the B record, each
-// side one bulk copy of 8 or 16 KB (two where the ring wraps).  A sub-step
-// record (32 bits; the MMA issuer sees the lower 16) tells the issuers what to
-// copy and the MMA issuer what to multiply:
+// side one bulk copy of 8 or 16 KB, or one unit of each of two K steps that have
+// one product each.  A sub-step record (32 bits) tells the issuers what to copy
+// and the MMA issuer what to multiply:
 //   bits 0-2: 1 + the group (s + t - glo) of the first A x first B slice,
+//   bit 3: a pair, two K steps of one product each (their slices add up to the
+//   last group): products A0 x B0 and A1 x B1, both in that group,
 //   bits 4-7: product mask, bit (2 i + j) for A slice a0 + i x B slice b0 + j,
 //   bits 8-11: groups its products write,
 //   bit 12: end of the super-tile, bit 13: no more super-tiles, bit 14: end of an
-//   accumulation segment (no data),
+//   accumulation segment (these three have no data and no stage), bit 15: second
+//   pass (A = Q, B = P), bits 16-19: groups that this segment writes first here,
 //   bits 20-21, 22-24: A slices to copy and the first of them, bits 25-26, 27-29:
 //   the same for B.  A super-tile whose K loop has at least
 //   seg_min K steps closes a segment after every 16 K steps: the epilogue adds
@@ -565,32 +591,41 @@ struct TcArgs {
 //   so no FP32 accumulator sums more than 16 K steps (512 products per
 //   element) and the groups stay exact for dense operands.
 //
-// What bounds the kernel is how fast its single-thread loops run, not the copy
-// path (a lone thread that issues 16 KB bulk copies fills 72 B per SM cycle out
-// of L2; a K step needs 27 KB and has 210 cycles of MMAs) and not the tensor
-// pipe (25%).  So the producer side is three warps: the planner finds the K
-// steps of a tile, reads their record headers and writes batches of sub-steps
-// (at most 32 K steps each) into NPLAN buffers; two issuers copy the units, one
-// the A side, one the B side.  The loops of the issuers and of the MMA issuer
-// are run by whole warps on warp-uniform values, with one elected lane acting:
-// tcgen05.mma and cp.async.bulk take their operands from uniform registers, and
-// in code that only one lane enters each operand is moved there at every use
-// (240 cycles a product and 130 a copy; 110 and about 60 with uniform loops).
-// Cycles per super-tile, water-like N = 24,000 and 96,000: one producer warp
-// 126,000 and 96,000; planner and one issuer 120,000 and 81,000 (with the
-// shorter epilogue loops); two issuers, uniform loops and 16 epilogue warps
-// 103,000 and 67,000.  Whole runs 172 -> 145 ms and 1,250 -> 855 ms.
+// What bounds the kernel is how fast its serial loops run (a warp by itself takes
+// 5 to 8 cycles an instruction, and the loop of a sub-step costs the MMA issuer
+// about 250 cycles a product where the tensor pipe takes 128), not the copy path
+// (a lone thread that issues 16 KB bulk copies fills 72 B per SM cycle out of L2;
+// a K step needs 27 KB and has 210 cycles of MMAs), not shared memory (32 B per
+// cycle of copies landing leave 128-wide MMAs at 66 cycles each) and not the
+// tensor pipe (33%).  So all that can be done for 32 K steps side by side is done
+// by the planner: it finds the K steps of a tile, reads their record headers and
+// writes batches of finished sub-step records (at most 32 K steps each) into
+// NPLAN buffers.  Two issuers copy the units, one the A side, one the B side, and
+// the MMA issuer reads the same records; each of the three is one elected thread
+// (elect.sync: in code that a comparison of the lane number guards, the operands
+// of tcgen05.mma and cp.async.bulk cost twice as long to set up), with the next
+// record loaded and the next stage's barrier tested ahead.
+// Cycles per super-tile, water-like N = 24,000 and 96,000, dense N = 4,096 with
+// five slices (both launches): one producer warp 126,000, 96,000, 508,000;
+// planner and one issuer 120,000, 81,000, 507,000; two issuers and 16 epilogue
+// warps 103,000, 67,000, 455,000; pairs of one-product K steps, finished records,
+// integer conversions in the epilogue 84,000, 58,000, 398,000.  Two MMA issuers
+// taking turns (one warp more, 80 registers instead of 96): 91,000, 64,000.  Two
+// sub-steps for each barrier: 87,000, 59,000.
 constexpr int UNIT_BYTES = 4 * SLICE_BYTES;
-constexpr int RING = 12;                           // units of one side's ring (96 KB; 192 KB in all)
-constexpr int STEPS = 16;                          // sub-steps in flight
+constexpr int STAGE_BYTES = 4 * UNIT_BYTES;
+constexpr int STAGES = 6;                          // sub-steps in flight
 constexpr int NPLAN = 4;                           // batches between the planner and the issuer
-constexpr int PLAN = 104;                          // entries of a batch: 32 K steps x 3 + segment ends
+constexpr int PLAN = 104;                          // entries of a batch: 32 K steps x 3 + segment ends (+ 1 read ahead)
 constexpr uint32_t REC_END = 1u << 12;
 constexpr int EPI_WARPS = 16;                      // epilogue warps 2..17
 constexpr int ISSUE_WARP = 2 + EPI_WARPS;          // issuer warps 18 (A units) and 19 (B units)
 constexpr int TC_THREADS = 32 * (2 + EPI_WARPS + 2);   // + planner warp 0, MMA warp 1
 constexpr uint32_t REC_LAST = 1u << 13;   // no more super-tiles (no data)
 constexpr uint32_t REC_SEG = 1u << 14;    // end of an accumulation segment of the super-tile (no data)
+constexpr uint32_t REC_PAIR = 1u << 3;
+constexpr uint32_t REC_PASS1 = 1u << 15;
+constexpr uint32_t REC_FRESH = 15u << 16;
 constexpr uint32_t REC_CTL = REC_END | REC_LAST | REC_SEG;
 constexpr uint32_t SEG_LAST = 1u << 31;   // segment record flag: last segment of its super-tile
 constexpr int SEG_RING = 4;               // accumulation segments in flight between MMA and epilogue
@@ -602,7 +637,7 @@ constexpr uint32_t HEAD_NONE = 0x07u;   // header of a K index outside the step 
 
 template <int K>
 struct TcCfg {
-  static constexpr int SMEM = 2 * RING * UNIT_BYTES + 2048 + NPLAN * PLAN * 16;
+  static constexpr int SMEM = STAGES * STAGE_BYTES + 2048 + NPLAN * PLAN * 16;
 };
 
 template <int K>
@@ -613,36 +648,35 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_square_tc(TcArgs a) {
   // slices take every group in one launch (compile-time constants)
   const int glo = K == 5 ? a.glo : 0, ghi = K == 5 ? a.ghi : K - 1, emode = K == 5 ? a.emode : 0;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
-  unsigned char* ring = smem_raw;
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem_raw + 2 * RING * UNIT_BYTES);   // [STEPS] the sub-step's units are in
-  uint64_t* empty = full + STEPS;          // [STEPS] its products are done
-  uint64_t* acc_full = empty + STEPS;      // [SEG_RING] MMAs of a segment done (commit) + its record written
+  unsigned char* stages = smem_raw;
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem_raw + STAGES * STAGE_BYTES);   // [STAGES] the sub-step's units are in
+  uint64_t* empty = full + STAGES;         // [STAGES] its products are done
+  uint64_t* acc_full = empty + STAGES;     // [SEG_RING] MMAs of a segment done (commit) + its record written
   uint64_t* tile_full = acc_full + SEG_RING;   // [NSLOT] tile slot written by the planner
   uint64_t* tile_empty = tile_full + NSLOT;    // [NSLOT] epilogue done with the tile slot (one arrive per warp)
   uint64_t* drain = tile_empty + NSLOT;    // MMAs issued before the exit are complete
   uint64_t* tmem_empty = drain + 1;        // [SEG_RING] every epilogue warp has read the segment's TMEM
   uint64_t* probe = tmem_empty + SEG_RING; // self-test: a barrier that nothing arrives at
   uint64_t* plan_full = probe + 1;         // [NPLAN] batch written by the planner
-  uint64_t* plan_empty = plan_full + NPLAN;    // [NPLAN] batch taken by the issuer
-  uint32_t* rec = reinterpret_cast<uint32_t*>(plan_empty + NPLAN);   // [STEPS] bits 0-15 of the sub-step's record, ring places of A0, A1, B0, B1
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(rec + STEPS);
+  uint64_t* plan_empty = plan_full + NPLAN;    // [NPLAN] batch read by the two issuers and the MMA issuer
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(plan_empty + NPLAN);
   int32_t* tslot = reinterpret_cast<int32_t*>(tmem_slot + 2);      // [NSLOT] super-tile list index, -1: none
   int32_t* kcount = tslot + NSLOT;                                  // [NSLOT][16] triplets per output tile
   uint32_t* gmap = reinterpret_cast<uint32_t*>(kcount + 16 * NSLOT);   // [SEG_RING] groups written, block of each, last flag
   int32_t* bcnt = reinterpret_cast<int32_t*>(gmap + SEG_RING);     // [NPLAN] entries of a batch
   int32_t* status = bcnt + NPLAN;                                   // [0] a wait timed out
-  uint4* steps = reinterpret_cast<uint4*>(smem_raw + 2 * RING * UNIT_BYTES + 1024);   // [8][8] sub-steps of (first A, first B slice)
-  uint4* plan = steps + 64;                                         // [NPLAN][PLAN] record, A unit, B unit, pass
+  uint4* steps = reinterpret_cast<uint4*>(smem_raw + STAGES * STAGE_BYTES + 1024);   // [8][8] sub-steps of (first A, first B slice)
+  uint4* plan = steps + 64;                                         // [NPLAN][PLAN] record, A unit, B unit, pair: steps to the second units
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
-    for (int s = 0; s < STEPS; ++s) {
+    for (int s = 0; s < STAGES; ++s) {
       mbar_init(&full[s], 2);     // each issuer's arrival, with its bulk bytes
       mbar_init(&empty[s], 1);
     }
     for (int b = 0; b < NPLAN; ++b) {
       mbar_init(&plan_full[b], 1);
-      mbar_init(&plan_empty[b], 2);   // both issuers
+      mbar_init(&plan_empty[b], 3);
     }
     for (int b = 0; b < SEG_RING; ++b) {
       mbar_init(&acc_full[b], 2);
@@ -666,7 +700,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_square_tc(TcArgs a) {
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = *tmem_slot;
+  const uint32_t tmem = __shfl_sync(FULLW, *tmem_slot, 0);
   const int total = *a.count;
 
   // Persistent and warp-specialised: the planner (warp 0) takes super-tiles from
@@ -713,7 +747,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_square_tc(TcArgs a) {
     }
     __syncwarp();
     bool ok = true;
-    int nbat = 0;      // batches handed to the issuer
+    int nbat = 0;      // batches handed to the issuers and the MMA issuer
+    unsigned long long nprod = 0;   // slice-pair products planned by this lane
     // all lanes: wait for the next batch buffer; false on timeout
     auto batch_open = [&]() -> bool {
       int good = 1;
@@ -794,6 +829,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_square_tc(TcArgs a) {
       }
       const bool segmented = a.seg_min > 0 && ktot >= a.seg_min;
       int kdone = 0;
+      uint32_t wmask = 0u;      // groups that the open segment has written
       // triplet counts: K steps with A tile q and B tile y both present, byte y of
       // acc[q] in every lane, moved to kc (lane 4 q + y) before a byte overflows
       int kc = 0, nacc = 0;
@@ -882,11 +918,51 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_square_tc(TcArgs a) {
 #pragma unroll
             for (int q = 0; q < 4; ++q) acc[q] += ((pa4 >> q) & 1u) ? eb4 : 0u;
             if (++nacc == 255) flush_counts();
-            const uint4 sv = steps[(ha & 7u) * 8u + (hb & 7u)];   // HEAD_NONE: no sub-steps
-            const int ns = (int)sv.w;
+            const uint4 sv = steps[(ha & 7u) * 8u + (hb & 7u)];   // HEAD_NONE: no sub-steps (and no products)
+            nprod += (unsigned)(__popc((sv.x >> 4) & 15u) + __popc((sv.y >> 4) & 15u) + __popc((sv.z >> 4) & 15u));
+            int ns = (int)sv.w;
             // a segmented tile also closes a segment before every seg_ksteps-th K
             // step inside the batch (the batch end closes one too)
             const int lead = (segmented && lane > 0 && (lane % a.seg_ksteps) == 0 && jb + lane < total) ? 1 : 0;
+            const uint32_t ua = (uint32_t)ea * K + ((sv.x >> 22) & 7u), ub = (uint32_t)eb * K + ((sv.x >> 27) & 7u);
+            // K steps of one product each are taken in pairs, in order: lane l of
+            // an even number of single steps since the last other step (or segment
+            // end) takes the next single step with it
+            uint32_t rv0 = sv.x, second = 0u;
+            const bool single = ns == 1 && ((sv.x >> 4) & 0xFu) == 1u;
+            const uint32_t sm = __ballot_sync(FULLW, single), mm = __ballot_sync(FULLW, ns > 0 && !single);
+            const uint32_t lt = (1u << lane) - 1u;
+            int run0 = 32 - __clz(mm & lt);                     // first lane of the run
+            if (segmented) run0 = max(run0, lane - lane % a.seg_ksteps);
+            const int rank = __popc(sm & lt & ~((1u << run0) - 1u));
+            const uint32_t later = sm & ~lt & ~(1u << lane);
+            const int nxt = later ? __ffs(later) - 1 : lane;
+            const uint32_t ua2 = __shfl_sync(FULLW, ua, nxt), ub2 = __shfl_sync(FULLW, ub, nxt);
+            const bool fits = nxt > lane && (mm & ~lt & ((1u << nxt) - 1u)) == 0u &&
+                              (!segmented || nxt / a.seg_ksteps == lane / a.seg_ksteps);
+            if (single) {
+              if (rank & 1) {
+                ns = 0;      // taken by the step before
+              } else if (fits) {
+                rv0 = (rv0 & ~((3u << 20) | (3u << 25))) | REC_PAIR | (1u << 7) | (2u << 20) | (2u << 25);
+                second = (ua2 - ua) | ((ub2 - ub) << 16);
+              }
+            }
+            // groups that a sub-step writes first in its segment (seg0: the lane where
+            // the segment begins)
+            const uint32_t need0 = ns > 0 ? (sv.x >> 8) & 15u : 0u, need1 = ns > 1 ? (sv.y >> 8) & 15u : 0u;
+            const uint32_t need2 = ns > 2 ? (sv.z >> 8) & 15u : 0u;
+            const int seg0 = segmented ? lane - lane % a.seg_ksteps : 0;
+            uint32_t before = seg0 == 0 ? wmask : 0u, all = 0u;
+#pragma unroll
+            for (int g = 0; g < 4; ++g) {
+              const uint32_t bal = __ballot_sync(FULLW, ((need0 | need1 | need2) >> g) & 1u);
+              if (bal & lt & ~((1u << seg0) - 1u)) before |= 1u << g;
+              if (bal) all |= 1u << g;
+            }
+            wmask = segmented ? 0u : wmask | all;      // a segmented tile's batch ends its segment
+            const uint32_t fr0 = (need0 & ~before) << 16, fr1 = (need1 & ~(before | need0)) << 16;
+            const uint32_t fr2 = (need2 & ~(before | need0 | need1)) << 16;
             int soff = ns + lead;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
@@ -898,14 +974,14 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_square_tc(TcArgs a) {
             ok = batch_open();
             if (!ok) break;
             uint4* ul = plan + (nbat % NPLAN) * PLAN;
-            const uint32_t ua = (uint32_t)ea * K, ub = (uint32_t)eb * K;
+            const uint32_t pbit = pass ? REC_PASS1 : 0u;
             auto entry = [&](uint32_t rv) {
-              return make_uint4(rv, ua + ((rv >> 22) & 7u), ub + ((rv >> 27) & 7u), (uint32_t)pass);
+              return make_uint4(rv | pbit, (uint32_t)ea * K + ((rv >> 22) & 7u), (uint32_t)eb * K + ((rv >> 27) & 7u), 0u);
             };
             if (lead) ul[soff - 1] = make_uint4(REC_SEG, 0u, 0u, 0u);
-            if (ns > 0) ul[soff] = entry(sv.x);
-            if (ns > 1) ul[soff + 1] = entry(sv.y);
-            if (ns > 2) ul[soff + 2] = entry(sv.z);
+            if (ns > 0) ul[soff] = make_uint4(rv0 | pbit | fr0, ua, ub, second);
+            if (ns > 1) ul[soff + 1] = entry(sv.y | fr1);
+            if (ns > 2) ul[soff + 2] = entry(sv.z | fr2);
             kdone += min(32, total - jb);
             if (segmented && kdone < ktot) {
               if (lane == 0) ul[nsub] = make_uint4(REC_SEG, 0u, 0u, 0u);
@@ -926,93 +1002,70 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_square_tc(TcArgs a) {
       __syncwarp();
       if (ok) ok = batch_ctl(REC_END);
     }
+    // slice-pair products (each 2 MMAs of 128 x 128 x 16)
+    if (a.err && nprod) atomicAdd(reinterpret_cast<unsigned long long*>(a.err + 2), nprod);
   } else if (warp >= ISSUE_WARP) {
-    // ---------------- issuers: one thread copies the A units of every planned
-    // sub-step into A's ring, the other the B units into B's, in order, once
-    // the sub-steps before it have left enough units free.
-    // As in the MMA issuer the whole warp runs the loop and an elected lane acts.
-    const bool leader = elect_one();
-    const int lead = __ffs(__ballot_sync(FULLW, leader)) - 1;
-    const int side = __shfl_sync(FULLW, warp, 0) - ISSUE_WARP;      // 0: A, 1: B
-    const uint32_t first_used = side ? 0x50u : 0x30u;       // products that read the side's first slice
-    const uint32_t mine = smem_u32(ring) + (uint32_t)side * (RING * UNIT_BYTES);
-    int s = 0, q = 0;              // next sub-step slot to issue, next to be released
-    uint32_t qpar = 0;             // phase of slot q
-    int busy = 0;                  // slots issued and not released
-    int pos = 0, nfree = RING;     // next unit of the ring, free units
-    uint32_t held = 0u;            // units of sub-step slot s: bits 2 s, 2 s + 1
-    int head = 0;                  // sub-steps issued
-    bool done = false;
-    for (int bat = 0; !done; ++bat) {
-      if (!__shfl_sync(FULLW, mbar_wait_sleep(&plan_full[bat % NPLAN], (uint32_t)(bat / NPLAN) & 1u) ? 1 : 0, lead)) {
-        if (leader) {
+    // ---------------- issuers: one thread of warp 18 copies the A units of every
+    // planned sub-step into the next stage, one of warp 19 the B units.
+    if (elect_one()) {
+      const int side = warp - ISSUE_WARP;      // 0: A, 1: B
+      const uint32_t first_used = side ? 0x50u : 0x30u;       // products that read the side's first slice
+      const uint32_t mine = smem_u32(stages) + (uint32_t)side * (2 * UNIT_BYTES);
+      int s = 0;                     // next stage
+      uint32_t par = 1u;             // phase that frees it
+      bool isfree = true;            // it was free when last looked at
+      int head = 0;                  // sub-steps issued
+      bool done = false;
+      for (int bat = 0; !done; ++bat) {
+        if (!mbar_wait_sleep(&plan_full[bat % NPLAN], (uint32_t)(bat / NPLAN) & 1u)) {
           status[0] = 1;
           note_timeout(a.err, 8);
+          break;
         }
-        break;
-      }
-      const uint4* ul = plan + (bat % NPLAN) * PLAN;
-      const int n = __shfl_sync(FULLW, bcnt[bat % NPLAN], 0);
-      uint4 nx = ul[0];
-      for (int u = 0; u < n && !done; ++u) {
-        const uint32_t rv = __shfl_sync(FULLW, nx.x, 0);
-        const uint32_t unit = __shfl_sync(FULLW, side ? nx.z : nx.y, 0);
-        const bool swap = __shfl_sync(FULLW, nx.w, 0) != 0u;
-        nx = ul[min(u + 1, n - 1)];
-        const int m = (int)((rv >> (side ? 25 : 20)) & 3u);
-        while (nfree < m || busy == STEPS) {
-          if (!__shfl_sync(FULLW, mbar_wait(&empty[q], qpar) ? 1 : 0, lead)) {
-            if (leader) {
-              status[0] = 1;
-              note_timeout(a.err, 2);
-            }
+        const uint4* ul = plan + (bat % NPLAN) * PLAN;
+        const int n = bcnt[bat % NPLAN];
+        uint4 nx = ul[0];
+        for (int u = 0; u < n; ++u) {
+          const uint4 en = nx;
+          nx = ul[u + 1];
+          const uint32_t rv = en.x;
+          if (rv & REC_CTL) {
+            if (rv & REC_LAST) done = true;
+            continue;
+          }
+          const uint32_t unit = side ? en.z : en.y, second = side ? en.w >> 16 : en.w & 0xFFFFu;
+          const __half* base = ((rv & REC_PASS1) != 0u) == (side != 0) ? a.P.data : a.Q.data;
+          const unsigned char* src = reinterpret_cast<const unsigned char*>(base) + (uint64_t)unit * UNIT_BYTES;
+          const uint32_t bytes = ((rv >> (side ? 25 : 20)) & 3u) * UNIT_BYTES;
+          const uint32_t part = second != 0u ? UNIT_BYTES : bytes;       // a pair: two copies
+          const uint32_t dst = mine + (uint32_t)s * STAGE_BYTES + ((rv & first_used) ? 0u : (uint32_t)UNIT_BYTES);
+          if (!isfree && !mbar_wait(&empty[s], par)) {
+            status[0] = 1;
+            note_timeout(a.err, 2);
             done = true;
             break;
           }
-          nfree += (int)((held >> (2 * q)) & 3u);
-          --busy;
-          if (++q == STEPS) { q = 0; qpar ^= 1u; }
-        }
-        if (done) break;
-        held = (held & ~(3u << (2 * s))) | ((uint32_t)m << (2 * s));
-        nfree -= m;
-        ++busy;
-        // ring places of the side's two slices (an unused first slice takes none)
-        const int p0 = pos;
-        int p1 = pos + ((rv & first_used) ? 1 : 0);
-        if (p1 == RING) p1 = 0;
-        pos += m;
-        if (pos >= RING) pos -= RING;
-        const __half* base = swap == (side != 0) ? a.P.data : a.Q.data;
-        const unsigned char* src = reinterpret_cast<const unsigned char*>(base) + (uint64_t)unit * UNIT_BYTES;
-        const uint32_t bytes = (uint32_t)m * UNIT_BYTES, part = m == 2 && p0 == RING - 1 ? UNIT_BYTES : bytes;
-        if (leader) {
-          uint8_t* rb = reinterpret_cast<uint8_t*>(rec + s);
-          if (side == 0) *reinterpret_cast<uint16_t*>(rb) = (uint16_t)rv;
-          rb[2 + side] = (uint8_t)(p0 | (p1 << 4));
           mbar_expect_tx(&full[s], bytes);
-          if (m > 0) bulk_g2s(mine + p0 * UNIT_BYTES, src, part, &full[s]);
-          if (part != bytes) bulk_g2s(mine, src + UNIT_BYTES, UNIT_BYTES, &full[s]);
+          bulk_g2s(dst, src, part, &full[s]);
+          if (second != 0u) bulk_g2s(dst + UNIT_BYTES, src + (uint64_t)second * UNIT_BYTES, UNIT_BYTES, &full[s]);
+          ++head;
+          if (++s == STAGES) { s = 0; par ^= 1u; }
+          isfree = mbar_test(&empty[s], par);
         }
-        __syncwarp();
-        ++head;
-        if (++s == STEPS) s = 0;
-        if (rv & REC_LAST) done = true;
+        mbar_arrive(&plan_empty[bat % NPLAN]);
       }
-      if (leader) mbar_arrive(&plan_empty[bat % NPLAN]);
-      __syncwarp();
-    }
-    // no bulk copy into this CTA's shared memory may be in flight when the CTA
-    // exits: wait (bounded) for those of the last STEPS sub-steps
-    if (leader)
-      for (int j = max(0, head - STEPS); j < head; ++j)
-        if (!mbar_wait(&full[j % STEPS], (uint32_t)(j / STEPS) & 1u)) {
+      // no bulk copy into this CTA's shared memory may be in flight when the CTA
+      // exits: wait (bounded) for those of the last STAGES sub-steps
+      for (int j = max(0, head - STAGES); j < head; ++j)
+        if (!mbar_wait(&full[j % STAGES], (uint32_t)(j / STAGES) & 1u)) {
           status[0] = 1;
           note_timeout(a.err, 9);
         }
+    }
+    __syncwarp();
   } else if (warp == 1) {
-    // ---------------- MMA issuer: the whole warp runs the loop, so that its values
-    // are warp-uniform; one elected lane issues.  TMEM is four blocks of 128 columns; a group
+    if (elect_one()) {
+    // ---------------- MMA issuer, one thread.  TMEM is four blocks of 128 columns; a group
     // accumulator of a segment (a whole super-tile, or 32 of its K steps) takes
     // a free block on its first product, and the blocks of a segment return to
     // the pool once every epilogue warp has read them (one arrival per warp on
@@ -1022,24 +1075,17 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_square_tc(TcArgs a) {
     uint32_t pend0 = 0u, pend1 = 0u, pend2 = 0u, pend3 = 0u;
     int released = 0;              // segments whose blocks are back in free_mask
     int seg = 0;                   // segments published
-    unsigned long long nprod = 0;
     bool ok = true, done = false;
-    // the shared-memory descriptor of a unit is that of the ring's start plus
+    // the shared-memory descriptor of a unit is that of the first stage plus
     // a constant (the start-address field holds address / 16 in 14 bits; every
     // address here is below 2^18)
-    const uint64_t dring = make_desc(smem_u32(ring), 128, 512);
+    const uint64_t dring = make_desc(smem_u32(stages), 128, 512);
     const uint32_t dlo = (uint32_t)dring & 0xFFFFu;              // start address / 16 (below 2^14 for every unit)
     const uint64_t dhi = dring & ~0xFFFFull;
-    const bool leader = elect_one();
-    const int lead = __ffs(__ballot_sync(FULLW, leader)) - 1;
-    // bounded wait of the whole warp: the leader's result in every lane
-    auto wait = [&](uint64_t* bar, uint32_t parity) -> bool {
-      return __shfl_sync(FULLW, mbar_wait(bar, parity) ? 1 : 0, lead) != 0;
-    };
     // take back the blocks of the oldest segment that still holds some; false on timeout
     auto reclaim = [&]() -> bool {
-      if (!wait(&tmem_empty[released & (SEG_RING - 1)], ((uint32_t)released >> 2) & 1u)) {
-        if (leader) note_timeout(a.err, 4);
+      if (!mbar_wait(&tmem_empty[released & (SEG_RING - 1)], ((uint32_t)released >> 2) & 1u)) {
+        note_timeout(a.err, 4);
         return false;
       }
       tc_fence_after();
@@ -1052,94 +1098,104 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_square_tc(TcArgs a) {
       ++released;
       return true;
     };
-    int s = 0;      // next sub-step slot and its phase
-    uint32_t par = 0;
-    while (ok && !done) {
-      uint32_t written = 0, gblk = 0, used = 0;
-      uint32_t kind = 0;
-      for (;;) {
-        const int cs = s;
-        const uint32_t cpar = par;
-        if (++s == STEPS) { s = 0; par ^= 1u; }
-        if (!wait(&full[cs], cpar)) {
-          ok = false;
-          if (leader) note_timeout(a.err, 3);
-          break;
-        }
-        tc_fence_after();
-        const uint32_t rv = __shfl_sync(FULLW, rec[cs], 0);
+    int s = 0;               // next stage and the phase that fills it
+    uint32_t par = 0u;
+    bool filled = false;     // stage s was full when last looked at
+    uint32_t gblk = 0u, used = 0u, written = 0u;   // open segment: block of each group, blocks, groups
+    for (int bat = 0; ok && !done; ++bat) {
+      if (!mbar_wait_sleep(&plan_full[bat % NPLAN], (uint32_t)(bat / NPLAN) & 1u)) {
+        note_timeout(a.err, 8);
+        ok = false;
+        break;
+      }
+      const uint4* ul = plan + (bat % NPLAN) * PLAN;
+      const int n = bcnt[bat % NPLAN];
+      uint32_t nx = ul[0].x;
+      for (int u = 0; u < n; ++u) {
+        const uint32_t rv = nx;
+        nx = ul[u + 1].x;
         if (rv & REC_CTL) {
-          if (leader) mma_commit(&empty[cs]);
-          kind = rv & REC_CTL;
+          if (rv & REC_LAST) { done = true; break; }
+          // publish the segment in ring slot seg % SEG_RING once the segment that used
+          // the slot before has been read and its blocks reclaimed
+          while (released < seg - (SEG_RING - 1) && ok) ok = reclaim();
+          if (!ok) break;
+          const int q = seg & (SEG_RING - 1);
+          switch (q) {
+            case 0: pend0 = used; break;
+            case 1: pend1 = used; break;
+            case 2: pend2 = used; break;
+            default: pend3 = used; break;
+          }
+          gmap[q] = written | (gblk << 8) | ((rv & REC_END) ? SEG_LAST : 0u);
+          mma_commit(&acc_full[q]);    // arrives once every MMA of the segment has completed
+          mbar_arrive(&acc_full[q]);   // release: segment record visible to the epilogue
+          ++seg;
+          gblk = used = written = 0u;
+          continue;
+        }
+        const uint32_t units = dlo + (uint32_t)s * (STAGE_BYTES >> 4);    // A0, A1, B0, B1 one unit apart
+        const int cs = s;
+        if (!filled && !mbar_wait(&full[cs], par)) {
+          ok = false;
+          note_timeout(a.err, 3);
           break;
         }
-        // groups (relative to the launch's window, at most four live) that this
-        // segment has not written yet: take a TMEM block; their first MMA overwrites it
-        uint32_t fresh = (rv >> 8) & ~written & 0xFu;
-        for (uint32_t f = fresh; f != 0u; f &= f - 1u) {
-          const int g = __ffs(f) - 1;
-          while (free_mask == 0u && ok) ok = reclaim();
-          if (!ok) break;
-          const uint32_t blk = (uint32_t)(__ffs(free_mask) - 1);
-          free_mask &= ~(1u << blk);
-          used |= 1u << blk;
-          gblk |= blk << (2 * g);
-          written |= 1u << g;
-        }
-        if (!ok) break;
+        if (++s == STAGES) { s = 0; par ^= 1u; }
+        // look at the next stage now: the answer is there when the products of
+        // this one have been issued
+        filled = mbar_test(&full[s], par);
+        // groups (relative to the launch's window, at most four live) that the
+        // segment writes first here take a TMEM block, and their first MMA overwrites it
         const int base = (int)(rv & 7u) - 1;     // group of A0 x B0
-        const uint32_t a0 = dlo + ((rv >> 16) & 15u) * (UNIT_BYTES >> 4), a1 = dlo + ((rv >> 20) & 15u) * (UNIT_BYTES >> 4);
-        const uint32_t b0 = dlo + (((rv >> 24) & 15u) + RING) * (UNIT_BYTES >> 4);
-        const uint32_t b1 = dlo + ((rv >> 28) + RING) * (UNIT_BYTES >> 4);
+        uint32_t fr = 0u;
+        if (rv & REC_FRESH) {
+          for (uint32_t f = (rv >> 16) & 15u; f != 0u; f &= f - 1u) {
+            const int g = __ffs(f) - 1;
+            while (free_mask == 0u && ok) ok = reclaim();
+            if (!ok) break;
+            const uint32_t blk = (uint32_t)(__ffs(free_mask) - 1);
+            free_mask &= ~(1u << blk);
+            used |= 1u << blk;
+            gblk |= blk << (2 * g);
+            written |= 1u << g;
+          }
+          if (!ok) break;
+          fr = (rv >> 16) & 15u;
+          fr = base >= 0 ? fr >> base : fr << 1;
+        }
         const uint32_t gb = base >= 0 ? gblk >> (2 * base) : gblk << 2;    // blocks of groups base, base + 1, base + 2
-        uint32_t fr = base >= 0 ? fresh >> base : fresh << 1;
-        if (leader) {
+        {
           // the unit of the super-column as the M operand, that of the super-row
           // as the N operand: TMEM holds the transposed super-tile
-          auto product = [&](uint32_t ua, uint32_t ub, int k) {
+          auto product = [&](int i, int j, int k, uint32_t acc) {
             const uint32_t dcol = tmem + ((gb >> (2 * k)) & 3u) * ST;
-            mma_f16(dcol, dhi | ub, dhi | ua, ((fr >> k) & 1u) ^ 1u);
+            const uint32_t ua = units + (uint32_t)(i * (UNIT_BYTES >> 4)), ub = units + (uint32_t)((2 + j) * (UNIT_BYTES >> 4));
+            mma_f16(dcol, dhi | ub, dhi | ua, acc);
             mma_f16(dcol, dhi | (ub + 16u), dhi | (ua + 16u), 1u);
           };
-          if (rv & (1u << 4)) { product(a0, b0, 0); }
-          if (rv & (1u << 5)) { product(a0, b1, 1); fr &= ~2u; }
-          if (rv & (1u << 6)) { product(a1, b0, 1); }
-          if (rv & (1u << 7)) { product(a1, b1, 2); }
+          if (rv & REC_PAIR) {
+            product(0, 0, 0, (fr & 1u) ^ 1u);
+            product(1, 1, 0, 1u);
+          } else {
+            if (rv & (1u << 4)) product(0, 0, 0, (fr & 1u) ^ 1u);
+            if (rv & (1u << 5)) product(0, 1, 1, ((fr >> 1) & 1u) ^ 1u);
+            if (rv & (1u << 6)) product(1, 0, 1, (((fr >> 1) & 1u) ^ 1u) | ((rv >> 5) & 1u));
+            if (rv & (1u << 7)) product(1, 1, 2, ((fr >> 2) & 1u) ^ 1u);
+          }
           mma_commit(&empty[cs]);
         }
-        __syncwarp();
-        nprod += (unsigned)__popc((rv >> 4) & 0xFu);
       }
-      if (!ok) break;
-      if (kind & REC_LAST) { done = true; break; }
-      // publish the segment in ring slot seg % SEG_RING once the segment that used
-      // the slot before has been read and its blocks reclaimed
-      while (released < seg - (SEG_RING - 1) && ok) ok = reclaim();
-      if (!ok) break;
-      const int q = seg & (SEG_RING - 1);
-      switch (q) {
-        case 0: pend0 = used; break;
-        case 1: pend1 = used; break;
-        case 2: pend2 = used; break;
-        default: pend3 = used; break;
-      }
-      if (leader) gmap[q] = written | (gblk << 8) | ((kind & REC_END) ? SEG_LAST : 0u);
-      if (leader) {
-        mma_commit(&acc_full[q]);    // arrives once every MMA of the segment has completed
-        mbar_arrive(&acc_full[q]);   // release: segment record visible to the epilogue
-      }
-      __syncwarp();
-      ++seg;
+      mbar_arrive(&plan_empty[bat % NPLAN]);
     }
     if (!ok) status[0] = 1;
-    // slice-pair products issued (each 2 MMAs of 128 x 128 x 16)
-    if (leader && a.err && nprod) atomicAdd(reinterpret_cast<unsigned long long*>(a.err + 2), nprod);
-    if (leader) mma_commit(drain);
-    __syncwarp();
-    if (!wait(drain, 0)) {
+    mma_commit(drain);
+    if (!mbar_wait(drain, 0)) {
       status[0] = 1;
-      if (leader) note_timeout(a.err, 5);
+      note_timeout(a.err, 5);
     }
+    }
+    __syncwarp();
   } else if (warp >= 2) {
     // ---------------- epilogue (warps 2-17, four per SM sub-partition).  TMEM holds
     // the super-tile transposed (lane = column, TMEM column = row): warp w reads
@@ -1291,21 +1347,38 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_square_tc(TcArgs a) {
           double prev[CH];
 #pragma unroll
           for (int i = 0; i < CH; ++i) prev[i] = emode == 2 ? O[e0 + i * TB] : 0.0;
+          // S0 = fx * su.  The sums of an iterate are below 2^53 units (|S_ij| <= 1),
+          // and then the conversion is exact and done on the integer pipes, all
+          // elements of the chunk side by side; the conversion instruction would
+          // take a slot of the FP64 pipe (phase 2 of a super-tile at N = 24,000:
+          // 51,000 -> 43,000 cycles; with a test for each element 84,000)
+          double S0[CH];
+          bool large = false;
+#pragma unroll
+          for (int i = 0; i < CH; ++i) {
+            if (gi0 + i >= a.n || gj >= a.n) fx[i] = 0;
+            large |= ((unsigned long long)(fx[i] < 0 ? -fx[i] : fx[i]) >> 53) != 0ull;
+          }
+          if (__any_sync(FULLW, large)) {
+#pragma unroll
+            for (int i = 0; i < CH; ++i) S0[i] = int_times_pow2((double)fx[i], lsu);
+          } else {
+#pragma unroll
+            for (int i = 0; i < CH; ++i) S0[i] = small_ll_times_pow2(fx[i], lsu);
+          }
           double out[CH];
           if (Z) {
 #pragma unroll
             for (int i = 0; i < CH; ++i) {
               const int64_t gi = gi0 + i;
               const bool inside = gi < a.n && gj < a.n;
-              const double fxd = inside ? (double)fx[i] : 0.0;
               const double z = inside ? zv[i] : 0.0;
               const bool dg = inside && gi == gj;
-              const double S0 = int_times_pow2(fxd, lsu);      // fx * su
-              if (emode == 1) { out[i] = S0; continue; }     // finer groups only: S is stored
+              if (emode == 1) { out[i] = S0[i]; continue; }     // finer groups only: S is stored
               // the diagonal of S = X~^2 is the squared row norm, taken in FP64
               // (its digit products are all positive and pass the exact range
               // of the FP32 group sums on dense rows)
-              const double S = (dg && a.dsq) ? a.dsq[gi] : (emode == 2 ? S0 + prev[i] : S0);
+              const double S = (dg && a.dsq) ? a.dsq[gi] : (emode == 2 ? S0[i] + prev[i] : S0[i]);
               double xn;
               // c2 S = (c2 su) fx exactly (su is a power of two)
               if (form == 1) xn = S;
@@ -1325,11 +1398,9 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_square_tc(TcArgs a) {
             for (int i = 0; i < CH; ++i) {
               const int64_t gi = gi0 + i;
               const bool inside = gi < a.n && gj < a.n;
-              const double fxd = inside ? (double)fx[i] : 0.0;
               const bool dg = inside && gi == gj;
-              const double S0 = int_times_pow2(fxd, lsu);
-              if (emode == 1) { out[i] = S0; continue; }
-              const double S = (dg && a.dsq) ? a.dsq[gi] : (emode == 2 ? S0 + prev[i] : S0);
+              if (emode == 1) { out[i] = S0[i]; continue; }
+              const double S = (dg && a.dsq) ? a.dsq[gi] : (emode == 2 ? S0[i] + prev[i] : S0[i]);
               double xn;
               if (form == 0) {
                 xn = fma(a.c2, S, dg ? a.c0 : 0.0);
