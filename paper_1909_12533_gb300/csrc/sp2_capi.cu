@@ -312,9 +312,9 @@ struct Fail {
 };
 
 // Device buffers of one tensor-core operand: super-row bitmaps, per-word
-// record counts and offsets, record index words, headers and slices.
+// record offsets, record index words, headers and slices.
 struct OpBufs {
-  Buf sbits, cnt, spos, index, head, data;
+  Buf sbits, spos, index, head, data;
 };
 
 // Per-iteration record for the adjoint: the kept tiles of X~_j and, every
@@ -344,11 +344,11 @@ struct sp2_ctx {
   int xset = 0;
   int tail_from = 0;   // first iteration of the FP64 tail (0: none yet)
   int selftest_pending = 0;   // error-path self-test still to run (1 timeout, 2 range)
-  Buf o_brow, o_bcol, o_slot, o_rowptr, o_bits;
+  Buf o_brow, o_bcol, o_slot, o_rowptr, o_bits, o_wpre;
   Buf pool[2];
   int cur = 0;
   FullPattern fp;
-  Buf fp_bits, fp_rowptr, fp_col, fp_ref, counts;
+  Buf fp_bits, fp_wpre, fp_rowptr, fp_col, fp_ref, counts;
   Buf p_e2, p_trS, p_trX, p_n2, p_kt, keep, scanbuf, scantmp, twork, rowlo, rowhi;
   Buf dsc, dcnt, d2;
   OpBufs opx, opy;   // tensor-core operands (the adjoint uses both)
@@ -356,7 +356,7 @@ struct sp2_ctx {
   // adjoint
   std::vector<Rec> recs;
   std::vector<Buf> seg;
-  Buf ident, fpB_bits, fpB_rowptr, fpB_col, fpB_ref, gpool[2], w_brow, w_bcol, w_rowptr, w_pool, dF;
+  Buf ident, fpB_bits, fpB_wpre, fpB_rowptr, fpB_col, fpB_ref, gpool[2], w_brow, w_bcol, w_rowptr, w_pool, dF;
   Buf amax, trbuf, dsq, rsq;
   Buf gflag, gpos, gkeep, u_brow, u_bcol, u_slot;   // general storage: upper sub-index
   FullPattern fpB;
@@ -376,10 +376,10 @@ struct sp2_ctx {
   sp2_ctx() {
     Buf* all[] = {&f_brow, &f_bcol, &f_slot, &f_rowptr, &f_pool, &x_brow, &x_bcol, &x_slot, &x_rowptr,
                   &y_brow, &y_bcol, &y_slot, &y_rowptr,
-                  &o_brow, &o_bcol, &o_slot, &o_rowptr, &o_bits, &pool[0], &pool[1], &fp_bits, &fp_rowptr,
+                  &o_brow, &o_bcol, &o_slot, &o_rowptr, &o_bits, &o_wpre, &fp_wpre, &fpB_wpre, &pool[0], &pool[1], &fp_bits, &fp_rowptr,
                   &fp_col, &fp_ref, &counts, &p_e2, &p_trS, &p_trX, &p_n2, &p_kt, &keep, &scanbuf, &scantmp,
                   &twork, &rowlo, &rowhi, &dsc, &dcnt, &d2, &d_brow, &d_bcol, &d_val, &opx.sbits,
-                  &opx.cnt, &opx.spos, &opx.index, &opx.head, &opx.data, &opy.sbits, &opy.cnt, &opy.spos,
+                  &opx.spos, &opx.index, &opx.head, &opx.data, &opy.sbits, &opy.spos,
                   &opy.index, &opy.head, &opy.data, &sflag, &spos, &slist, &errflag, &scount, &tcscratch, &redwork, &ident, &fpB_bits, &fpB_rowptr, &fpB_col,
                   &fpB_ref, &gpool[0], &gpool[1], &w_brow, &w_bcol, &w_rowptr, &w_pool, &dF, &amax, &trbuf, &dsq, &rsq, &gflag, &gpos, &gkeep,
                   &u_brow, &u_bcol, &u_slot};
@@ -419,23 +419,21 @@ void set_tiles(TileSet& s, Buf& br, Buf& bc, Buf& sl, Buf& rp, int64_t nnzb) {
 }
 
 // Both-triangle pattern of a tile set (bitmap + neighbour lists).
-void build_full(sp2_ctx* c, const TileSet& s, FullPattern& fp, Buf& bits, Buf& rowptr, Buf& col, Buf& ref) {
+void build_full(sp2_ctx* c, const TileSet& s, FullPattern& fp, Buf& bits, Buf& wpre, Buf& rowptr, Buf& col, Buf& ref) {
   c->ensure(bits, (size_t)c->nb * c->words * 4);
+  c->ensure(wpre, (size_t)c->nb * c->words * 4);
   c->ensure(rowptr, (size_t)(c->nb + 1) * 4);
   c->ensure(col, (size_t)std::max<int64_t>(2 * s.nnzb, 1) * 4);
   c->ensure(ref, (size_t)std::max<int64_t>(2 * s.nnzb, 1) * 4);
-  c->ensure(c->counts, (size_t)(c->nb + 1) * 4);
-  c->ensure(c->scantmp, scan_tmp_bytes(c->nb + 1) + scan_tmp_bytes(std::max<int64_t>(s.nnzb, c->nb)) + 4096);
   fp.words = c->words;
   fp.bits = bits.as<uint32_t>();
+  fp.wpre = wpre.as<int32_t>();
   fp.rowptr = rowptr.as<int32_t>();
   fp.col = col.as<int32_t>();
   fp.ref = ref.as<uint32_t>();
   fp.nnz = 2 * s.nnzb;
   c->ck(launch_bitmap(s, c->nb, fp, c->st), "bitmap");
-  c->ck(launch_row_popc(fp.bits, c->nb, c->words, c->counts.as<int32_t>(), c->st), "row popc");
-  c->ck(launch_scan_i32(c->counts.as<int32_t>(), fp.rowptr, c->nb, fp.rowptr + c->nb, c->scantmp.p, c->st),
-        "scan");
+  c->ck(launch_rows_scan(fp.bits, c->nb, c->words, fp.wpre, fp.rowptr, nullptr, c->st), "row offsets");
   c->ck(launch_fill_full(s, c->nb, fp, c->st), "fill full");
 }
 
@@ -511,8 +509,10 @@ TileSet compact_into_set(sp2_ctx* c, const TileSet& in, int set) {
 TileSet truncate_launch(sp2_ctx* c, const TileSet& in, const double* n2, double tau, int set) {
   // n2 may live in p_n2: only the flag buffers are (re)sized here
   c->ensure(c->keep, (size_t)std::max<int64_t>(in.nnzb, 1) * 4);
-  select_keep(c, in, n2, tau, c->keep.as<int32_t>());
-  return compact_into_set(c, in, set);
+  TileSet own = in;
+  own.slot = nullptr;    // F's tiles and a square's output tiles lie at their own index
+  select_keep(c, own, n2, tau, c->keep.as<int32_t>());
+  return compact_into_set(c, own, set);
 }
 
 // General storage: the same selection as the symmetric storage, made on the
@@ -546,12 +546,11 @@ TileSet truncate_launch_general(sp2_ctx* c, const TileSet& in, const double* n2,
   return compact_into_set(c, in, set);
 }
 
-// Make `t` (with its host-side count) the current X~ and build its row offsets.
+// Make `t` (with its host-side count; row offsets filled) the current X~.
 void adopt_X(sp2_ctx* c, TileSet t, int64_t nnzb, int set) {
   t.nnzb = nnzb;
   c->X = t;
   c->xset = set;
-  c->ck(launch_rowptr_from_brow(c->X.brow, c->X.nnzb, c->nb, c->X.rowptr, c->st), "rowptr");
 }
 
 
@@ -576,7 +575,7 @@ void ensure_ident(sp2_ctx* c, int64_t n) {
 // General storage of X~_0: from the symmetric set c->X (values in pool[cur])
 // to both triangles in index set 1 / pool[1 - cur], slots = tile index.
 void expand_to_general(sp2_ctx* c) {
-  build_full(c, c->X, c->fp, c->fp_bits, c->fp_rowptr, c->fp_col, c->fp_ref);
+  build_full(c, c->X, c->fp, c->fp_bits, c->fp_wpre, c->fp_rowptr, c->fp_col, c->fp_ref);
   const int64_t nG = read_count(c, c->fp.rowptr + c->nb);
   const size_t cap = (size_t)std::max<int64_t>(nG, 1) * 4;
   c->ensure(c->y_brow, cap);
@@ -592,6 +591,7 @@ void expand_to_general(sp2_ctx* c) {
   TileSet g;
   set_tiles(g, c->y_brow, c->y_bcol, c->y_slot, c->y_rowptr, 0);
   c->cur = nxt;
+  c->ck(launch_rowptr_from_brow(g.brow, nG, c->nb, g.rowptr, c->st), "rowptr");
   adopt_X(c, g, nG, 1);
 }
 
@@ -608,8 +608,14 @@ void build_general(sp2_ctx* c, bool by_index) {
     ensure_ident(c, X.nnzb);
     rslot = c->ident.as<int32_t>();
   }
+  c->ensure(c->fp_wpre, (size_t)c->nb * c->words * 4);
+  c->ensure(c->counts, (size_t)(c->nb + 1) * 4);
+  c->ck(launch_rows_scan(c->fp_bits.as<uint32_t>(), c->nb, c->words, c->fp_wpre.as<int32_t>(), c->counts.as<int32_t>(),
+                         nullptr, c->st),
+        "row offsets");
   c->fp.words = c->words;
   c->fp.bits = c->fp_bits.as<uint32_t>();
+  c->fp.wpre = c->fp_wpre.as<int32_t>();
   c->fp.rowptr = X.rowptr;
   c->fp.col = X.bcol;
   c->fp.ref = reinterpret_cast<uint32_t*>(const_cast<int32_t*>(rslot));
@@ -674,14 +680,9 @@ TcOp prepare_operand(sp2_ctx* c, const TileSet& x, const double* pool, const Ful
   const int nsr = (c->nb + 3) / 4;
   const int64_t nw = (int64_t)nsr * c->words;
   c->ensure(ob.sbits, (size_t)nw * 4);
-  c->ck(launch_super_bits(fp, c->nb, nsr, ob.sbits.as<uint32_t>(), c->st), "super bits");
-  c->ensure(ob.cnt, (size_t)nw * 4);
   c->ensure(ob.spos, (size_t)(nw + 1) * 4);
-  c->ensure(c->scantmp, scan_tmp_bytes(nw) + 4096);
-  c->ck(launch_popc_words(ob.sbits.as<uint32_t>(), nw, ob.cnt.as<int32_t>(), c->st), "popc");
-  c->ck(launch_scan_i32(ob.cnt.as<int32_t>(), ob.spos.as<int32_t>(), nw, ob.spos.as<int32_t>() + nw, c->scantmp.p,
-                        c->st),
-        "scan");
+  c->ck(launch_super_scan(fp, c->nb, nsr, ob.sbits.as<uint32_t>(), ob.spos.as<int32_t>(), nullptr, c->st),
+        "super rows");
   const int64_t nrec = read_count(c, ob.spos.as<int32_t>() + nw);
   const size_t nr = (size_t)std::max<int64_t>(nrec, 1);
   c->ensure(ob.index, nr * 16);
@@ -726,30 +727,27 @@ double pow2_scale(sp2_ctx* c, const TileSet& x, const double* pool) {
 }
 
 // Run the tcgen05 kernel on the output tiles given by the upper bitmap `obits`
-// (row offsets `orowptr`); L carries operands, coefficients and pools.
-void run_tc(sp2_ctx* c, TcLaunch& L, const uint32_t* obits, const int32_t* orowptr) {
+// (bits before each word `owpre`, row offsets `orowptr`); L carries operands, coefficients and pools.
+void run_tc(sp2_ctx* c, TcLaunch& L, const uint32_t* obits, const int32_t* owpre, const int32_t* orowptr) {
   const int k = c->prm.slices;
   const int nsr = (c->nb + 3) / 4;
   const int64_t npair = super_order_size(nsr);
   c->ensure(c->sflag, (size_t)npair * 4);
   c->ensure(c->spos, (size_t)npair * 4);
   c->ensure(c->scantmp, scan_tmp_bytes(npair) + 4096);
-  c->ck(launch_super_flags(obits, c->nb, c->words, nsr, c->sflag.as<int32_t>(), c->st, L.general), "super flags");
   c->ensure(c->scount, 16);
-  c->ck(launch_scan_i32(c->sflag.as<int32_t>(), c->spos.as<int32_t>(), npair, c->scount.as<int32_t>(),
-                        c->scantmp.p, c->st),
-        "scan");
   // no host round trip: a persistent kernel with one CTA per SM reads the
   // number of active super-tiles and takes them from a work counter
   const int64_t ubound = L.general ? (int64_t)nsr * nsr : (int64_t)nsr * (nsr + 1) / 2;
   c->ensure(c->slist, (size_t)std::max<int64_t>(ubound, 1) * 4);
-  c->ck(cudaMemsetAsync(c->scount.as<int32_t>() + 1, 0, 4, c->st), "memset");
+  c->ck(launch_super_list(obits, c->nb, c->words, nsr, c->slist.as<int32_t>(), c->scount.as<int32_t>(),
+                          c->sflag.as<int32_t>(), c->spos.as<int32_t>(), c->scantmp.p, c->st, L.general),
+        "super list");
   int sms = 0;
   c->ck(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, 0), "attribute");
   const int64_t nsuper = std::min<int64_t>(std::max(sms, 1), std::max<int64_t>(ubound, 1));
-  c->ck(launch_super_fill(c->sflag.as<int32_t>(), c->spos.as<int32_t>(), npair, nsr, c->slist.as<int32_t>(), c->st),
-        "super fill");
   L.obits = obits;
+  L.owpre = owpre;
   L.orowptr = orowptr;
   L.list = c->slist.as<int32_t>();
   L.count = c->scount.as<int32_t>();
@@ -792,6 +790,17 @@ void run_tc(sp2_ctx* c, TcLaunch& L, const uint32_t* obits, const int32_t* orowp
   c->ck(cudaEventRecord(c->evs1, c->st), "event");
 }
 
+// o_bits and o_wpre of the upper tiles of `s`
+void upper_pattern(sp2_ctx* c, const TileSet& s) {
+  c->ensure(c->o_bits, (size_t)c->nb * c->words * 4);
+  c->ensure(c->o_wpre, (size_t)c->nb * c->words * 4);
+  c->ensure(c->counts, (size_t)(c->nb + 1) * 4);
+  c->ck(launch_upper_bits(s, c->nb, c->words, c->o_bits.as<uint32_t>(), c->st), "upper bits");
+  c->ck(launch_rows_scan(c->o_bits.as<uint32_t>(), c->nb, c->words, c->o_wpre.as<int32_t>(), c->counts.as<int32_t>(),
+                         nullptr, c->st),
+        "row offsets");
+}
+
 // Forward: S = X~^2 on the product pattern (o_bits, upper only) with the fused epilogue.
 void square_tc(sp2_ctx* c, double c0, double c1, double c2, double* outpool, bool general) {
   TcLaunch L{};
@@ -811,7 +820,7 @@ void square_tc(sp2_ctx* c, double c0, double c1, double c2, double* outpool, boo
   L.opool = outpool;
   L.part = partials(c);
   L.c0 = c0; L.c1 = c1; L.c2 = c2;
-  run_tc(c, L, c->o_bits.as<uint32_t>(), c->o_rowptr.as<int32_t>());
+  run_tc(c, L, c->o_bits.as<uint32_t>(), c->o_wpre.as<int32_t>(), c->o_rowptr.as<int32_t>());
 }
 
 int fill_stats_sched(sp2_ctx* c) {
@@ -1013,7 +1022,7 @@ void finish_create(sp2_ctx* c, int64_t nnzb) {
   set_tiles(c->F, c->f_brow, c->f_bcol, c->f_slot, c->f_rowptr, nnzb);
   c->ck(launch_rowptr_from_brow(c->F.brow, nnzb, c->nb, c->F.rowptr, c->st), "rowptr");
   // Gershgorin (Section 4, Step 1)
-  build_full(c, c->F, c->fp, c->fp_bits, c->fp_rowptr, c->fp_col, c->fp_ref);
+  build_full(c, c->F, c->fp, c->fp_bits, c->fp_wpre, c->fp_rowptr, c->fp_col, c->fp_ref);
   c->ensure(c->rowlo, c->n * 8);
   c->ensure(c->rowhi, c->n * 8);
   c->ensure(c->d2, 16);
@@ -1160,6 +1169,8 @@ int sp2_run(sp2_ctx* c, sp2_stats* stats_out) {
     const long long launches0 = g_launches;
     c->ensure(c->errflag, 32);
     c->ck(cudaMemsetAsync(c->errflag.p, 0, 32, c->st), "memset");
+    c->ensure(c->redwork, reduce_work_bytes());
+    c->ck(cudaMemsetAsync(c->redwork.p, 0, 32, c->st), "memset");
     c->ck(cudaEventRecord(c->ev0, c->st), "event");
     // Algorithm 1: X_0 on F's pattern, then X~_0 = trunc(X_0, tau_0)
     const int64_t nF = c->F.nnzb;
@@ -1204,17 +1215,15 @@ int sp2_run(sp2_ctx* c, sp2_stats* stats_out) {
           ensure_ident(c, c->X.nnzb);
           Xc.slot = c->ident.as<int32_t>();
         }
-        build_full(c, Xc, c->fp, c->fp_bits, c->fp_rowptr, c->fp_col, c->fp_ref);
+        build_full(c, Xc, c->fp, c->fp_bits, c->fp_wpre, c->fp_rowptr, c->fp_col, c->fp_ref);
       }
       c->ensure(c->o_bits, (size_t)c->nb * c->words * 4);
       c->ensure(c->o_rowptr, (size_t)(c->nb + 1) * 4);
-      c->ensure(c->counts, (size_t)(c->nb + 1) * 4);
-      c->ensure(c->scantmp, scan_tmp_bytes(c->nb + 1) + 4096);
+      c->ensure(c->o_wpre, (size_t)c->nb * c->words * 4);
       c->ck(launch_product_bits(c->fp, c->fp, c->nb, c->o_bits.as<uint32_t>(), c->st, !general), "product bits");
-      c->ck(launch_row_popc(c->o_bits.as<uint32_t>(), c->nb, c->words, c->counts.as<int32_t>(), c->st), "popc");
-      c->ck(launch_scan_i32(c->counts.as<int32_t>(), c->o_rowptr.as<int32_t>(), c->nb,
-                            c->o_rowptr.as<int32_t>() + c->nb, c->scantmp.p, c->st),
-            "scan");
+      c->ck(launch_rows_scan(c->o_bits.as<uint32_t>(), c->nb, c->words, c->o_wpre.as<int32_t>(),
+                             c->o_rowptr.as<int32_t>(), nullptr, c->st),
+            "row offsets");
       const int64_t nout = read_count(c, c->o_rowptr.as<int32_t>() + c->nb);
       c->ensure(c->o_brow, nout * 4);
       c->ensure(c->o_bcol, nout * 4);
@@ -1257,7 +1266,6 @@ int sp2_run(sp2_ctx* c, sp2_stats* stats_out) {
         c->ck(cudaEventRecord(c->evs1, c->st), "event");
       }
       c->ensure(c->dsc, sizeof(StepScalars));
-      c->ensure(c->redwork, reduce_work_bytes());
       c->ck(launch_reduce_step(sa.part, nout, c->dsc.as<StepScalars>(), c->redwork.p, c->st), "reduce");
       // X~_i = trunc(X_i, tau_i) before the stop test on e_{i-1} is known (X_i's tiles
       // live in pool[nxt] at slot = output index); X~_{i-1} keeps its own index set
@@ -1521,7 +1529,7 @@ int sp2_backward(sp2_ctx* c, const sp2_bsr* W, sp2_bsr* dF) {
       vals[0] = c->recs[cp].val.as<double>();
       for (int j = cp + 1; j < i; ++j) {
         TileSet prev = rec_tiles(c, j - 1), cur = rec_tiles(c, j);
-        build_full(c, prev, c->fpB, c->fpB_bits, c->fpB_rowptr, c->fpB_col, c->fpB_ref);
+        build_full(c, prev, c->fpB, c->fpB_bits, c->fpB_wpre, c->fpB_rowptr, c->fpB_col, c->fpB_ref);
         Buf& dst = c->seg[j - cp];
         c->ensure(dst, (size_t)std::max<int64_t>(cur.nnzb, 1) * TE * 8);
         ensure_partials(c, std::max<int64_t>(cur.nnzb, 1));
@@ -1532,8 +1540,7 @@ int sp2_backward(sp2_ctx* c, const sp2_bsr* W, sp2_bsr* dF) {
           TcLaunch L{};
           L.P = prepare_operand(c, prev, vals[j - 1 - cp], c->fpB, c->opy, 1.0);
           L.Q = L.P;
-          c->ensure(c->o_bits, (size_t)c->nb * c->words * 4);
-          c->ck(launch_upper_bits(cur, c->nb, c->words, c->o_bits.as<uint32_t>(), c->st), "upper bits");
+          upper_pattern(c, cur);
           L.two_pass = false;
           L.scale = 1.0;
           L.Z = &c->fpB;
@@ -1541,7 +1548,7 @@ int sp2_backward(sp2_ctx* c, const sp2_bsr* W, sp2_bsr* dF) {
           L.opool = dst.as<double>();
           L.part = partials(c);
           L.c0 = c0; L.c1 = c1; L.c2 = c2;
-          run_tc(c, L, c->o_bits.as<uint32_t>(), cur.rowptr);
+          run_tc(c, L, c->o_bits.as<uint32_t>(), c->o_wpre.as<int32_t>(), cur.rowptr);
           vals[j - cp] = dst.as<double>();
           continue;
         }
@@ -1560,8 +1567,8 @@ int sp2_backward(sp2_ctx* c, const sp2_bsr* W, sp2_bsr* dF) {
       // reverse steps i .. cp+1:  G_{j-1} = mask_{j-1}( c1 G_j + c2 (G_j X~_{j-1} + X~_{j-1} G_j) )
       for (; i > cp; --i) {
         TileSet tg = rec_tiles(c, i), tp = rec_tiles(c, i - 1);
-        build_full(c, tg, c->fp, c->fp_bits, c->fp_rowptr, c->fp_col, c->fp_ref);
-        build_full(c, tp, c->fpB, c->fpB_bits, c->fpB_rowptr, c->fpB_col, c->fpB_ref);
+        build_full(c, tg, c->fp, c->fp_bits, c->fp_wpre, c->fp_rowptr, c->fp_col, c->fp_ref);
+        build_full(c, tp, c->fpB, c->fpB_bits, c->fpB_wpre, c->fpB_rowptr, c->fpB_col, c->fpB_ref);
         const int nxt = 1 - gcur;
         c->ensure(c->gpool[nxt], (size_t)std::max<int64_t>(tp.nnzb, 1) * TE * 8);
         ensure_partials(c, std::max<int64_t>(tp.nnzb, 1));
@@ -1573,8 +1580,7 @@ int sp2_backward(sp2_ctx* c, const sp2_bsr* W, sp2_bsr* dF) {
           TcLaunch L{};
           L.P = prepare_operand(c, tg, c->gpool[gcur].as<double>(), c->fp, c->opx, sg);
           L.Q = prepare_operand(c, tp, vals[i - 1 - cp], c->fpB, c->opy, 1.0);
-          c->ensure(c->o_bits, (size_t)c->nb * c->words * 4);
-          c->ck(launch_upper_bits(tp, c->nb, c->words, c->o_bits.as<uint32_t>(), c->st), "upper bits");
+          upper_pattern(c, tp);
           L.two_pass = true;
           L.scale = sg;
           L.Z = &c->fp;
@@ -1582,7 +1588,7 @@ int sp2_backward(sp2_ctx* c, const sp2_bsr* W, sp2_bsr* dF) {
           L.opool = c->gpool[nxt].as<double>();
           L.part = partials(c);
           L.c0 = 0.0; L.c1 = c1; L.c2 = c2;
-          run_tc(c, L, c->o_bits.as<uint32_t>(), tp.rowptr);
+          run_tc(c, L, c->o_bits.as<uint32_t>(), c->o_wpre.as<int32_t>(), tp.rowptr);
           gcur = nxt;
           continue;
         }

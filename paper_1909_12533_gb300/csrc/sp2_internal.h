@@ -20,15 +20,18 @@ struct TileSet {
   int32_t* bcol = nullptr;
   int32_t* slot = nullptr;
   int32_t* rowptr = nullptr;    // [nb + 1] offsets of each tile row
+  const int32_t* cnt = nullptr; // device count of the tiles when the host does not know it yet (nnzb: an upper bound)
 };
 
 // Both-triangle view of a symmetric tile pattern, used by the products.
 //  bits:  nb x words bitmap, bit K of row R set iff tile (R, K) or (K, R) is stored.
+//  wpre:  for every word of bits, the set bits of its row before it.
 //  rowptr/col/ref: for row R, the stored neighbours K in ascending order; ref =
 //  slot | (1u << 31) when X_RK is the transpose of the stored tile (K, R).
 struct FullPattern {
   int32_t words = 0;
   uint32_t* bits = nullptr;
+  int32_t* wpre = nullptr;      // [nb x words]
   int32_t* rowptr = nullptr;    // [nb + 1]
   int32_t* col = nullptr;       // [nnz]
   uint32_t* ref = nullptr;      // [nnz]
@@ -59,7 +62,9 @@ struct StepScalars {
 // ---------------------------------------------------------------- launchers
 // pattern.cu
 cudaError_t launch_bitmap(const TileSet& s, int nb, FullPattern& fp, cudaStream_t st);
-cudaError_t launch_row_popc(const uint32_t* bits, int nb, int words, int32_t* counts, cudaStream_t st);
+// wpre and rowptr of a bitmap in one launch; total (nullptr: skipped) also gets rowptr[nb]
+cudaError_t launch_rows_scan(const uint32_t* bits, int nb, int words, int32_t* wpre, int32_t* rowptr, int32_t* total,
+                             cudaStream_t st);
 cudaError_t launch_scan_i32(const int32_t* in, int32_t* out_excl, int64_t n, int32_t* total_dev,
                             void* tmp, cudaStream_t st);
 size_t scan_tmp_bytes(int64_t n);
@@ -96,6 +101,7 @@ struct SquareArgs {
 };
 cudaError_t launch_square_f64(const SquareArgs& a, cudaStream_t st);
 size_t reduce_work_bytes();
+// work: reduce_work_bytes(), its first word zero (the kernel leaves it zero)
 cudaError_t launch_reduce_step(const Partials& p, int64_t ntiles, StepScalars* out, void* work, cudaStream_t st);
 
 // trunc.cu: choose the tiles to drop (Frobenius / Frob-Inf readings)
@@ -116,6 +122,7 @@ cudaError_t mixed_select(const TileSet& x, const double* n2, int nb, double tau,
                          int32_t* keep, cudaStream_t st);
 
 // compact.cu
+// (out.rowptr is filled too when `in` has row offsets and every row of `in` has a tile)
 cudaError_t launch_compact(const TileSet& in, const int32_t* keep, int nb, TileSet& out, int32_t* count_dev,
                            void* scan_tmp, int32_t* scan_buf, cudaStream_t st);
 cudaError_t launch_gather_tiles(const TileSet& s, const double* pool, double* dst, cudaStream_t st);
@@ -168,6 +175,7 @@ struct TcLaunch {
   const int32_t* zslot;      // value slot of each tile index of Z's pattern (nullptr: identity)
   const double* zpool;
   const uint32_t* obits;     // output pattern bitmap (upper tiles only)
+  const int32_t* owpre;      // set bits of its row before each word
   const int32_t* orowptr;
   const int32_t* list;       // active super-tiles
   const int32_t* count;      // their number on the device
@@ -200,17 +208,19 @@ cudaError_t launch_row_sq_sum(const int32_t* spos, int nsr, int words, const dou
 cudaError_t launch_panel_slices(const uint32_t* index, int64_t nrec, const int32_t* slot, const double* pool,
                                 void* data, uint8_t* head, int k, int32_t* err, double* rsq, double scale,
                                 bool report_range, cudaStream_t st);
-cudaError_t launch_popc_words(const uint32_t* bits, int64_t n, int32_t* cnt, cudaStream_t st);
 cudaError_t launch_panel_fill(const FullPattern& fp, int nb, const uint32_t* sbits, const int32_t* spos,
                               uint32_t* index, cudaStream_t st);
 cudaError_t launch_absmax(const TileSet& x, const double* pool, unsigned long long* out, cudaStream_t st);
 cudaError_t launch_upper_bits(const TileSet& x, int nb, int words, uint32_t* bits, cudaStream_t st);
-cudaError_t launch_super_bits(const FullPattern& fp, int nb, int nsr, uint32_t* sb, cudaStream_t st);
-int64_t super_order_size(int nsr);   // length of the (padded) launch-order index space
-cudaError_t launch_super_flags(const uint32_t* obits, int nb, int words, int nsr, int32_t* flag, cudaStream_t st,
-                               bool general = false);
-cudaError_t launch_super_fill(const int32_t* flag, const int32_t* pos, int64_t n, int nsr, int32_t* list,
+// super-row bitmaps sb, offsets spos [nsr x words + 1] of their set bits; total (nullptr: skipped) also gets the last
+cudaError_t launch_super_scan(const FullPattern& fp, int nb, int nsr, uint32_t* sb, int32_t* spos, int32_t* total,
                               cudaStream_t st);
+int64_t super_order_size(int nsr);   // length of the (padded) launch-order index space
+// active super-tiles in launch order: list, count[0] = their number, count[1] = 0
+// (the work counter of k_square_tc); flag and pos (super_order_size each) and tmp
+// are scratch of the large case
+cudaError_t launch_super_list(const uint32_t* obits, int nb, int words, int nsr, int32_t* list, int32_t* count,
+                              int32_t* flag, int32_t* pos, void* tmp, cudaStream_t st, bool general = false);
 cudaError_t launch_square_tc(const TcLaunch& L, cudaStream_t st);
 
 }  // namespace sp2

@@ -170,7 +170,7 @@ __global__ void __launch_bounds__(256) k_square_f64(SqDev a) {
 // Fixed-order two-level reduction of the per-tile partials.  Block g sums the
 // contiguous range [g c, (g+1) c), c = ceil(nt / RED_BLOCKS): thread k takes
 // entries k, k + 256, ... of the range in order, then a fixed tree; one block
-// then sums the RED_BLOCKS results with the same tree.  The result depends on
+// (the last to finish) then sums the RED_BLOCKS results with the same tree.  The result depends on
 // nt only, not on scheduling.
 constexpr int RED_BLOCKS = 256;
 
@@ -179,9 +179,10 @@ struct RedPart {
   long long k;
 };
 
-__device__ void block_tree(double a, double b, double c, long long k, RedPart* out) {
+__device__ RedPart block_tree(double a, double b, double c, long long k) {
   __shared__ double s0[256], s1[256], s2[256];
   __shared__ long long s3[256];
+  __syncthreads();
   s0[threadIdx.x] = a; s1[threadIdx.x] = b; s2[threadIdx.x] = c; s3[threadIdx.x] = k;
   __syncthreads();
   for (int h = 128; h > 0; h >>= 1) {
@@ -193,10 +194,13 @@ __device__ void block_tree(double a, double b, double c, long long k, RedPart* o
     }
     __syncthreads();
   }
-  if (threadIdx.x == 0) *out = RedPart{s0[0], s1[0], s2[0], s3[0]};
+  return RedPart{s0[0], s1[0], s2[0], s3[0]};
 }
 
-__global__ void __launch_bounds__(256) k_reduce_part(Partials p, int64_t nt, RedPart* part) {
+// The block that finishes last sums the results of all (ticket: zero before and
+// after the launch).
+__global__ void __launch_bounds__(256) k_reduce_step(Partials p, int64_t nt, RedPart* part, unsigned* ticket,
+                                                     StepScalars* out) {
   const int64_t c = (nt + RED_BLOCKS - 1) / RED_BLOCKS;
   const int64_t lo = (int64_t)blockIdx.x * c, hi = min(nt, lo + c);
   double a = 0.0, b = 0.0, d = 0.0;
@@ -207,19 +211,25 @@ __global__ void __launch_bounds__(256) k_reduce_part(Partials p, int64_t nt, Red
     d += p.trX[i];
     k += p.ktiles[i];
   }
-  block_tree(a, b, d, k, &part[blockIdx.x]);
-}
-
-__global__ void __launch_bounds__(256) k_reduce_step(const RedPart* __restrict__ part, StepScalars* out) {
-  const RedPart q = part[threadIdx.x];   // RED_BLOCKS == blockDim.x
-  __shared__ RedPart r;
-  block_tree(q.e2, q.trS, q.trX, q.k, &r);
+  const RedPart mine = block_tree(a, b, d, k);
+  __shared__ bool last;
+  if (threadIdx.x == 0) {
+    part[blockIdx.x] = mine;
+    __threadfence();
+    last = atomicAdd(ticket, 1u) == RED_BLOCKS - 1;
+  }
   __syncthreads();
+  if (!last) return;
+  __threadfence();
+  const volatile RedPart* vp = part;
+  const RedPart q{vp[threadIdx.x].e2, vp[threadIdx.x].trS, vp[threadIdx.x].trX, vp[threadIdx.x].k};   // RED_BLOCKS == blockDim.x
+  const RedPart r = block_tree(q.e2, q.trS, q.trX, q.k);
   if (threadIdx.x == 0) {
     out->e2 = r.e2;
     out->trS = r.trS;
     out->trX = r.trX;
     out->triplets = r.k;
+    *ticket = 0u;
   }
 }
 
@@ -242,13 +252,13 @@ cudaError_t launch_square_f64(const SquareArgs& a, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-size_t reduce_work_bytes() { return RED_BLOCKS * sizeof(RedPart); }
+size_t reduce_work_bytes() { return (RED_BLOCKS + 1) * sizeof(RedPart); }
 
 cudaError_t launch_reduce_step(const Partials& p, int64_t ntiles, StepScalars* out, void* work, cudaStream_t st) {
-  RedPart* part = static_cast<RedPart*>(work);
-  g_launches += 2;
-  k_reduce_part<<<RED_BLOCKS, 256, 0, st>>>(p, ntiles, part);
-  k_reduce_step<<<1, RED_BLOCKS, 0, st>>>(part, out);
+  unsigned* ticket = static_cast<unsigned*>(work);
+  RedPart* part = static_cast<RedPart*>(work) + 1;
+  ++g_launches;
+  k_reduce_step<<<RED_BLOCKS, 256, 0, st>>>(p, ntiles, part, ticket, out);
   return cudaGetLastError();
 }
 

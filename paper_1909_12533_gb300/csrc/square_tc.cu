@@ -50,6 +50,7 @@
 //     output tiles present.
 // Every wait is bounded; on timeout the kernel records an error flag, stops
 // issuing work and still frees its tensor memory.
+#include "cluster_scan.h"
 #include "sp2_internal.h"
 #include <cuda_fp16.h>
 
@@ -464,17 +465,33 @@ __global__ void __launch_bounds__(128) k_row_sq_sum(const int32_t* __restrict__ 
   if (gi < n) dsq[gi] = acc;
 }
 
-// super-row bitmap: OR of the 4 tile rows
-__global__ void k_super_bits(const uint32_t* __restrict__ bits, int nb, int words, int nsr, uint32_t* sb) {
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i >= (int64_t)nsr * words) return;
-  const int R = (int)(i / words), w = (int)(i % words);
-  uint32_t m = 0;
-  for (int a = 0; a < 4; ++a) {
-    const int row = 4 * R + a;
-    if (row < nb) m |= bits[(int64_t)row * words + w];
+// Super-row bitmaps (OR of the 4 tile rows) and the exclusive prefix sums of
+// their words' set bits, one cluster launch.
+__global__ void __cluster_dims__(SCAN_CTAS, 1, 1) __launch_bounds__(SCAN_THREADS)
+    k_super_scan(const uint32_t* __restrict__ bits, int nb, int words, int nsr, uint32_t* sb, int32_t* spos,
+                 int32_t* total) {
+  const int64_t n = (int64_t)nsr * words;
+  auto word = [&](int64_t i) {
+    const int R = (int)(i / words), w = (int)(i % words);
+    uint32_t m = 0;
+    for (int a = 0; a < 4; ++a) {
+      const int row = 4 * R + a;
+      if (row < nb) m |= bits[(int64_t)row * words + w];
+    }
+    return m;
+  };
+  const int all = cluster_scan(
+      n,
+      [&](int64_t i) {
+        const uint32_t m = word(i);
+        sb[i] = m;
+        return __popc(m);
+      },
+      [&](int64_t i, int, int ex) { spos[i] = ex; });
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    spos[n] = all;
+    if (total) *total = all;
   }
-  sb[i] = m;
 }
 
 // Launch order of the super-tiles: blocks of RB super-rows x CB super-columns,
@@ -496,25 +513,46 @@ __device__ inline void blocked_decode(int64_t i, int nsr, int& R, int& C) {
   C = (int)((b % nbc) * CB + w % CB);
 }
 
-// flag of the i-th super-tile (R, C) in launch order: an output tile present
-// (and R <= C unless the storage is general)
-__global__ void k_super_flags(const uint32_t* __restrict__ obits, int nb, int words, int nsr, int general,
-                              int32_t* flag) {
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i >= blocked_size(nsr)) return;
-  int R, C;
+// 1 if the i-th super-tile (R, C) in launch order has an output tile (and R <= C
+// unless the storage is general)
+__device__ __forceinline__ int super_flag(const uint32_t* __restrict__ obits, int nb, int words, int nsr, int general,
+                                          int64_t i, int& R, int& C) {
   blocked_decode(i, nsr, R, C);
   int f = 0;
   if (R < nsr && C < nsr && (general || R <= C)) {
-    for (int a = 0; a < 4 && !f; ++a) {
+    for (int a = 0; a < 4; ++a) {
       const int row = 4 * R + a;
       if (row >= nb) break;
       const int col0 = 4 * C;
-      const uint32_t m = obits[(int64_t)row * words + (col0 >> 5)] >> (col0 & 31);
-      f = (m & 0xFu) != 0;
+      f |= ((obits[(int64_t)row * words + (col0 >> 5)] >> (col0 & 31)) & 0xFu) != 0;
     }
   }
-  flag[i] = f;
+  return f;
+}
+
+__global__ void k_super_flags(const uint32_t* __restrict__ obits, int nb, int words, int nsr, int general,
+                              int32_t* flag) {
+  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  int R, C;
+  if (i < blocked_size(nsr)) flag[i] = super_flag(obits, nb, words, nsr, general, i, R, C);
+}
+
+// flags, scan and list in one cluster launch
+__global__ void __cluster_dims__(SCAN_CTAS, 1, 1) __launch_bounds__(SCAN_THREADS)
+    k_super_list(const uint32_t* __restrict__ obits, int nb, int words, int nsr, int general, int32_t* list,
+                 int32_t* count) {
+  int R, C;
+  const int all = cluster_scan(
+      blocked_size(nsr), [&](int64_t i) { return super_flag(obits, nb, words, nsr, general, i, R, C); },
+      [&](int64_t i, int v, int ex) {
+        if (!v) return;
+        blocked_decode(i, nsr, R, C);
+        list[ex] = R * nsr + C;
+      });
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    count[0] = all;
+    count[1] = 0;
+  }
 }
 
 __global__ void k_super_fill(const int32_t* __restrict__ flag, const int32_t* __restrict__ pos, int64_t n, int nsr,
@@ -542,11 +580,13 @@ struct TcArgs {
   TcOperand P, Q;           // S = sum_K P_IK Q_KJ  (+ Q_IK P_KJ when two_pass)
   int two_pass;
   const uint32_t* zbits;    // Z (the c1 term): pattern and FP64 values
+  const int32_t* zwpre;
   const int32_t* zrowptr;
   const uint32_t* zref;
   const int32_t* zslot;     // value slot of Z's tile index (nullptr: identity)
   const double* zpool;
   const uint32_t* obits;    // output pattern bitmap, upper tiles only
+  const int32_t* owpre;     // set bits of its row before each word
   const int32_t* orowptr;   // output tile row offsets
   const int32_t* list;      // active super-tiles, R * nsr + C
   const int32_t* count;     // number of active super-tiles (device)
@@ -1231,17 +1271,13 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_square_tc(TcArgs a) {
     //   x^2 (c0 = c1 = 0, c2 = 1): S itself;  2x - x^2 (c0 = 0, c1 = 2, c2 = -1): 2 z - S.
     const int form = (a.c0 == 0.0 && a.c1 == 0.0 && a.c2 == 1.0) ? 1
                    : (a.c0 == 0.0 && a.c1 == 2.0 && a.c2 == -1.0) ? 2 : 0;
-    // index of tile (row, col) in a pattern given by row bitmaps and row
-    // offsets, -1 if absent; the lanes share the popcount of the row's words
-    auto find = [&](const uint32_t* bits, const int32_t* rowptr, int row, int col) -> int {
-      const uint32_t* rb = bits + (int64_t)row * a.words;
-      const int wc = col >> 5;
-      const uint32_t m = rb[wc];
+    // index of tile (row, col) in a pattern given by row bitmaps, the bits before
+    // each word and row offsets, -1 if absent
+    auto find = [&](const uint32_t* bits, const int32_t* wpre, const int32_t* rowptr, int row, int col) -> int {
+      const int64_t w = (int64_t)row * a.words + (col >> 5);
+      const uint32_t m = bits[w];
       if (!((m >> (col & 31)) & 1u)) return -1;
-      int cnt = 0;
-      for (int w = lane; w < wc; w += 32) cnt += __popc(rb[w]);
-      cnt = __reduce_add_sync(FULLW, cnt);
-      return rowptr[row] + cnt + __popc(m & ((1u << (col & 31)) - 1u));
+      return rowptr[row] + wpre[w] + __popc(m & ((1u << (col & 31)) - 1u));
     };
     int seg = 0;   // segments consumed
     const uint64_t pol = policy_evict_last();
@@ -1264,13 +1300,13 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_square_tc(TcArgs a) {
       long long* scr = a.scratch + (int64_t)blockIdx.x * (ST * ST) + quarter * 32 + lane;
       const int Ia = I0 + bt;                // tile row of this warp
       // output tile index
-      const int oi = (Ia < a.nb && Jb < a.nb && (a.general || Ia <= Jb)) ? find(a.obits, a.orowptr, Ia, Jb) : -1;
+      const int oi = (Ia < a.nb && Jb < a.nb && (a.general || Ia <= Jb)) ? find(a.obits, a.owpre, a.orowptr, Ia, Jb) : -1;
       // Z_IJ of the output tile (X~_IJ in the forward step; absent -> null),
       // looked up and its rows requested into L2 before the accumulators are
       // waited for, so that the chain of dependent loads overlaps the wait
       const double* Z = nullptr;
       if (oi >= 0 && emode != 1) {
-        const int zp = find(a.zbits, a.zrowptr, Ia, Jb);
+        const int zp = find(a.zbits, a.zwpre, a.zrowptr, Ia, Jb);
         if (zp >= 0) {
           const int64_t zi = (int64_t)(a.zref[zp] & ~REF_T);
           Z = a.zpool + (int64_t)(a.zslot ? a.zslot[zi] : zi) * TE;
@@ -1468,12 +1504,6 @@ cudaError_t launch_panel_slices(const uint32_t* index, int64_t nrec, const int32
   return cudaGetLastError();
 }
 
-// number of set bits of each word
-__global__ void k_popc_words(const uint32_t* __restrict__ bits, int64_t n, int32_t* cnt) {
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i < n) cnt[i] = __popc(bits[i]);
-}
-
 // Record index words: one warp per tile row; every stored tile (row, K) of the
 // both-triangle pattern writes its word (slot row % 4) of the record of
 // (super-row row / 4, K): compact tile index, bit 31 when the stored tile is
@@ -1498,13 +1528,6 @@ cudaError_t launch_row_sq_sum(const int32_t* spos, int nsr, int words, const dou
   if (nsr == 0) return cudaSuccess;
   ++g_launches;
   k_row_sq_sum<<<(unsigned)nsr, 128, 0, st>>>(spos, words, rsq, n, dsq);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_popc_words(const uint32_t* bits, int64_t n, int32_t* cnt, cudaStream_t st) {
-  if (n == 0) return cudaSuccess;
-  ++g_launches;
-  k_popc_words<<<grid_for(n, 256), 256, 0, st>>>(bits, n, cnt);
   return cudaGetLastError();
 }
 
@@ -1554,23 +1577,34 @@ cudaError_t launch_upper_bits(const TileSet& x, int nb, int words, uint32_t* bit
   return cudaGetLastError();
 }
 
-cudaError_t launch_super_bits(const FullPattern& fp, int nb, int nsr, uint32_t* sb, cudaStream_t st) {
+cudaError_t launch_super_scan(const FullPattern& fp, int nb, int nsr, uint32_t* sb, int32_t* spos, int32_t* total,
+                              cudaStream_t st) {
   ++g_launches;
-  k_super_bits<<<grid_for((int64_t)nsr * fp.words, 256), 256, 0, st>>>(fp.bits, nb, fp.words, nsr, sb);
+  k_super_scan<<<SCAN_CTAS, SCAN_THREADS, 0, st>>>(fp.bits, nb, fp.words, nsr, sb, spos, total);
   return cudaGetLastError();
 }
 
 int64_t super_order_size(int nsr) { return blocked_size(nsr); }
 
-cudaError_t launch_super_flags(const uint32_t* obits, int nb, int words, int nsr, int32_t* flag, cudaStream_t st,
-                               bool general) {
-  ++g_launches;
-  k_super_flags<<<grid_for(blocked_size(nsr), 256), 256, 0, st>>>(obits, nb, words, nsr, general ? 1 : 0, flag);
-  return cudaGetLastError();
-}
+// Launch positions up to which one cluster lists the super-tiles; above, one
+// launch over all SMs for each phase.  The cluster takes 9 us for 512 positions and
+// 19 us for 37,000, the five launches 17 us for 37,000 and the gaps between them.
+constexpr int64_t LIST_CLUSTER_MAX = 1 << 15;
 
-cudaError_t launch_super_fill(const int32_t* flag, const int32_t* pos, int64_t n, int nsr, int32_t* list,
-                              cudaStream_t st) {
+cudaError_t launch_super_list(const uint32_t* obits, int nb, int words, int nsr, int32_t* list, int32_t* count,
+                              int32_t* flag, int32_t* pos, void* tmp, cudaStream_t st, bool general) {
+  const int64_t n = blocked_size(nsr);
+  if (n <= LIST_CLUSTER_MAX) {
+    ++g_launches;
+    k_super_list<<<SCAN_CTAS, SCAN_THREADS, 0, st>>>(obits, nb, words, nsr, general ? 1 : 0, list, count);
+    return cudaGetLastError();
+  }
+  ++g_launches;
+  k_super_flags<<<grid_for(n, 256), 256, 0, st>>>(obits, nb, words, nsr, general ? 1 : 0, flag);
+  cudaError_t e = launch_scan_i32(flag, pos, n, count, tmp, st);
+  if (e != cudaSuccess) return e;
+  e = cudaMemsetAsync(count + 1, 0, 4, st);
+  if (e != cudaSuccess) return e;
   ++g_launches;
   k_super_fill<<<grid_for(n, 256), 256, 0, st>>>(flag, pos, n, nsr, list);
   return cudaGetLastError();
@@ -1582,8 +1616,8 @@ cudaError_t launch_square_tc(const TcLaunch& L, cudaStream_t st) {
   a.P = TcOperand{L.P.sbits, L.P.spos, L.P.head, static_cast<const __half*>(L.P.data)};
   a.Q = TcOperand{L.Q.sbits, L.Q.spos, L.Q.head, static_cast<const __half*>(L.Q.data)};
   a.two_pass = L.two_pass ? 1 : 0;
-  a.zbits = L.Z->bits; a.zrowptr = L.Z->rowptr; a.zref = L.Z->ref; a.zslot = L.zslot; a.zpool = L.zpool;
-  a.obits = L.obits; a.orowptr = L.orowptr; a.list = L.list; a.count = L.count; a.work = L.work;
+  a.zbits = L.Z->bits; a.zwpre = L.Z->wpre; a.zrowptr = L.Z->rowptr; a.zref = L.Z->ref; a.zslot = L.zslot; a.zpool = L.zpool;
+  a.obits = L.obits; a.owpre = L.owpre; a.orowptr = L.orowptr; a.list = L.list; a.count = L.count; a.work = L.work;
   a.opool = L.opool;
   a.part = L.part; a.c0 = L.c0; a.c1 = L.c1; a.c2 = L.c2; a.scale = L.scale; a.n = L.n; a.nb = L.nb;
   a.words = L.words; a.nsr = L.nsr; a.err = L.err; a.scratch = static_cast<long long*>(L.scratch);

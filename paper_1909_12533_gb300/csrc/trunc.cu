@@ -144,6 +144,7 @@ constexpr int64_t CL_MANY = 4096;   // tiles of a segment (mean) from which the 
 constexpr int CL_BINS = 4096;
 constexpr int CL_PASSES = 9;      // 6 over the norm (52, 41, 30, 19, 8, 0), 3 over the index (21, 10, 0)
 constexpr size_t CL_SMEM = (size_t)CL_BINS * 12;
+constexpr int MLP = 4;            // norms of a thread loaded at once
 
 __device__ __forceinline__ int cl_shift(int p) {
   return p < 5 ? 52 - 11 * p : p == 5 ? 0 : p == 6 ? 21 : p == 7 ? 10 : 0;
@@ -202,21 +203,31 @@ __global__ void __cluster_dims__(CTAS, 1, 1) __launch_bounds__(THREADS)
     __syncthreads();
     const int sh = cl_shift(p), psh = p > 0 ? cl_shift(p - 1) : 0;
     const uint32_t dm = p == 0 ? 0xFFFu : p == 5 ? 0xFFu : p == 8 ? 0x3FFu : 0x7FFu;
-    for (int64_t t = c0 + tid; t < c1; t += THREADS) {
-      const unsigned long long hi = __double_as_longlong(n2[slot ? slot[t] : t]);
-      uint32_t lo = 0u;
-      bool in = true;
-      if (p > 0 && p <= 6) in = (hi >> psh) == ph;
-      if (p > 6) in = hi == ph;
-      if (in && p >= 6) {
-        lo = (uint32_t)brow[t] * (uint32_t)nb + (uint32_t)bcol[t];
-        if (p > 6) in = (lo >> psh) == pl;
+    for (int64_t t0 = c0 + tid; t0 < c1; t0 += MLP * THREADS) {
+      unsigned long long h[MLP];
+#pragma unroll
+      for (int u = 0; u < MLP; ++u) {
+        const int64_t t = t0 + u * THREADS;
+        h[u] = t < c1 ? (unsigned long long)__double_as_longlong(n2[slot ? slot[t] : t]) : 0ull;
       }
-      if (in && mode == 1) in = bcol[t] / pt == C;
-      if (in) {
-        const uint32_t d = (p < 6 ? (uint32_t)(hi >> sh) : lo >> sh) & dm;
-        atomicAdd(&hist[d], q[t]);
-        atomicAdd(&cnt[d], 1u);
+#pragma unroll
+      for (int u = 0; u < MLP; ++u) {
+        const int64_t t = t0 + u * THREADS;
+        const unsigned long long hi = h[u];
+        uint32_t lo = 0u;
+        bool in = t < c1;
+        if (p > 0 && p <= 6) in = in && (hi >> psh) == ph;
+        if (p > 6) in = in && hi == ph;
+        if (in && p >= 6) {
+          lo = (uint32_t)brow[t] * (uint32_t)nb + (uint32_t)bcol[t];
+          if (p > 6) in = (lo >> psh) == pl;
+        }
+        if (in && mode == 1) in = bcol[t] / pt == C;
+        if (in) {
+          const uint32_t d = (p < 6 ? (uint32_t)(hi >> sh) : lo >> sh) & dm;
+          atomicAdd(&hist[d], q[t]);
+          atomicAdd(&cnt[d], 1u);
+        }
       }
     }
     cl.sync();
@@ -289,6 +300,7 @@ __global__ void __cluster_dims__(CTAS, 1, 1) __launch_bounds__(THREADS)
   }
   // dropped: keys below the prefix; the prefix's own bucket only when everything fits
   const int dsh = depth > 0 ? cl_shift(depth - 1) : 0;
+#pragma unroll 4
   for (int64_t t = c0 + tid; t < c1; t += THREADS) {
     if (mode == 1 && bcol[t] / pt != C) continue;
     const unsigned long long hi = __double_as_longlong(n2[slot ? slot[t] : t]);
