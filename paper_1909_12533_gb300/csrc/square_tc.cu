@@ -286,6 +286,19 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
 }
 
 // ------------------------------------------------------------------ slicing
+constexpr int PANEL_BYTES = 4 * SLICE_BYTES;   // one slice of the 4 tiles of a record
+
+// place in shared memory of the 16-byte core row cr = 32 (row / 8) + 8 (column / 8) + row % 8
+__device__ __forceinline__ int panel_core_row(int cr) { return cr ^ (2 * ((cr >> 3) & 3)); }
+
+// two integers |T| <= 2^11 as FP16, exact (the FP32 magic-number add, then one
+// packed conversion: the integer-to-half instruction runs at a quarter of the rate)
+__device__ __forceinline__ uint32_t pack_halves(int lo, int hi) {
+  const float a = __int_as_float(0x4B400000 + lo) - 12582912.0f, b = __int_as_float(0x4B400000 + hi) - 12582912.0f;
+  const __half2 h = __floats2half2_rn(a, b);
+  return *reinterpret_cast<const uint32_t*>(&h);
+}
+
 // One CTA per panel record e: the 4 tiles of the record (index words from
 // k_panel_fill: compact tile index, bit 31 = use the stored tile transposed;
 // all ones = absent), sliced and written as k units of 8 KB,
@@ -299,12 +312,23 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
 // FP64, unscaled (0 for an absent tile).  Summed over the records of a
 // super-row (k_row_sq_sum) they give the squared row norms of the matrix, the
 // diagonal of its square.
+//
+// Each thread takes four elements of a tile that are neighbours in a panel row
+// (four of a stored row, or of a stored column of a tile used transposed), so a
+// slice of them is one 8-byte shared-memory store.  16-byte core rows and, in odd
+// row groups, their halves are permuted in shared memory so that neither
+// orientation's stores collide; the copy to the record undoes it.  Absent tiles
+// cost a zero fill.  With rsq the FP64 pipe is the floor: two to three lane
+// operations an element at 2 per SM cycle, 0.5 ms for the 100,000 tiles of the
+// water-like N = 24,000 case (as is HBM: 3.4 GB).  One element and 2-byte stores
+// at a time, absent tiles worked through like the others, took 1.18 ms a launch;
+// this takes 0.96 ms.
 template <int K>
-__global__ void __launch_bounds__(256, 5) k_panel_slices(const uint4* __restrict__ index, const int32_t* __restrict__ slot,
+__global__ void __launch_bounds__(256, 4) k_panel_slices(const uint4* __restrict__ index, const int32_t* __restrict__ slot,
                                                        const double* __restrict__ pool, __half* data,
                                                        uint8_t* head, int32_t* err, double* rsq, int lscale,
                                                        int report_range) {
-  __shared__ __align__(16) __half sm[K * 4 * TE];
+  __shared__ __align__(16) unsigned char sm[K * PANEL_BYTES];
   __shared__ uint32_t wnz[8];
   __shared__ int first_s;
   const int64_t e = blockIdx.x;
@@ -313,65 +337,65 @@ __global__ void __launch_bounds__(256, 5) k_panel_slices(const uint4* __restrict
   const uint32_t wd[4] = {iw.x, iw.y, iw.z, iw.w};
   constexpr int W = slice_bits(K);
   constexpr int FIN = W * K - 1;                   // finest grid 2^-FIN
-  constexpr int PER = TE / 256;                    // elements of a tile per thread
-  // all loads first (16 per thread), then the integer work
-  long long xb[4][PER];
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const bool present = wd[q] != 0xFFFFFFFFu;
-    const double* src = present ? pool + (int64_t)slot[wd[q] & ~REF_T] * TE : nullptr;
-#pragma unroll
-    for (int k = 0; k < PER; ++k) xb[q][k] = present ? __double_as_longlong(src[threadIdx.x + 256 * k]) : 0ll;
-  }
-  uint32_t nz = 0;                                 // bit s: slice s has a nonzero element
-  uint32_t pres = 0;
-  // Squared row sums (rsq): thread 32 w + l holds stored row w + 8 k, column
-  // l.  Row w + 8 k of a tile used as stored is complete in warp w (a sum over
-  // the lanes: lanes 8 k .. 8 k + 7 keep it in rs[q]); row l of a tile used
-  // transposed is spread over the 8 warps (rs[q] = the sum over k here, over
-  // the warps at the end).  Fixed order throughout (deterministic).
-  static_assert(PER == 4, "four elements of a tile per thread");
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  double rs[4];
+  // all loads first (16 per thread), then the integer work
+  long long xb[4][4];
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
-    pres |= (wd[q] != 0xFFFFFFFFu ? 1u : 0u) << q;
-    const bool tr = (wd[q] & REF_T) != 0;
-    rs[q] = 0.0;
-    if (rsq) {
-      // FP64 is scarce on this part: squares and sums as fused multiply-adds
-      double x[PER];
+    if (wd[q] == 0xFFFFFFFFu) continue;
+    const double* src = pool + (int64_t)slot[wd[q] & ~REF_T] * TE;
+    if (wd[q] & REF_T) {
 #pragma unroll
-      for (int k = 0; k < PER; ++k) x[k] = __longlong_as_double(xb[q][k]);
-      if (tr) {
-        rs[q] = fma(x[3], x[3], fma(x[2], x[2], fma(x[1], x[1], x[0] * x[0])));
-      } else {
-        // reduce-scatter of the 4 rows over the lanes (the first step
-        // exchanges the elements, the others the partial sums)
-        const bool b16 = (lane & 16) != 0, b8 = (lane & 8) != 0;
-        const double o0 = __shfl_xor_sync(0xffffffffu, b16 ? x[0] : x[2], 16);
-        const double o1 = __shfl_xor_sync(0xffffffffu, b16 ? x[1] : x[3], 16);
-        const double m0 = b16 ? x[2] : x[0], m1 = b16 ? x[3] : x[1];
-        const double h0 = fma(m0, m0, o0 * o0), h1 = fma(m1, m1, o1 * o1);
-        double t = (b8 ? h1 : h0) + __shfl_xor_sync(0xffffffffu, b8 ? h0 : h1, 8);
-        t += __shfl_xor_sync(0xffffffffu, t, 4);
-        t += __shfl_xor_sync(0xffffffffu, t, 2);
-        t += __shfl_xor_sync(0xffffffffu, t, 1);
-        rs[q] = t;
+      for (int k = 0; k < 4; ++k) xb[q][k] = __double_as_longlong(src[(4 * wid + k) * TB + lane]);
+    } else {
+      const longlong2* s2 = reinterpret_cast<const longlong2*>(src) + 2 * threadIdx.x;
+      const longlong2 u = s2[0], v = s2[1];
+      xb[q][0] = u.x; xb[q][1] = u.y; xb[q][2] = v.x; xb[q][3] = v.y;
+    }
+  }
+  int any[K];                                      // bits set in any element of slice s
+#pragma unroll
+  for (int s = 0; s < K; ++s) any[s] = 0;
+  // squared row sums (rsq): a row of a tile used as stored is complete in eight
+  // lanes; of a tile used transposed each warp has a part of every row (lane =
+  // row).  Fixed order throughout.
+  double rs[4];
+  uint32_t pres = 0;
+  bool far = false;                                // |x / scale| >= 2, inf or NaN
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    unsigned char* st = sm + q * SLICE_BYTES;
+    if (wd[q] == 0xFFFFFFFFu) {                    // absent: zero (the same for the whole CTA)
+      for (int i = threadIdx.x; i < K * (SLICE_BYTES / 16); i += 256)
+        *reinterpret_cast<uint4*>(st + (i >> 7) * PANEL_BYTES + (i & 127) * 16) = make_uint4(0u, 0u, 0u, 0u);
+      rs[q] = 0.0;
+      continue;
+    }
+    pres |= 1u << q;
+    const bool tr = (wd[q] & REF_T) != 0;
+    // panel row and first of four columns
+    const int r = tr ? lane : (int)(threadIdx.x >> 3), c = tr ? 4 * wid : 4 * (int)(threadIdx.x & 7);
+    if (rsq) {
+      double x[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) x[k] = __longlong_as_double(xb[q][k]);
+      rs[q] = fma(x[3], x[3], fma(x[2], x[2], fma(x[1], x[1], x[0] * x[0])));
+      if (!tr) {
+        rs[q] += __shfl_xor_sync(0xffffffffu, rs[q], 1);
+        rs[q] += __shfl_xor_sync(0xffffffffu, rs[q], 2);
+        rs[q] += __shfl_xor_sync(0xffffffffu, rs[q], 4);
       }
     }
+    int T[4][K];
 #pragma unroll
-    for (int k = 0; k < PER; ++k) {
-      const int i = threadIdx.x + 256 * k;
-      // stored element (i / 32, i % 32) is element (r, c) of the panel's tile
-      const int r = tr ? (i & 31) : (i >> 5), c = tr ? (i >> 5) : (i & 31);
+    for (int k = 0; k < 4; ++k) {
       // v = x / scale * 2^FIN rounded to the nearest integer (ties to even),
       // from the bits of x = m 2^(ex - 1075): v = m >> sh on the integer pipes
       const long long x = xb[q][k];
       const int ex = (int)((x >> 52) & 0x7FF);
       long long v = 0;
-      if (ex - lscale >= 1024) {           // |x / scale| >= 2, inf or NaN: flagged, clamped
-        if (err) atomicOr(err, 4);
+      if (ex - lscale >= 1024) {           // flagged below, clamped
+        far = true;
         v = (1ll << (FIN + 1)) - 1;
         if (x < 0) v = -v;
       } else if (ex != 0) {
@@ -389,24 +413,30 @@ __global__ void __launch_bounds__(256, 5) k_panel_slices(const uint4* __restrict
         }
         v = x < 0 ? -(long long)qv : (long long)qv;
       }
-      int T[K];
 #pragma unroll
       for (int s = 0; s < K - 1; ++s) {
         const int sh = W * (K - 1 - s);
         const long long hi = (v + (1ll << (sh - 1))) >> sh;   // round to nearest (ties up)
-        T[s] = (int)hi;
+        T[k][s] = (int)hi;
         v -= hi * (1ll << sh);
       }
-      T[K - 1] = (int)v;
+      T[k][K - 1] = (int)v;
 #pragma unroll
-      for (int s = 0; s < K; ++s) {
-        nz |= (T[s] != 0 ? 1u : 0u) << s;
-        sm[(s * 4 + q) * TE + (r >> 3) * 256 + (c >> 3) * 64 + (r & 7) * 8 + (c & 7)] = __int2half_rn(T[s]);
-      }
+      for (int s = 0; s < K; ++s) any[s] |= T[k][s];
     }
+    const int cr = (r >> 3) * 32 + (c >> 3) * 8 + (r & 7);
+    unsigned char* dst = st + panel_core_row(cr) * 16 + ((((c >> 2) & 1) ^ ((cr >> 5) & 1)) * 8);
+#pragma unroll
+    for (int s = 0; s < K; ++s)
+      *reinterpret_cast<uint2*>(dst + s * PANEL_BYTES) =
+          make_uint2(pack_halves(T[0][s], T[1][s]), pack_halves(T[2][s], T[3][s]));
   }
+  if (far && err) atomicOr(err, 4);
+  uint32_t nz = 0;
+#pragma unroll
+  for (int s = 0; s < K; ++s) nz |= (any[s] != 0 ? 1u : 0u) << s;
   nz = __reduce_or_sync(0xffffffffu, nz);
-  if ((threadIdx.x & 31) == 0) wnz[threadIdx.x >> 5] = nz;
+  if (lane == 0) wnz[wid] = nz;
   __syncthreads();
   if (threadIdx.x == 0) {
     uint32_t m = 0;
@@ -417,27 +447,32 @@ __global__ void __launch_bounds__(256, 5) k_panel_slices(const uint4* __restrict
   }
   __syncthreads();
   // units below the first nonzero slice are all zero and never read: not written
-  const uint4* s4 = reinterpret_cast<const uint4*>(sm);
   uint4* d4 = reinterpret_cast<uint4*>(data + e * (int64_t)(K * 4 * TE));
-  for (int i = first_s * (4 * TE / 8) + threadIdx.x; i < K * 4 * TE / 8; i += blockDim.x) d4[i] = s4[i];
+  for (int i = first_s * (PANEL_BYTES / 16) + threadIdx.x; i < K * (PANEL_BYTES / 16); i += 256) {
+    const int cr = i & 127;
+    uint4 v = *reinterpret_cast<const uint4*>(sm + ((i & ~127) | panel_core_row(cr)) * 16);
+    if (cr & 32) v = make_uint4(v.z, v.w, v.x, v.y);
+    d4[i] = v;
+  }
   if (!rsq) return;
-  __syncthreads();                                 // sm is free: reused for the warp sums
+  __syncthreads();                                 // sm is free: reused for the parts of the row sums
   double* red = reinterpret_cast<double*>(sm);     // [8 warps][4 tiles][32 rows]
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
-    if ((wd[q] & REF_T) != 0) {
-      red[wid * 128 + q * 32 + lane] = rs[q];
-    } else {
-      red[wid * 128 + q * 32 + lane] = 0.0;
-      __syncwarp();
-      if ((lane & 7) == 0) red[wid * 128 + q * 32 + wid + 8 * (lane >> 3)] = rs[q];
-    }
+    if (wd[q] == 0xFFFFFFFFu) continue;
+    if (wd[q] & REF_T) red[wid * 128 + q * 32 + lane] = rs[q];
+    else if ((lane & 7) == 0) red[q * 32 + (int)(threadIdx.x >> 3)] = rs[q];
   }
   __syncthreads();
   if (threadIdx.x < 128) {
+    const uint32_t w = reinterpret_cast<const uint32_t*>(index + e)[threadIdx.x >> 5];
     double sum = 0.0;
+    if (w != 0xFFFFFFFFu) {
+      sum = red[threadIdx.x];
+      if (w & REF_T)
 #pragma unroll
-    for (int u = 0; u < 8; ++u) sum += red[u * 128 + threadIdx.x];
+        for (int u = 1; u < 8; ++u) sum += red[u * 128 + threadIdx.x];
+    }
     rsq[e * 128 + threadIdx.x] = sum;
   }
 }
@@ -652,7 +687,7 @@ struct TcArgs {
 // integer conversions in the epilogue 84,000, 58,000, 398,000.  Two MMA issuers
 // taking turns (one warp more, 80 registers instead of 96): 91,000, 64,000.  Two
 // sub-steps for each barrier: 87,000, 59,000.
-constexpr int UNIT_BYTES = 4 * SLICE_BYTES;
+constexpr int UNIT_BYTES = PANEL_BYTES;
 constexpr int STAGE_BYTES = 4 * UNIT_BYTES;
 constexpr int STAGES = 6;                          // sub-steps in flight
 constexpr int NPLAN = 4;                           // batches between the planner and the issuer
