@@ -243,8 +243,17 @@ cudaMemPool_t device_pool() {
 // Page-locked host scratch of a context (step scalars, counts): blocks of the
 // process are kept on a free list, so creating a context costs no page-locked
 // allocation after the first.
-struct HostBlock {
+struct StepStatus {        // what a step of sp2_run tells the host, one device block and one copy
+  int32_t err[2];          // error bits, timeout sites
+  long long products;      // slice-pair products issued so far
+  double trace;            // trace(X~_i) in the trace-correcting mode
+  int32_t kept;            // tiles of X~_i
+  int32_t nout, nrec;      // next square: output tiles, records of the operand
+  int32_t pad[5];
   StepScalars sc;
+};
+struct HostBlock {
+  StepStatus st;
   int32_t cnt[4];
   double d2[2];
 };
@@ -350,19 +359,19 @@ struct sp2_ctx {
   FullPattern fp;
   Buf fp_bits, fp_wpre, fp_rowptr, fp_col, fp_ref, counts;
   Buf p_e2, p_trS, p_trX, p_n2, p_kt, keep, scanbuf, scantmp, twork, rowlo, rowhi;
-  Buf dsc, dcnt, d2;
+  Buf dcnt, d2;
   OpBufs opx, opy;   // tensor-core operands (the adjoint uses both)
   Buf sflag, spos, slist, errflag, scount, tcscratch, redwork;
   // adjoint
   std::vector<Rec> recs;
   std::vector<Buf> seg;
   Buf ident, fpB_bits, fpB_wpre, fpB_rowptr, fpB_col, fpB_ref, gpool[2], w_brow, w_bcol, w_rowptr, w_pool, dF;
-  Buf amax, trbuf, dsq, rsq;
+  Buf amax, dsq, rsq;
   Buf gflag, gpos, gkeep, u_brow, u_bcol, u_slot;   // general storage: upper sub-index
   FullPattern fpB;
   double backward_ms = 0.0;
   HostBlock* hb = nullptr;
-  StepScalars* h_sc = nullptr;
+  StepStatus* h_st = nullptr;
   int32_t* h_cnt = nullptr;
   double* h_d2 = nullptr;
   cudaEvent_t ev0 = nullptr, ev1 = nullptr, evs0 = nullptr, evs1 = nullptr;
@@ -378,10 +387,10 @@ struct sp2_ctx {
                   &y_brow, &y_bcol, &y_slot, &y_rowptr,
                   &o_brow, &o_bcol, &o_slot, &o_rowptr, &o_bits, &o_wpre, &fp_wpre, &fpB_wpre, &pool[0], &pool[1], &fp_bits, &fp_rowptr,
                   &fp_col, &fp_ref, &counts, &p_e2, &p_trS, &p_trX, &p_n2, &p_kt, &keep, &scanbuf, &scantmp,
-                  &twork, &rowlo, &rowhi, &dsc, &dcnt, &d2, &d_brow, &d_bcol, &d_val, &opx.sbits,
+                  &twork, &rowlo, &rowhi, &dcnt, &d2, &d_brow, &d_bcol, &d_val, &opx.sbits,
                   &opx.spos, &opx.index, &opx.head, &opx.data, &opy.sbits, &opy.spos,
                   &opy.index, &opy.head, &opy.data, &sflag, &spos, &slist, &errflag, &scount, &tcscratch, &redwork, &ident, &fpB_bits, &fpB_rowptr, &fpB_col,
-                  &fpB_ref, &gpool[0], &gpool[1], &w_brow, &w_bcol, &w_rowptr, &w_pool, &dF, &amax, &trbuf, &dsq, &rsq, &gflag, &gpos, &gkeep,
+                  &fpB_ref, &gpool[0], &gpool[1], &w_brow, &w_bcol, &w_rowptr, &w_pool, &dF, &amax, &dsq, &rsq, &gflag, &gpos, &gkeep,
                   &u_brow, &u_bcol, &u_slot};
     for (Buf* b : all) bufs.push_back(b);
   }
@@ -406,6 +415,8 @@ struct sp2_ctx {
     b.cap = want;
   }
   void sync() { ck(cudaStreamSynchronize(st), "stream sync"); }
+  // the device block of StepStatus (its error words are errflag)
+  StepStatus* dev_status() const { return errflag.as<StepStatus>(); }
 };
 
 namespace {
@@ -464,9 +475,6 @@ int32_t read_count(sp2_ctx* c, const int32_t* dev) {
   return *c->h_cnt;
 }
 
-// Truncate the tile set `in` (values indexed by slot, norms in n2[slot]) and
-// compact its index into index set `set`; the kept-tile count is left in dcnt[0]
-// (no host round trip).  Returns the target TileSet (nnzb not yet known).
 // keep flags of the tiles of `in` under the context's truncation norm
 void select_keep(sp2_ctx* c, const TileSet& in, const double* n2, double tau, int32_t* keep) {
   const int64_t part_tiles = std::max<int64_t>(1, c->prm.frobinf_part / TB);
@@ -481,7 +489,7 @@ void select_keep(sp2_ctx* c, const TileSet& in, const double* n2, double tau, in
 }
 
 // Compact the tiles of `in` whose keep flag (c->keep) is set into index set
-// `set`; the kept-tile count is left in dcnt[0] (no host round trip).
+// `set`; the kept-tile count is left in the status block (no host round trip).
 TileSet compact_into_set(sp2_ctx* c, const TileSet& in, int set) {
   const size_t cap = (size_t)std::max<int64_t>(in.nnzb, 1) * 4;
   Buf& br = set ? c->y_brow : c->x_brow;
@@ -492,20 +500,21 @@ TileSet compact_into_set(sp2_ctx* c, const TileSet& in, int set) {
   c->ensure(bc, cap);
   c->ensure(sl, cap);
   c->ensure(rp, (size_t)(c->nb + 1) * 4);
-  c->ensure(c->dcnt, 16);
   c->ensure(c->scanbuf, cap);
   c->ensure(c->scantmp, scan_tmp_bytes(in.nnzb) + 4096);
   TileSet t;
   set_tiles(t, br, bc, sl, rp, 0);
-  c->ck(launch_compact(in, c->keep.as<int32_t>(), c->nb, t, c->dcnt.as<int32_t>(), c->scantmp.p,
+  c->ck(launch_compact(in, c->keep.as<int32_t>(), c->nb, t, &c->dev_status()->kept, c->scantmp.p,
                        c->scanbuf.as<int32_t>(), c->st),
         "compact");
+  t.nnzb = in.nnzb;      // an upper bound until the host has read the count
+  t.cnt = &c->dev_status()->kept;
   return t;
 }
 
 // Truncate the tile set `in` (values indexed by slot, norms in n2[slot]) and
-// compact its index into index set `set`; the kept-tile count is left in dcnt[0]
-// (no host round trip).  Returns the target TileSet (nnzb not yet known).
+// compact its index into index set `set` (no host round trip: the target's tile
+// count is on the device).
 TileSet truncate_launch(sp2_ctx* c, const TileSet& in, const double* n2, double tau, int set) {
   // n2 may live in p_n2: only the flag buffers are (re)sized here
   c->ensure(c->keep, (size_t)std::max<int64_t>(in.nnzb, 1) * 4);
@@ -549,6 +558,7 @@ TileSet truncate_launch_general(sp2_ctx* c, const TileSet& in, const double* n2,
 // Make `t` (with its host-side count; row offsets filled) the current X~.
 void adopt_X(sp2_ctx* c, TileSet t, int64_t nnzb, int set) {
   t.nnzb = nnzb;
+  t.cnt = nullptr;
   c->X = t;
   c->xset = set;
 }
@@ -667,6 +677,15 @@ bool use_tc(const sp2_ctx* c, int i) {
   return true;
 }
 
+// Super-row bitmaps and record offsets of an operand (total: also to *total).
+void super_rows(sp2_ctx* c, const FullPattern& fp, OpBufs& ob, int32_t* total) {
+  const int nsr = (c->nb + 3) / 4;
+  const int64_t nw = (int64_t)nsr * c->words;
+  c->ensure(ob.sbits, (size_t)nw * 4);
+  c->ensure(ob.spos, (size_t)(nw + 1) * 4);
+  c->ck(launch_super_scan(fp, c->nb, nsr, ob.sbits.as<uint32_t>(), ob.spos.as<int32_t>(), total, c->st), "super rows");
+}
+
 // FP16 slices (scale: power of two applied before slicing) of the tiles of `x`
 // (values by slot in `pool`) into `slices`, plus the super-row bitmap of `fp`.
 // Panel records of the tiles of `x` (values at pool slot x.slot[t] of tile
@@ -674,16 +693,16 @@ bool use_tc(const sp2_ctx* c, int i) {
 // offsets, record index words, then the FP16 slices and header of every
 // record.  Reads the number of records back (one host round trip).  With
 // dsq: also the squared row norms of x into dsq (n doubles; FP64, unscaled).
+// nrec_known >= 0: super_rows() has run and its count has been read.
 TcOp prepare_operand(sp2_ctx* c, const TileSet& x, const double* pool, const FullPattern& fp, OpBufs& ob,
-                     double scale, double* dsq = nullptr) {
+                     double scale, double* dsq = nullptr, int64_t nrec_known = -1) {
   const int k = c->prm.slices;
   const int nsr = (c->nb + 3) / 4;
-  const int64_t nw = (int64_t)nsr * c->words;
-  c->ensure(ob.sbits, (size_t)nw * 4);
-  c->ensure(ob.spos, (size_t)(nw + 1) * 4);
-  c->ck(launch_super_scan(fp, c->nb, nsr, ob.sbits.as<uint32_t>(), ob.spos.as<int32_t>(), nullptr, c->st),
-        "super rows");
-  const int64_t nrec = read_count(c, ob.spos.as<int32_t>() + nw);
+  int64_t nrec = nrec_known;
+  if (nrec < 0) {
+    super_rows(c, fp, ob, nullptr);
+    nrec = read_count(c, ob.spos.as<int32_t>() + (int64_t)nsr * c->words);
+  }
   const size_t nr = (size_t)std::max<int64_t>(nrec, 1);
   c->ensure(ob.index, nr * 16);
   c->ensure(ob.head, nr);
@@ -801,13 +820,26 @@ void upper_pattern(sp2_ctx* c, const TileSet& s) {
         "row offsets");
 }
 
+// Product pattern of c->fp with itself (o_bits, o_wpre, o_rowptr) and its number
+// of tiles in the status block.
+void product_pattern(sp2_ctx* c, bool upper) {
+  c->ensure(c->o_bits, (size_t)c->nb * c->words * 4);
+  c->ensure(c->o_wpre, (size_t)c->nb * c->words * 4);
+  c->ensure(c->o_rowptr, (size_t)(c->nb + 1) * 4);
+  c->ck(launch_product_bits(c->fp, c->fp, c->nb, c->o_bits.as<uint32_t>(), c->st, upper), "product bits");
+  c->ck(launch_rows_scan(c->o_bits.as<uint32_t>(), c->nb, c->words, c->o_wpre.as<int32_t>(),
+                         c->o_rowptr.as<int32_t>(), &c->dev_status()->nout, c->st),
+        "row offsets");
+}
+
 // Forward: S = X~^2 on the product pattern (o_bits, upper only) with the fused epilogue.
-void square_tc(sp2_ctx* c, double c0, double c1, double c2, double* outpool, bool general) {
+void square_tc(sp2_ctx* c, double c0, double c1, double c2, double* outpool, bool general, int64_t nrec) {
   TcLaunch L{};
   // the diagonal of S = X~^2 from the FP64 squared row norms of X~, summed
   // while the records of A are sliced
   c->ensure(c->dsq, (size_t)c->n * 8);
-  L.P = prepare_operand(c, c->X, c->pool[c->cur].as<double>(), c->fp, c->opx, 1.0, c->dsq.as<double>());
+  L.P = prepare_operand(c, c->X, c->pool[c->cur].as<double>(), c->fp, c->opx, 1.0, c->dsq.as<double>(),
+                        nrec);
   // general storage: B is read by columns, from its own records
   L.Q = general ? prepare_operand(c, c->X, c->pool[c->cur].as<double>(), c->fpB, c->opy, 1.0) : L.P;
   L.general = general;
@@ -821,6 +853,28 @@ void square_tc(sp2_ctx* c, double c0, double c1, double c2, double* outpool, boo
   L.part = partials(c);
   L.c0 = c0; L.c1 = c1; L.c2 = c2;
   run_tc(c, L, c->o_bits.as<uint32_t>(), c->o_wpre.as<int32_t>(), c->o_rowptr.as<int32_t>());
+}
+
+// Symbolic part of the square of the symmetric set X (its count may still be on
+// the device): both-triangle pattern, product pattern (upper + diagonal) and,
+// for the tensor path, the operand's super-rows.  The tensor path addresses
+// tiles by compact index (slices), the FP64 path by slot.  The numbers of output
+// tiles and of records are left in the status block.
+void symbolic(sp2_ctx* c, TileSet X, bool tc) {
+  if (tc) {
+    ensure_ident(c, X.nnzb);
+    X.slot = c->ident.as<int32_t>();
+  }
+  build_full(c, X, c->fp, c->fp_bits, c->fp_wpre, c->fp_rowptr, c->fp_col, c->fp_ref);
+  product_pattern(c, true);
+  if (tc) super_rows(c, c->fp, c->opx, &c->dev_status()->nrec);
+}
+
+// The status block on the host (synchronises the stream).
+const StepStatus& read_status(sp2_ctx* c) {
+  c->ck(cudaMemcpyAsync(c->h_st, c->errflag.p, sizeof(StepStatus), cudaMemcpyDeviceToHost, c->st), "d2h");
+  c->sync();
+  return *c->h_st;
 }
 
 int fill_stats_sched(sp2_ctx* c) {
@@ -998,7 +1052,7 @@ void init_ctx_resources(sp2_ctx* c) {
     c->last_error = "page-locked host allocation failed";
     throw Fail{SP2_ERR_OOM};
   }
-  c->h_sc = &c->hb->sc;
+  c->h_st = &c->hb->st;
   c->h_cnt = c->hb->cnt;
   c->h_d2 = c->hb->d2;
 }
@@ -1167,8 +1221,8 @@ int sp2_run(sp2_ctx* c, sp2_stats* stats_out) {
       S.prec_hist[i] = -1;
     }
     const long long launches0 = g_launches;
-    c->ensure(c->errflag, 32);
-    c->ck(cudaMemsetAsync(c->errflag.p, 0, 32, c->st), "memset");
+    c->ensure(c->errflag, sizeof(StepStatus));
+    c->ck(cudaMemsetAsync(c->errflag.p, 0, sizeof(StepStatus), c->st), "memset");
     c->ensure(c->redwork, reduce_work_bytes());
     c->ck(cudaMemsetAsync(c->redwork.p, 0, 32, c->st), "memset");
     c->ck(cudaEventRecord(c->ev0, c->st), "event");
@@ -1181,23 +1235,28 @@ int sp2_run(sp2_ctx* c, sp2_stats* stats_out) {
           "x0");
     c->cur = 0;
     const bool trace_mode = c->prm.mode == SP2_MODE_TRACE;
-    {
-      TileSet t0 = truncate_launch(c, c->F, c->p_n2.as<double>(), sch.tau[0], 0);
-      if (trace_mode) {
-        // trace(X~_0) for the first choice (X_0's tiles in F's order, values in pool[0])
-        c->ensure(c->trbuf, 16);
-        c->ck(launch_trace_kept(c->F, c->keep.as<int32_t>(), c->pool[0].as<double>(), c->nb, c->n,
-                                c->trbuf.as<double>(), c->st),
-              "trace");
-        c->ck(cudaMemcpyAsync(c->h_d2 + 1, c->trbuf.p, 8, cudaMemcpyDeviceToHost, c->st), "d2h");
-      }
-      adopt_X(c, t0, read_count(c, c->dcnt.as<int32_t>()), 0);
-    }
-    double tr_cur = trace_mode ? c->h_d2[1] : 0.0;   // trace(X~_{i-1}) in trace mode
     const bool general = c->prm.storage == SP2_STORAGE_GENERAL;
+    StepStatus* const ds = c->dev_status();
+    c->tail_from = 0;
+    // One host round trip per step.  The symbolic part of the next square is
+    // queued behind the truncation, before the host knows whether the iteration
+    // stops there, so that its counts come back with the step's scalars (reading
+    // the output tiles, the records and the scalars one after the other left the
+    // GPU idle three times per step).  symbolic_tc: the path it was
+    // queued for.
+    bool symbolic_tc = use_tc(c, 1);
+    TileSet t0 = truncate_launch(c, c->F, c->p_n2.as<double>(), sch.tau[0], 0);
+    if (trace_mode)
+      // trace(X~_0) for the first choice (X_0's tiles in F's order, values in pool[0])
+      c->ck(launch_trace_kept(c->F, c->keep.as<int32_t>(), c->pool[0].as<double>(), c->nb, c->n, &ds->trace, c->st),
+            "trace");
+    if (!general) symbolic(c, t0, symbolic_tc);
+    read_status(c);
+    adopt_X(c, t0, c->h_st->kept, 0);
+    double tr_cur = c->h_st->trace;   // trace(X~_{i-1}) in trace mode
+    int64_t nout = c->h_st->nout, nrec = c->h_st->nrec;
     if (general) expand_to_general(c);
     S.nnzb_hist[0] = c->X.nnzb;
-    c->tail_from = 0;
     free_recs(c);
     record(c, 0);
     std::vector<double> ev, tv;
@@ -1205,26 +1264,15 @@ int sp2_run(sp2_ctx* c, sp2_stats* stats_out) {
     bool converged = false;
     for (int i = 1; i <= sch.n_max + 1; ++i) {
       const bool tc = use_tc(c, i);
-      // symbolic: both-triangle pattern of X~_{i-1}, product pattern (upper + diagonal);
-      // the tensor path addresses tiles by compact index (slices), the FP64 path by slot
       if (general) {
         build_general(c, tc);
-      } else {
-        TileSet Xc = c->X;
-        if (tc) {
-          ensure_ident(c, c->X.nnzb);
-          Xc.slot = c->ident.as<int32_t>();
-        }
-        build_full(c, Xc, c->fp, c->fp_bits, c->fp_wpre, c->fp_rowptr, c->fp_col, c->fp_ref);
+        product_pattern(c, false);
+        nout = read_status(c).nout;
+      } else if (tc != symbolic_tc) {      // the FP64 tail begins here
+        symbolic(c, c->X, tc);
+        nout = read_status(c).nout;
+        nrec = c->h_st->nrec;
       }
-      c->ensure(c->o_bits, (size_t)c->nb * c->words * 4);
-      c->ensure(c->o_rowptr, (size_t)(c->nb + 1) * 4);
-      c->ensure(c->o_wpre, (size_t)c->nb * c->words * 4);
-      c->ck(launch_product_bits(c->fp, c->fp, c->nb, c->o_bits.as<uint32_t>(), c->st, !general), "product bits");
-      c->ck(launch_rows_scan(c->o_bits.as<uint32_t>(), c->nb, c->words, c->o_wpre.as<int32_t>(),
-                             c->o_rowptr.as<int32_t>(), nullptr, c->st),
-            "row offsets");
-      const int64_t nout = read_count(c, c->o_rowptr.as<int32_t>() + c->nb);
       c->ensure(c->o_brow, nout * 4);
       c->ensure(c->o_bcol, nout * 4);
       c->ensure(c->o_slot, nout * 4);
@@ -1259,14 +1307,13 @@ int sp2_run(sp2_ctx* c, sp2_stats* stats_out) {
       sa.n = c->n; sa.nb = c->nb;
       sa.part = partials(c);
       if (tc) {
-        square_tc(c, c0, c1, c2, sa.outpool, general);
+        square_tc(c, c0, c1, c2, sa.outpool, general, general ? -1 : nrec);
       } else {
         c->ck(cudaEventRecord(c->evs0, c->st), "event");
         c->ck(launch_square_f64(sa, c->st), "square f64");
         c->ck(cudaEventRecord(c->evs1, c->st), "event");
       }
-      c->ensure(c->dsc, sizeof(StepScalars));
-      c->ck(launch_reduce_step(sa.part, nout, c->dsc.as<StepScalars>(), c->redwork.p, c->st), "reduce");
+      c->ck(launch_reduce_step(sa.part, nout, &ds->sc, c->redwork.p, c->st), "reduce");
       // X~_i = trunc(X_i, tau_i) before the stop test on e_{i-1} is known (X_i's tiles
       // live in pool[nxt] at slot = output index); X~_{i-1} keeps its own index set
       const bool more = i <= sch.n_max;
@@ -1274,44 +1321,40 @@ int sp2_run(sp2_ctx* c, sp2_stats* stats_out) {
       if (more)
         next = general ? truncate_launch_general(c, c->out, c->p_n2.as<double>(), sch.tau[i], 1 - c->xset)
                        : truncate_launch(c, c->out, c->p_n2.as<double>(), sch.tau[i], 1 - c->xset);
-      if (more && trace_mode) {
+      if (more && trace_mode)
         // trace(X~_i) for the next choice: the kept diagonal tiles of the output
-        c->ck(launch_trace_kept(c->out, c->keep.as<int32_t>(), c->pool[nxt].as<double>(), c->nb, c->n,
-                                c->trbuf.as<double>(), c->st),
+        c->ck(launch_trace_kept(c->out, c->keep.as<int32_t>(), c->pool[nxt].as<double>(), c->nb, c->n, &ds->trace,
+                                c->st),
               "trace");
-        c->ck(cudaMemcpyAsync(c->h_d2 + 1, c->trbuf.p, 8, cudaMemcpyDeviceToHost, c->st), "d2h");
+      if (more && !general) {
+        symbolic_tc = use_tc(c, i + 1);
+        symbolic(c, next, symbolic_tc);
       }
-      // one host round trip per step: scalars, error flags, kept-tile count
-      c->ck(cudaMemcpyAsync(c->h_sc, c->dsc.p, sizeof(StepScalars), cudaMemcpyDeviceToHost, c->st), "d2h");
-      c->ck(cudaMemcpyAsync(c->h_cnt + 2, c->errflag.p, 8, cudaMemcpyDeviceToHost, c->st), "d2h");
-      c->ck(cudaMemcpyAsync(c->h_d2, c->errflag.as<char>() + 8, 8, cudaMemcpyDeviceToHost, c->st), "d2h");
-      if (more) c->ck(cudaMemcpyAsync(c->h_cnt, c->dcnt.p, 4, cudaMemcpyDeviceToHost, c->st), "d2h");
-      c->sync();
-      if (c->h_cnt[2] & 1) {
+      const StepStatus& hs = read_status(c);
+      if (hs.err[0] & 1) {
         char sites[16];
-        snprintf(sites, sizeof sites, "0x%x", (unsigned)c->h_cnt[3]);
+        snprintf(sites, sizeof sites, "0x%x", (unsigned)hs.err[1]);
         c->last_error = std::string("tensor-core square: a bounded wait timed out (sites ") + sites + ")";
         fprintf(stderr, "sp2_run: %s\n", c->last_error.c_str());
         throw Fail{SP2_ERR_TIMEOUT};
       }
-      if (c->h_cnt[2] & 4) {
+      if (hs.err[0] & 4) {
         c->last_error = "an element of the iterate reached |x| >= 2, outside the range of the tensor-core slices";
         fprintf(stderr, "sp2_run: %s\n", c->last_error.c_str());
         throw Fail{SP2_ERR_RANGE};
       }
       if (tc) {
         // slice-pair products issued, each two 128 x 128 x 16 MMAs
-        const long long products = *reinterpret_cast<long long*>(c->h_d2);
-        S.tc_hw_flops = (double)products * 2.0 * 128.0 * 128.0 * 32.0;
+        S.tc_hw_flops = (double)hs.products * 2.0 * 128.0 * 128.0 * 32.0;
       }
       float ms = 0.f;
       c->ck(cudaEventElapsedTime(&ms, c->evs0, c->evs1), "elapsed");
       S.square_ms += ms;
       S.squares += 1;
-      S.tile_triplets += c->h_sc->triplets;
+      S.tile_triplets += hs.sc.triplets;
       const int j = i - 1;
-      const double ej = std::sqrt(std::max(c->h_sc->e2, 0.0));
-      const double tj = c->h_sc->trX - c->h_sc->trS;
+      const double ej = std::sqrt(std::max(hs.sc.e2, 0.0));
+      const double tj = hs.sc.trX - hs.sc.trS;
       if (!std::isfinite(ej) || !std::isfinite(tj)) {
         c->last_error = "e_j or t_j is not finite";
         fprintf(stderr, "sp2_run: %s\n", c->last_error.c_str());
@@ -1334,8 +1377,10 @@ int sp2_run(sp2_ctx* c, sp2_stats* stats_out) {
       }
       if (stop) { n_out = j; converged = true; break; }
       if (!more) { n_out = j; break; }
-      adopt_X(c, next, c->h_cnt[0], 1 - c->xset);
-      if (trace_mode) tr_cur = c->h_d2[1];
+      adopt_X(c, next, hs.kept, 1 - c->xset);
+      tr_cur = hs.trace;
+      nout = hs.nout;
+      nrec = hs.nrec;
       c->cur = nxt;
       S.nnzb_hist[i] = c->X.nnzb;
       record(c, i);
@@ -1354,6 +1399,7 @@ int sp2_run(sp2_ctx* c, sp2_stats* stats_out) {
       Dx.bcol = c->u_bcol.as<int32_t>();
       Dx.slot = c->u_slot.as<int32_t>();
       Dx.rowptr = nullptr;
+      c->ensure(c->dcnt, 16);
       c->ck(launch_compact(c->X, c->gflag.as<int32_t>(), c->nb, Dx, c->dcnt.as<int32_t>(), c->scantmp.p,
                            c->gpos.as<int32_t>(), c->st),
             "upper tiles");
@@ -1477,8 +1523,8 @@ int sp2_backward(sp2_ctx* c, const sp2_bsr* W, sp2_bsr* dF) {
   if (n < 0 || (int)c->recs.size() < n + 1) return SP2_ERR_STATE;
   try {
     c->ck(cudaEventRecord(c->ev0, c->st), "event");
-    c->ensure(c->errflag, 32);
-    c->ck(cudaMemsetAsync(c->errflag.p, 0, 32, c->st), "memset");
+    c->ensure(c->errflag, sizeof(StepStatus));
+    c->ck(cudaMemsetAsync(c->errflag.p, 0, sizeof(StepStatus), c->st), "memset");
     const Schedule& sch = c->sch;
     const int k = c->prm.ckpt_every;
     // W -> device, validated like F (diagonal tiles not required)
