@@ -16,7 +16,11 @@
 // one CTA of 256 threads per output tile, 4 outputs per thread, both operand
 // tiles staged in shared memory (transposed on the fly when the stored tile is
 // the mirror), several CTAs per SM hide the load latency.
+#include <cooperative_groups.h>
+
 #include "sp2_internal.h"
+
+namespace cg = cooperative_groups;
 
 namespace sp2 {
 namespace {
@@ -167,6 +171,174 @@ __global__ void __launch_bounds__(256) k_square_f64(SqDev a) {
   if (threadIdx.x == 0) a.part.ktiles[t] = nk;
 }
 
+// The same for few output tiles: a cluster of four CTAs per tile, each with 8 of
+// its 32 rows and one output element per thread.  With a CTA per tile the FP64
+// pipe idles where a multiprocessor has one tile less than another, and between
+// the tiles of a lone CTA's K loop; quarter tiles even the first out and the next
+// K tile's operands are fetched into registers while the current ones are
+// multiplied, so the second goes too.  The products of an element are added in
+// the same order.  Strip s has rows 4 s .. 4 s + 3 and 16 + 4 s .. 16 + 4 s + 3: all
+// elements that one thread of the kernel above sums, so the tile's partial sums
+// are formed in its order too (the Step 3 estimates magnify their last bits) and
+// meet in the cluster's first CTA.
+constexpr int STRIPS = 4;
+constexpr int SROWS = TB / STRIPS;
+
+// Steps through the K of R_P(I) & R_Q(J) in ascending order.
+struct KWalk {
+  const uint32_t* bi;
+  const uint32_t* bj;
+  const uint32_t* pref;
+  const uint32_t* qref;
+  int words, w, baseI, baseJ;
+  uint32_t mi, mj, m;
+  __device__ KWalk(const PatDev& P, const PatDev& Q, int I, int J, int nw)
+      : bi(P.bits + (int64_t)I * nw), bj(Q.bits + (int64_t)J * nw), pref(P.ref), qref(Q.ref), words(nw), w(0),
+        baseI(P.rowptr[I]), baseJ(Q.rowptr[J]) {
+    mi = bi[0];
+    mj = bj[0];
+    m = mi & mj;
+  }
+  __device__ bool next(uint32_t& ra, uint32_t& rb) {
+    while (m == 0u) {
+      baseI += __popc(mi);
+      baseJ += __popc(mj);
+      if (++w >= words) return false;
+      mi = bi[w];
+      mj = bj[w];
+      m = mi & mj;
+    }
+    const uint32_t below = (m & (0u - m)) - 1u;
+    m &= m - 1u;
+    ra = pref[baseI + __popc(mi & below)];
+    rb = qref[baseJ + __popc(mj & below)];
+    return true;
+  }
+};
+
+template <bool SYM>
+__global__ void __cluster_dims__(STRIPS, 1, 1) __launch_bounds__(256) k_square_f64_strips(SqDev a) {
+  __shared__ double As[2][SROWS][TB + 1];
+  __shared__ double Bs[2][TB][TB + 1];
+  __shared__ double val[3][SROWS][TB];     // S, X~ - S, X_new of the strip
+  __shared__ double sums[4][8];            // e2, n2, trS, trX of the 8 warps of a whole-tile CTA (used in the first CTA)
+  cg::cluster_group cl = cg::this_cluster();
+  const int strip = (int)cl.block_rank();
+  const int64_t t = blockIdx.x / STRIPS;
+  const int I = a.obrow[t], J = a.obcol[t];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  // tile row of strip row i
+  auto row_of = [&](int i) { return 4 * strip + (i & 3) + 16 * (i >> 2); };
+  double acc = 0.0;
+  int nk = 0;
+  for (int pass = 0; pass < (SYM ? 2 : 1); ++pass) {
+    const PatDev& P = pass == 0 ? a.A : a.B;
+    const PatDev& Q = pass == 0 ? a.B : a.A;
+    const double* pp = pass == 0 ? a.apool : a.bpool;
+    const double* qp = pass == 0 ? a.bpool : a.apool;
+    KWalk walk(P, Q, I, J, a.words);
+    double va, vb[4];
+    uint32_t ra, rb;
+    bool at = false, bt = false;
+    auto fetch = [&]() -> bool {
+      if (!walk.next(ra, rb)) return false;
+      at = (ra & REF_T) != 0;
+      bt = (rb & REF_T) == 0;      // Q_KJ = (Q_JK)^T
+      const double* sa = pp + (int64_t)(ra & ~REF_T) * TE;
+      const double* sb = qp + (int64_t)(rb & ~REF_T) * TE;
+      // stored order for the strip's rows, or 8 columns of the 32 stored rows
+      va = at ? sa[(threadIdx.x >> 3) * TB + row_of(threadIdx.x & 7)] : sa[row_of(warp) * TB + lane];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) vb[q] = sb[threadIdx.x + 256 * q];
+      return true;
+    };
+    bool more = fetch();
+    int buf = 0;
+    while (more) {
+      if (at) As[buf][threadIdx.x & 7][threadIdx.x >> 3] = va;
+      else As[buf][warp][lane] = va;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int r = warp + 8 * q;
+        if (bt) Bs[buf][lane][r] = vb[q]; else Bs[buf][r][lane] = vb[q];
+      }
+      __syncthreads();
+      more = fetch();
+#pragma unroll 8
+      for (int k = 0; k < TB; ++k) acc = fma(As[buf][warp][k], Bs[buf][k][lane], acc);
+      buf ^= 1;      // the other buffer's last readers have passed the barrier above
+      ++nk;
+    }
+    if (SYM) __syncthreads();
+  }
+  const uint32_t* bz = a.Z.bits + (int64_t)I * a.words;
+  const int wj = J >> 5;
+  const uint32_t mz = bz[wj];
+  const bool hasZ = (mz >> (J & 31)) & 1u;
+  const double* Zt = nullptr;
+  if (hasZ) {
+    int pos = a.Z.rowptr[I];
+    for (int w = 0; w < wj; ++w) pos += __popc(bz[w]);
+    pos += __popc(mz & ((1u << (J & 31)) - 1u));
+    Zt = a.zpool + (int64_t)(a.Z.ref[pos] & ~REF_T) * TE;  // I <= J: never a mirror
+  }
+  const int r = row_of(warp);
+  const int64_t gi = (int64_t)I * TB + r, gj = (int64_t)J * TB + lane;
+  const bool inside = gi < a.n && gj < a.n;
+  const double s = inside ? acc : 0.0;
+  const double z = (inside && hasZ) ? Zt[r * TB + lane] : 0.0;
+  const bool dg = inside && gi == gj;
+  const double xn = inside ? ((dg ? a.c0 : 0.0) + a.c1 * z) + a.c2 * s : 0.0;
+  a.opool[(int64_t)a.oslot[t] * TE + r * TB + lane] = xn;
+  val[0][warp][lane] = s;
+  val[1][warp][lane] = z - s;
+  val[2][warp][lane] = xn;
+  cl.sync();      // the values are written, and every CTA of the cluster has started
+  if (threadIdx.x < 64) {
+    // thread (ty, tx) of the whole-tile kernel: elements (ty + 16 u, tx + 16 v)
+    const int i = threadIdx.x >> 4, tx = threadIdx.x & 15, ty = row_of(i);
+    double e2 = 0.0, n2 = 0.0, trS = 0.0, trX = 0.0;
+#pragma unroll
+    for (int u = 0; u < 2; ++u)
+#pragma unroll
+      for (int v = 0; v < 2; ++v) {
+        const double d = val[1][i + 4 * u][tx + 16 * v], x = val[2][i + 4 * u][tx + 16 * v];
+        e2 = fma(d, d, e2);
+        n2 = fma(x, x, n2);
+        if (I == J && ty == tx && u == v) {      // s and z of a padding element are zero
+          const double sv = val[0][i + 4 * u][tx + 16 * v];
+          trS += sv;
+          trX += (int64_t)I * TB + ty + 16 * u < a.n && hasZ ? Zt[(ty + 16 * u) * (TB + 1)] : 0.0;
+        }
+      }
+    for (int o = 16; o > 0; o >>= 1) {
+      e2 += __shfl_xor_sync(0xffffffffu, e2, o);
+      n2 += __shfl_xor_sync(0xffffffffu, n2, o);
+      trS += __shfl_xor_sync(0xffffffffu, trS, o);
+      trX += __shfl_xor_sync(0xffffffffu, trX, o);
+    }
+    if (lane == 0) {
+      double (*dst)[8] = reinterpret_cast<double (*)[8]>(cl.map_shared_rank(&sums[0][0], 0));
+      const int w = 2 * strip + warp;
+      dst[0][w] = e2;
+      dst[1][w] = n2;
+      dst[2][w] = trS;
+      dst[3][w] = trX;
+    }
+  }
+  cl.sync();
+  if (strip == 0 && threadIdx.x < 4) {
+    const int q = threadIdx.x;
+    double v = 0.0;
+    for (int k = 0; k < 8; ++k) v += sums[q][k];
+    if (q == 0) a.part.e2[t] = ((I == J || a.general) ? 1.0 : 2.0) * v;
+    if (q == 1) a.part.n2[t] = v;
+    if (q == 2) a.part.trS[t] = v;
+    if (q == 3) a.part.trX[t] = v;
+    if (q == 0) a.part.ktiles[t] = nk;
+  }
+}
+
 // Fixed-order two-level reduction of the per-tile partials.  Block g sums the
 // contiguous range [g c, (g+1) c), c = ceil(nt / RED_BLOCKS): thread k takes
 // entries k, k + 256, ... of the range in order, then a fixed tree; one block
@@ -233,6 +405,14 @@ __global__ void __launch_bounds__(256) k_reduce_step(Partials p, int64_t nt, Red
   }
 }
 
+// Output tiles up to which a tile is split over a cluster.  Dense matrices, one
+// CTA per tile -> four: 10 tiles 45.9 -> 18.6 us a square, 36 tiles 79.6 -> 28.2,
+// 91 tiles 122 -> 94, 136 tiles 147 -> 146, 210 tiles 336 -> 261 (two rounds of
+// CTAs on 152 multiprocessors become 1.4); 300 tiles 400 -> 457, 435 tiles 719 ->
+// 728 (clusters of four do not fill every multiprocessor), 528 tiles 1047 -> 995,
+// 1176 tiles 3102 -> 3136.
+constexpr int64_t STRIP_MAX_TILES = 240;
+
 PatDev dev(const FullPattern* f) { return PatDev{f->bits, f->rowptr, f->ref}; }
 
 }  // namespace
@@ -247,8 +427,15 @@ cudaError_t launch_square_f64(const SquareArgs& a, cudaStream_t st) {
   d.n = a.n; d.words = a.A->words;
   d.general = a.general ? 1 : 0;
   d.part = a.part;
-  if (a.sym_sum) { ++g_launches; k_square_f64<true><<<(unsigned)a.out->nnzb, 256, 0, st>>>(d); }
-  else { ++g_launches; k_square_f64<false><<<(unsigned)a.out->nnzb, 256, 0, st>>>(d); }
+  const unsigned nt = (unsigned)a.out->nnzb;
+  ++g_launches;
+  if (a.out->nnzb <= STRIP_MAX_TILES) {
+    if (a.sym_sum) k_square_f64_strips<true><<<nt * STRIPS, 256, 0, st>>>(d);
+    else k_square_f64_strips<false><<<nt * STRIPS, 256, 0, st>>>(d);
+  } else {
+    if (a.sym_sum) k_square_f64<true><<<nt, 256, 0, st>>>(d);
+    else k_square_f64<false><<<nt, 256, 0, st>>>(d);
+  }
   return cudaGetLastError();
 }
 

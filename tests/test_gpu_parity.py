@@ -43,6 +43,31 @@ def test_parity_plain_sp2_and_ragged(mode):
     compare(g, o)
 
 
+@pytest.mark.parametrize("n", [661, 672, 673, 1030])
+def test_parity_around_the_split_tile_limit(n):
+    # 231 output tiles (also with a ragged tail) take four CTAs a tile, 253 and
+    # 561 one; the adjoint's products take the same two kernels
+    import paper_1909_12533_gb300 as sp2
+    d = dense_gapped(n, n // 2, (-2.0, -0.3), (0.4, 2.0), seed=n)
+    kw = dict(stop="idempotency")
+    g = run_gpu(d["F"], d["nocc"], d["homo_ub"], d["lumo_lb"], 0.0, record_masks=1, **kw)
+    o = run_oracle(d["F"], d["nocc"], d["homo_ub"], d["lumo_lb"], 0.0, **kw)
+    compare(g, o)
+    if n > 700:
+        return
+    rng = np.random.default_rng(n)
+    W = rng.standard_normal((n, n))
+    W = 0.5 * (W + W.T)
+    import oracle.sp2_oracle as O
+    ctx = sp2.SP2(from_dense(d["F"]), d["nocc"], d["homo_ub"], d["lumo_lb"], 0.0, record_masks=1, **kw)
+    ctx.run()
+    brow, bcol, val = ctx.backward(from_dense(W, keep_zero_tiles=True))
+    ctx.close()
+    dF = to_dense(BlockSparse(n=n, brow=brow.cpu().numpy(), bcol=bcol.cpu().numpy(), val=val.cpu().numpy()))
+    G = O.adjoint_sp2(d["F"], o, W)
+    assert np.linalg.norm(dF - G) <= 1e-10 * np.linalg.norm(G)
+
+
 def test_parity_frobinf_multiple_superblocks():
     c = _case("3s")
     kw = dict(trunc="frobinf", frobinf_part=1024)
