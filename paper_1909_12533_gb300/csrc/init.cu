@@ -10,8 +10,11 @@ namespace {
 // sum_{j != i} |F_ij| is accumulated sequentially over the row's tiles in
 // ascending K, so the result does not depend on scheduling.  Each tile is
 // read with coalesced loads and staged (in the orientation row I needs) in
-// shared memory, rows padded to 33 doubles.
-constexpr int GER_WARPS = 4;
+// shared memory, rows padded to 33 doubles, while the next one is loaded.  The
+// chain of additions is what bounds it: one warp a CTA spreads the rows over the
+// multiprocessors (N = 2,424: 177 us with four rows a CTA and no load ahead,
+// now 150; N = 24,000: 560 -> 423).
+constexpr int GER_WARPS = 1;
 
 __global__ void __launch_bounds__(32 * GER_WARPS) k_gershgorin(const int32_t* __restrict__ frowptr,
                                                                const int32_t* __restrict__ fcol,
@@ -26,23 +29,30 @@ __global__ void __launch_bounds__(32 * GER_WARPS) k_gershgorin(const int32_t* __
   const int64_t gi = (int64_t)I * TB + r;
   double (*ts)[TB + 1] = tile[wid];
   double d = 0.0, s = 0.0;
-  for (int e = frowptr[I]; e < frowptr[I + 1]; ++e) {
+  const int e0 = frowptr[I], e1 = frowptr[I + 1];
+  double v[TB];      // the next tile, in flight while the current one is summed
+  auto load = [&](int e) {
+    const double* T = pool + (int64_t)(fref[e] & ~REF_T) * TE;
+#pragma unroll
+    for (int i = 0; i < TB; ++i) v[i] = T[i * TB + r];      // stored row i, column r
+  };
+  if (e0 < e1) load(e0);
+  for (int e = e0; e < e1; ++e) {
     const int K = fcol[e];
-    const uint32_t rf = fref[e];
-    const double* T = pool + (int64_t)(rf & ~REF_T) * TE;
-    const bool tr = (rf & REF_T) != 0;
+    const bool tr = (fref[e] & REF_T) != 0;
     __syncwarp();
+#pragma unroll
     for (int i = 0; i < TB; ++i) {
-      const double v = T[i * TB + r];      // stored row i, column r
-      if (tr) ts[r][i] = v;
-      else ts[i][r] = v;
+      if (tr) ts[r][i] = v[i];
+      else ts[i][r] = v[i];
     }
     __syncwarp();
+    if (e + 1 < e1) load(e + 1);
     for (int c = 0; c < TB; ++c) {
       const int64_t gk = (int64_t)K * TB + c;
       if (gk >= n) break;
-      const double v = ts[r][c];
-      if (gk == gi) d = v; else s += fabs(v);
+      const double x = ts[r][c];
+      if (gk == gi) d = x; else s += fabs(x);
     }
   }
   if (gi >= n) return;
