@@ -95,17 +95,29 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
   return ok != 0;
 }
 
-// whether the phase has completed, without waiting
-__device__ __forceinline__ bool mbar_test(uint64_t* bar, uint32_t parity) {
-  uint32_t ok;
+// How many of the four ring stages from s on have completed their phase (those
+// past the wrap at `stages` the next one), without waiting: four tests in a row,
+// whose latencies overlap; a stage counts if all before it have completed.
+__device__ __forceinline__ int mbar_ready4(uint64_t* ring, int s, uint32_t parity, int stages) {
+  const bool w1 = s + 1 >= stages, w2 = s + 2 >= stages, w3 = s + 3 >= stages;
+  const uint32_t b = smem_u32(ring);
+  int m;
   asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(smem_u32(bar)), "r"(parity)
+      "{\n\t.reg .pred p, q, r, s;\n\t.reg .b32 x;\n\t"
+      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %5;\n\t"
+      "mbarrier.test_wait.parity.shared::cta.b64 q, [%2], %6;\n\t"
+      "mbarrier.test_wait.parity.shared::cta.b64 r, [%3], %7;\n\t"
+      "mbarrier.test_wait.parity.shared::cta.b64 s, [%4], %8;\n\t"
+      "selp.b32 x, 4, 3, s;\n\t"
+      "selp.b32 x, x, 2, r;\n\t"
+      "selp.b32 x, x, 1, q;\n\t"
+      "selp.b32 %0, x, 0, p;\n\t}"
+      : "=r"(m)
+      : "r"(b + 8u * (uint32_t)s), "r"(b + 8u * (uint32_t)(w1 ? s + 1 - stages : s + 1)),
+        "r"(b + 8u * (uint32_t)(w2 ? s + 2 - stages : s + 2)), "r"(b + 8u * (uint32_t)(w3 ? s + 3 - stages : s + 3)),
+        "r"(parity), "r"(parity ^ (w1 ? 1u : 0u)), "r"(parity ^ (w2 ? 1u : 0u)), "r"(parity ^ (w3 ? 1u : 0u))
       : "memory");
-  return ok != 0;
+  return m;
 }
 
 __device__ __forceinline__ unsigned long long now_ns() {
@@ -669,7 +681,7 @@ struct TcArgs {
 //
 // What bounds the kernel is how fast its serial loops run (a warp by itself takes
 // 5 to 8 cycles an instruction, and the loop of a sub-step costs the MMA issuer
-// about 250 cycles a product where the tensor pipe takes 128), not the copy path
+// 200 to 300 cycles a product where the tensor pipe takes 128), not the copy path
 // (a lone thread that issues 16 KB bulk copies fills 72 B per SM cycle out of L2;
 // a K step needs 27 KB and has 210 cycles of MMAs), not shared memory (32 B per
 // cycle of copies landing leave 128-wide MMAs at 66 cycles each) and not the
@@ -680,12 +692,17 @@ struct TcArgs {
 // the MMA issuer reads the same records; each of the three is one elected thread
 // (elect.sync: in code that a comparison of the lane number guards, the operands
 // of tcgen05.mma and cp.async.bulk cost twice as long to set up), with the next
-// record loaded and the next stage's barrier tested ahead.
+// record loaded ahead.  Each tests four stages' barriers at once and then runs
+// through as many sub-steps as are ready in an inner loop without a wait: a test
+// or a wait in that loop, even one that never has to wait, makes every MMA dearer
+// (a lone loop of four MMAs a sub-step: 445 cycles, 600 beside warps that do FP64
+// work; four sub-steps at a time 335 and 375, the tensor pipe's time being 256).
 // Cycles per super-tile, water-like N = 24,000 and 96,000, dense N = 4,096 with
 // five slices (both launches): one producer warp 126,000, 96,000, 508,000;
 // planner and one issuer 120,000, 81,000, 507,000; two issuers and 16 epilogue
 // warps 103,000, 67,000, 455,000; pairs of one-product K steps, finished records,
-// integer conversions in the epilogue 84,000, 58,000, 398,000.  Two MMA issuers
+// integer conversions in the epilogue 84,000, 58,000, 398,000; ready sub-steps
+// without waits between them 80,000, 56,000, 341,000.  Two MMA issuers
 // taking turns (one warp more, 80 registers instead of 96): 91,000, 64,000.  Two
 // sub-steps for each barrier: 87,000, 59,000.
 constexpr int UNIT_BYTES = PANEL_BYTES;
@@ -1089,7 +1106,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_square_tc(TcArgs a) {
       const uint32_t mine = smem_u32(stages) + (uint32_t)side * (2 * UNIT_BYTES);
       int s = 0;                     // next stage
       uint32_t par = 1u;             // phase that frees it
-      bool isfree = true;            // it was free when last looked at
+      int ready = 0;                 // stages from s on known to be free
       int head = 0;                  // sub-steps issued
       bool done = false;
       for (int bat = 0; !done; ++bat) {
@@ -1100,33 +1117,46 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_square_tc(TcArgs a) {
         }
         const uint4* ul = plan + (bat % NPLAN) * PLAN;
         const int n = bcnt[bat % NPLAN];
-        uint4 nx = ul[0];
-        for (int u = 0; u < n; ++u) {
-          const uint4 en = nx;
-          nx = ul[u + 1];
-          const uint32_t rv = en.x;
-          if (rv & REC_CTL) {
-            if (rv & REC_LAST) done = true;
+        int u = 0;
+        uint4 nx = ul[0];              // record u
+        while (u < n) {
+          if (nx.x & REC_CTL) {
+            if (nx.x & REC_LAST) done = true;
+            nx = ul[++u];
             continue;
           }
-          const uint32_t unit = side ? en.z : en.y, second = side ? en.w >> 16 : en.w & 0xFFFFu;
-          const __half* base = ((rv & REC_PASS1) != 0u) == (side != 0) ? a.P.data : a.Q.data;
-          const unsigned char* src = reinterpret_cast<const unsigned char*>(base) + (uint64_t)unit * UNIT_BYTES;
-          const uint32_t bytes = ((rv >> (side ? 25 : 20)) & 3u) * UNIT_BYTES;
-          const uint32_t part = second != 0u ? UNIT_BYTES : bytes;       // a pair: two copies
-          const uint32_t dst = mine + (uint32_t)s * STAGE_BYTES + ((rv & first_used) ? 0u : (uint32_t)UNIT_BYTES);
-          if (!isfree && !mbar_wait(&empty[s], par)) {
-            status[0] = 1;
-            note_timeout(a.err, 2);
-            done = true;
-            break;
+          if (ready == 0) {
+            ready = mbar_ready4(empty, s, par, STAGES);
+            if (ready == 0) {
+              if (!mbar_wait(&empty[s], par)) {
+                status[0] = 1;
+                note_timeout(a.err, 2);
+                done = true;
+                break;
+              }
+              ready = 1;
+            }
           }
-          mbar_expect_tx(&full[s], bytes);
-          bulk_g2s(dst, src, part, &full[s]);
-          if (second != 0u) bulk_g2s(dst + UNIT_BYTES, src + (uint64_t)second * UNIT_BYTES, UNIT_BYTES, &full[s]);
-          ++head;
-          if (++s == STAGES) { s = 0; par ^= 1u; }
-          isfree = mbar_test(&empty[s], par);
+          // the free stages' copies, without a wait or a test among them
+          uint4 en = nx;
+#pragma unroll 1
+          do {
+            const uint32_t rv = en.x;
+            const uint32_t unit = side ? en.z : en.y, second = side ? en.w >> 16 : en.w & 0xFFFFu;
+            en = ul[++u];
+            const __half* base = ((rv & REC_PASS1) != 0u) == (side != 0) ? a.P.data : a.Q.data;
+            const unsigned char* src = reinterpret_cast<const unsigned char*>(base) + (uint64_t)unit * UNIT_BYTES;
+            const uint32_t bytes = ((rv >> (side ? 25 : 20)) & 3u) * UNIT_BYTES;
+            const uint32_t part = second != 0u ? UNIT_BYTES : bytes;       // a pair: two copies
+            const uint32_t dst = mine + (uint32_t)s * STAGE_BYTES + ((rv & first_used) ? 0u : (uint32_t)UNIT_BYTES);
+            mbar_expect_tx(&full[s], bytes);
+            bulk_g2s(dst, src, part, &full[s]);
+            if (second != 0u) bulk_g2s(dst + UNIT_BYTES, src + (uint64_t)second * UNIT_BYTES, UNIT_BYTES, &full[s]);
+            ++head;
+            if (++s == STAGES) { s = 0; par ^= 1u; }
+            --ready;
+          } while (ready > 0 && u < n && (en.x & REC_CTL) == 0u);
+          nx = en;
         }
         mbar_arrive(&plan_empty[bat % NPLAN]);
       }
@@ -1176,8 +1206,34 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_square_tc(TcArgs a) {
     };
     int s = 0;               // next stage and the phase that fills it
     uint32_t par = 0u;
-    bool filled = false;     // stage s was full when last looked at
+    int ready = 0;           // stages from s on known to be full
     uint32_t gblk = 0u, used = 0u, written = 0u;   // open segment: block of each group, blocks, groups
+    // the products of a sub-step, from the next stage; fr: groups (from the first
+    // product's on) that it writes first, its first MMA into them overwrites
+    auto sub_step = [&](uint32_t rv, uint32_t fr) {
+      const uint32_t units = dlo + (uint32_t)s * (STAGE_BYTES >> 4);    // A0, A1, B0, B1 one unit apart
+      const int base = (int)(rv & 7u) - 1;     // group of A0 x B0
+      const uint32_t gb = base >= 0 ? gblk >> (2 * base) : gblk << 2;    // blocks of groups base, base + 1, base + 2
+      // the unit of the super-column as the M operand, that of the super-row
+      // as the N operand: TMEM holds the transposed super-tile
+      auto product = [&](int i, int j, int k, uint32_t acc) {
+        const uint32_t dcol = tmem + ((gb >> (2 * k)) & 3u) * ST;
+        const uint32_t ua = units + (uint32_t)(i * (UNIT_BYTES >> 4)), ub = units + (uint32_t)((2 + j) * (UNIT_BYTES >> 4));
+        mma_f16(dcol, dhi | ub, dhi | ua, acc);
+        mma_f16(dcol, dhi | (ub + 16u), dhi | (ua + 16u), 1u);
+      };
+      if (rv & REC_PAIR) {
+        product(0, 0, 0, (fr & 1u) ^ 1u);
+        product(1, 1, 0, 1u);
+      } else {
+        if (rv & (1u << 4)) product(0, 0, 0, (fr & 1u) ^ 1u);
+        if (rv & (1u << 5)) product(0, 1, 1, ((fr >> 1) & 1u) ^ 1u);
+        if (rv & (1u << 6)) product(1, 0, 1, (((fr >> 1) & 1u) ^ 1u) | ((rv >> 5) & 1u));
+        if (rv & (1u << 7)) product(1, 1, 2, ((fr >> 2) & 1u) ^ 1u);
+      }
+      mma_commit(&empty[s]);
+      if (++s == STAGES) { s = 0; par ^= 1u; }
+    };
     for (int bat = 0; ok && !done; ++bat) {
       if (!mbar_wait_sleep(&plan_full[bat % NPLAN], (uint32_t)(bat / NPLAN) & 1u)) {
         note_timeout(a.err, 8);
@@ -1186,10 +1242,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_square_tc(TcArgs a) {
       }
       const uint4* ul = plan + (bat % NPLAN) * PLAN;
       const int n = bcnt[bat % NPLAN];
-      uint32_t nx = ul[0].x;
-      for (int u = 0; u < n; ++u) {
+      int u = 0;
+      uint32_t nx = ul[0].x;   // record u
+      while (u < n) {
         const uint32_t rv = nx;
-        nx = ul[u + 1].x;
         if (rv & REC_CTL) {
           if (rv & REC_LAST) { done = true; break; }
           // publish the segment in ring slot seg % SEG_RING once the segment that used
@@ -1208,24 +1264,23 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_square_tc(TcArgs a) {
           mbar_arrive(&acc_full[q]);   // release: segment record visible to the epilogue
           ++seg;
           gblk = used = written = 0u;
+          nx = ul[++u].x;
           continue;
         }
-        const uint32_t units = dlo + (uint32_t)s * (STAGE_BYTES >> 4);    // A0, A1, B0, B1 one unit apart
-        const int cs = s;
-        if (!filled && !mbar_wait(&full[cs], par)) {
-          ok = false;
-          note_timeout(a.err, 3);
-          break;
+        if (ready == 0) {
+          ready = mbar_ready4(full, s, par, STAGES);
+          if (ready == 0) {
+            if (!mbar_wait(&full[s], par)) {
+              ok = false;
+              note_timeout(a.err, 3);
+              break;
+            }
+            ready = 1;
+          }
         }
-        if (++s == STAGES) { s = 0; par ^= 1u; }
-        // look at the next stage now: the answer is there when the products of
-        // this one have been issued
-        filled = mbar_test(&full[s], par);
-        // groups (relative to the launch's window, at most four live) that the
-        // segment writes first here take a TMEM block, and their first MMA overwrites it
-        const int base = (int)(rv & 7u) - 1;     // group of A0 x B0
-        uint32_t fr = 0u;
         if (rv & REC_FRESH) {
+          // groups (relative to the launch's window, at most four live) that the
+          // segment writes first here take a TMEM block
           for (uint32_t f = (rv >> 16) & 15u; f != 0u; f &= f - 1u) {
             const int g = __ffs(f) - 1;
             while (free_mask == 0u && ok) ok = reclaim();
@@ -1237,30 +1292,24 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_square_tc(TcArgs a) {
             written |= 1u << g;
           }
           if (!ok) break;
-          fr = (rv >> 16) & 15u;
+          const int base = (int)(rv & 7u) - 1;
+          uint32_t fr = (rv >> 16) & 15u;
           fr = base >= 0 ? fr >> base : fr << 1;
+          nx = ul[++u].x;
+          sub_step(rv, fr);
+          --ready;
+          continue;
         }
-        const uint32_t gb = base >= 0 ? gblk >> (2 * base) : gblk << 2;    // blocks of groups base, base + 1, base + 2
-        {
-          // the unit of the super-column as the M operand, that of the super-row
-          // as the N operand: TMEM holds the transposed super-tile
-          auto product = [&](int i, int j, int k, uint32_t acc) {
-            const uint32_t dcol = tmem + ((gb >> (2 * k)) & 3u) * ST;
-            const uint32_t ua = units + (uint32_t)(i * (UNIT_BYTES >> 4)), ub = units + (uint32_t)((2 + j) * (UNIT_BYTES >> 4));
-            mma_f16(dcol, dhi | ub, dhi | ua, acc);
-            mma_f16(dcol, dhi | (ub + 16u), dhi | (ua + 16u), 1u);
-          };
-          if (rv & REC_PAIR) {
-            product(0, 0, 0, (fr & 1u) ^ 1u);
-            product(1, 1, 0, 1u);
-          } else {
-            if (rv & (1u << 4)) product(0, 0, 0, (fr & 1u) ^ 1u);
-            if (rv & (1u << 5)) product(0, 1, 1, ((fr >> 1) & 1u) ^ 1u);
-            if (rv & (1u << 6)) product(1, 0, 1, (((fr >> 1) & 1u) ^ 1u) | ((rv >> 5) & 1u));
-            if (rv & (1u << 7)) product(1, 1, 2, ((fr >> 2) & 1u) ^ 1u);
-          }
-          mma_commit(&empty[cs]);
-        }
+        // the full stages' sub-steps, without a wait or a test among them
+        uint32_t r = rv;
+#pragma unroll 1
+        do {
+          const uint32_t cur = r;
+          r = ul[++u].x;
+          sub_step(cur, 0u);
+          --ready;
+        } while (ready > 0 && u < n && (r & (REC_CTL | REC_FRESH)) == 0u);
+        nx = r;
       }
       mbar_arrive(&plan_empty[bat % NPLAN]);
     }
