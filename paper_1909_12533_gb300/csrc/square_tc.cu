@@ -1453,89 +1453,127 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_square_tc(TcArgs a) {
       if (oi >= 0) {
         double trS = 0.0, trX = 0.0, n2 = 0.0, e2 = 0.0;
         double* O = a.opool + (int64_t)oi * TE;
+        // Everything that only some tiles need (the matrix edge, the diagonal) is
+        // under a branch of its own, outside the loops over the chunk's rows: the
+        // kernel is long for the instruction caches (99 KB; one instruction fetch in
+        // nine missed the multiprocessor's cache), and the single-thread loops of the
+        // issuers, which bound it, wait for their share of the misses.  With the
+        // cases inside the row loops: water-like N = 24,000 115 ms a run, now 105,
+        // N = 96,000 705 ms, now 610, dense N = 4,096 with five slices 47.0, now 45.7.
+        const bool edge = (int64_t)(Ia + 1) * TB > a.n || (int64_t)(Jb + 1) * TB > a.n;
+        const bool diag = Ia == Jb;
+        const bool general = Z != nullptr || (form == 0 && diag);
 #pragma unroll 1
         for (int ch = 0; ch < TB / CH; ++ch) {     // CH rows per chunk
-          const int64_t gi0 = (int64_t)Ia * TB + ch * CH;
           const long long* sp = scr + (bt * 32 + ch * CH) * ST;
           const int e0 = ch * CH * TB + lane;     // element of the chunk's first row in a tile
           double zv[CH];
+          if (Z) {
 #pragma unroll
-          for (int i = 0; i < CH; ++i) zv[i] = Z ? Z[e0 + i * TB] : 0.0;
+            for (int i = 0; i < CH; ++i) zv[i] = Z[e0 + i * TB];
+          } else {
+#pragma unroll
+            for (int i = 0; i < CH; ++i) zv[i] = 0.0;
+          }
           long long fx[CH];
 #pragma unroll
           for (int i = 0; i < CH; ++i) fx[i] = ld_staging(sp + i * ST, pol);
           // emode 2: the finer groups' S, left in the output tile by the launch before
           double prev[CH];
+          if (emode == 2) {
 #pragma unroll
-          for (int i = 0; i < CH; ++i) prev[i] = emode == 2 ? O[e0 + i * TB] : 0.0;
-          // S0 = fx * su.  The sums of an iterate are below 2^53 units (|S_ij| <= 1),
+            for (int i = 0; i < CH; ++i) prev[i] = O[e0 + i * TB];
+          } else {
+#pragma unroll
+            for (int i = 0; i < CH; ++i) prev[i] = 0.0;
+          }
+          if (edge) {
+            const int rows = gj < a.n ? (int)min((int64_t)CH, a.n - ((int64_t)Ia * TB + ch * CH)) : 0;
+#pragma unroll
+            for (int i = 0; i < CH; ++i)
+              if (i >= rows) {
+                fx[i] = 0;
+                zv[i] = 0.0;
+              }
+          }
+          // S = fx * su.  The sums of an iterate are below 2^53 units (|S_ij| <= 1),
           // and then the conversion is exact and done on the integer pipes, all
           // elements of the chunk side by side; the conversion instruction would
           // take a slot of the FP64 pipe (phase 2 of a super-tile at N = 24,000:
           // 51,000 -> 43,000 cycles; with a test for each element 84,000)
-          double S0[CH];
+          double S[CH];
           bool large = false;
 #pragma unroll
-          for (int i = 0; i < CH; ++i) {
-            if (gi0 + i >= a.n || gj >= a.n) fx[i] = 0;
-            large |= ((unsigned long long)(fx[i] < 0 ? -fx[i] : fx[i]) >> 53) != 0ull;
-          }
+          for (int i = 0; i < CH; ++i) large |= ((unsigned long long)(fx[i] < 0 ? -fx[i] : fx[i]) >> 53) != 0ull;
           if (__any_sync(FULLW, large)) {
 #pragma unroll
-            for (int i = 0; i < CH; ++i) S0[i] = int_times_pow2((double)fx[i], lsu);
+            for (int i = 0; i < CH; ++i) S[i] = int_times_pow2((double)fx[i], lsu);
           } else {
 #pragma unroll
-            for (int i = 0; i < CH; ++i) S0[i] = small_ll_times_pow2(fx[i], lsu);
+            for (int i = 0; i < CH; ++i) S[i] = small_ll_times_pow2(fx[i], lsu);
           }
-          double out[CH];
-          if (Z || (form == 0 && Ia == Jb)) {
+          double out[CH];      // emode 1 (finer groups only): S
+          if (emode == 2) {
 #pragma unroll
-            for (int i = 0; i < CH; ++i) {
-              const int64_t gi = gi0 + i;
-              const bool inside = gi < a.n && gj < a.n;
-              const double z = inside ? zv[i] : 0.0;
-              const bool dg = inside && gi == gj;
-              if (emode == 1) { out[i] = S0[i]; continue; }     // finer groups only: S is stored
+            for (int i = 0; i < CH; ++i) S[i] += prev[i];
+          }
+          if (emode == 1) {
+#pragma unroll
+            for (int i = 0; i < CH; ++i) out[i] = S[i];
+          } else {
+            const int dr = diag && gj < a.n ? lane - ch * CH : -1;      // the chunk's row on the diagonal
+            if (dr >= 0 && dr < CH) {
               // the diagonal of S = X~^2 is the squared row norm, taken in FP64
               // (its digit products are all positive and pass the exact range
               // of the FP32 group sums on dense rows)
-              const double S = (dg && a.dsq) ? a.dsq[gi] : (emode == 2 ? S0[i] + prev[i] : S0[i]);
-              double xn;
-              // c2 S = (c2 su) fx exactly (su is a power of two)
-              if (form == 1) xn = S;
-              else if (form == 2) xn = twice(z) - S;
-              else xn = fma(a.c2, S, fma(a.c1, z, dg ? a.c0 : 0.0));
-              out[i] = xn;
-              const double df = z - S;
-              e2 = fma(df, df, e2);
-              n2 = fma(xn, xn, n2);
-              if (dg) { trS += S; trX += z; }
-            }
-          } else {
-            // no X~ tile here: z = 0.  X_new = S or 2 z - S = -S (forms 1 and 2):
-            // every (z - S)^2 equals xn^2, so one FMA per element gives both sums
-            // (e2 is set from n2 below; the same values in the same order).  With
-            // acceleration (form 0) ||X_new||^2 is c2^2 ||S||^2; a tile without
-            // X~ tile on the diagonal, where c0 counts, takes the path above.
+              const double nrm = a.dsq ? a.dsq[gj] : 0.0;
 #pragma unroll
-            for (int i = 0; i < CH; ++i) {
-              const int64_t gi = gi0 + i;
-              const bool inside = gi < a.n && gj < a.n;
-              const bool dg = inside && gi == gj;
-              if (emode == 1) { out[i] = S0[i]; continue; }
-              const double S = (dg && a.dsq) ? a.dsq[gi] : (emode == 2 ? S0[i] + prev[i] : S0[i]);
-              double xn;
-              if (form == 0) xn = fma(a.c2, S, dg ? a.c0 : 0.0);
-              else xn = form == 1 ? S : negated(S);
-              out[i] = xn;
-              n2 = form == 0 ? fma(S, S, n2) : fma(xn, xn, n2);
-              if (dg) trS += S;
+              for (int i = 0; i < CH; ++i)
+                if (i == dr) {
+                  if (a.dsq) S[i] = nrm;
+                  trS += S[i];
+                  trX += zv[i];
+                }
+            }
+            if (general) {
+              if (form == 1) {
+#pragma unroll
+                for (int i = 0; i < CH; ++i) out[i] = S[i];
+              } else if (form == 2) {
+#pragma unroll
+                for (int i = 0; i < CH; ++i) out[i] = twice(zv[i]) - S[i];
+              } else {
+                // c2 S = (c2 su) fx exactly (su is a power of two)
+#pragma unroll
+                for (int i = 0; i < CH; ++i) out[i] = fma(a.c2, S[i], fma(a.c1, zv[i], i == dr ? a.c0 : 0.0));
+              }
+#pragma unroll
+              for (int i = 0; i < CH; ++i) {
+                const double df = zv[i] - S[i];
+                e2 = fma(df, df, e2);
+                n2 = fma(out[i], out[i], n2);
+              }
+            } else {
+              // no X~ tile here: z = 0.  X_new = S or 2 z - S = -S (forms 1 and 2):
+              // every (z - S)^2 equals X_new^2, so one FMA per element gives both sums
+              // (e2 is set from n2 below; the same values in the same order).  With
+              // acceleration (form 0) ||X_new||^2 is c2^2 ||S||^2; a tile without
+              // X~ tile on the diagonal, where c0 counts, takes the path above.
+#pragma unroll
+              for (int i = 0; i < CH; ++i) n2 = fma(S[i], S[i], n2);
+              if (form == 0) {
+#pragma unroll
+                for (int i = 0; i < CH; ++i) out[i] = fma(a.c2, S[i], 0.0);
+              } else {
+#pragma unroll
+                for (int i = 0; i < CH; ++i) out[i] = form == 1 ? S[i] : negated(S[i]);
+              }
             }
           }
 #pragma unroll
           for (int i = 0; i < CH; ++i) O[e0 + i * TB] = out[i];
         }
-        if (!Z && !(form == 0 && Ia == Jb)) {
+        if (!general) {
           e2 = n2;
           if (form == 0) n2 = (a.c2 * a.c2) * n2;
         }
@@ -1547,7 +1585,6 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_square_tc(TcArgs a) {
           trX += __shfl_xor_sync(FULLW, trX, o);
         }
         if (lane == 0 && emode != 1) {
-          const bool diag = Ia == Jb;
           a.part.e2[oi] = (diag || a.general ? 1.0 : 2.0) * e2;
           a.part.n2[oi] = n2;
           a.part.trS[oi] = diag ? trS : 0.0;
