@@ -229,7 +229,7 @@ def main(argv=None) -> int:
     ap.add_argument("--precision", default="split16", choices=["fp64", "split16"])
     ap.add_argument("--slices", type=int, default=4)
     ap.add_argument("--split-supply", type=int, default=None, choices=[0, 1],
-                    help="tensor path: B slices through copy warps (1) or bulk copies only (0); default: library")
+                    help="accepted for compatibility of the call, no effect")
     ap.add_argument("--fp64-tail", type=float, default=None,
                     help="tensor path with the idempotency stop: FP64 squares once e_j < this (0: none); "
                          "default: library")

@@ -650,7 +650,7 @@ struct TcArgs {
   int seg_min;              // K loops of at least this many steps are cut into segments (0: never)
   int seg_ksteps;           // K steps per segment (8 or 16, divides the 32-step batch)
   unsigned long long wait_ns;   // limit of every bounded wait
-  int selftest;             // 1: the producer first waits on a barrier nothing arrives at (timeout path test)
+  int selftest;             // 1: the planner first waits on a barrier nothing arrives at (timeout path test)
   int general;              // general storage: output tiles on both sides of the diagonal, weight 1 in e^2
   const double* dsq;        // S_ii = sum_k x_ik^2 in FP64 per global row (nullptr: from the tensor cores)
   int glo, ghi;             // slice-pair groups s + t of this launch (ghi - glo <= 3)

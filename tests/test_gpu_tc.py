@@ -144,8 +144,7 @@ def test_split16_fp64_tail_reaches_idempotency_tolerance():
 @pytest.mark.parametrize("key,extra", [(1, {}), ("2s", {}), ("3s", {}), ("4s", {}),
                                        ("5s", {"acc_flush_min": 1}), ("2s", {"storage": "general"})])
 def test_split_supply_gives_the_same_result(key, extra):
-    # the B slices through the copy warps (cp.async) instead of bulk copies: the
-    # same bytes land in the same stages, so D is the same bit for bit
+    # both values of the parameter are accepted and give the same bits
     c = make_config(key)
     kw = dict(stop=c["stop"], precision="split16", slices=4, **extra)
     a = run_gpu(c["F"], c["nocc"], c["homo_ub"], c["lumo_lb"], c["tau"], split_supply=0, **kw)
