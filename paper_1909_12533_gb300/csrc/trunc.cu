@@ -93,11 +93,18 @@ __global__ void k_seg_scale(Work w, double tau) {
   w.scale[s] = budget > 0.0 ? Q_SCALE / budget : 0.0;
 }
 
-// budget units of a tile of squared norm v and weight wt (1: stored once, 2: mirrored)
+// budget units of a tile of squared norm v and weight wt (1: stored once, 2: mirrored),
+// at most Q_CAP, which no budget holds: also for a NaN (a tile with a NaN, a
+// norm that was never computed), so that the sums of a selection stay below
+// 2^64 (2^27 tiles are a terabyte) and exactly one bin holds its cut.  A NaN
+// converted to an integer would be 2^63 units, a wrapped sum would let several
+// CTAs of a cluster name a cut, and one could leave while another still reads
+// its shared memory.  A zero tile has no units, whatever the scale (infinite
+// for a tau whose square is subnormal).
 __device__ __forceinline__ unsigned long long budget_units(double v, double wt, double sc) {
-  if (sc == 0.0) return (v == 0.0) ? 0ull : Q_CAP;
+  if (v == 0.0) return 0ull;
   const double x = (wt * v) * sc;
-  return (x >= (double)Q_CAP) ? Q_CAP : (unsigned long long)ceil(x);
+  return sc != 0.0 && x < (double)Q_CAP ? (unsigned long long)ceil(x) : Q_CAP;
 }
 
 // mode 0: one segment, scale sc; mode 1: the segment's scale.  Its own launch

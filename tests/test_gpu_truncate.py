@@ -102,6 +102,34 @@ def test_keep_flags_of_both_segment_selects(n, part, tau):
     assert np.array_equal(g, o), np.nonzero(g != o)
 
 
+@pytest.mark.parametrize("n,mode,part", [(2030, "frobenius", 4096), (500, "frobenius", 4096), (2030, "frobinf", 256),
+                                         (5900, "frobinf", 3008)])
+@pytest.mark.parametrize("tau", [0.0, 1e-3, 1e3])
+def test_tiles_with_nan_are_kept(n, mode, part, tau):
+    """A tile whose norm is a NaN fits into no budget and ranks above every finite
+    one: the flags are those of the same tiles with a huge norm instead.  Several
+    NaNs per selection, in the one-CTA select, both segment selects and the cluster."""
+    import paper_1909_12533_gb300 as sp2
+    X = _decaying(n, 31)
+    bad = np.linspace(1, X.nnzb - 2, 9).astype(int)
+    Y = BlockSparse(n=n, brow=X.brow, bcol=X.bcol, val=X.val.copy())
+    X.val[bad, 3, 5] = np.nan
+    Y.val[bad, 3, 5] = 1e100
+    g = sp2.sp2_truncate(X, tau, mode, part)
+    o = _oracle_keep(Y, tau, mode, part)
+    assert np.array_equal(g, o), np.nonzero(g != o)
+    assert g[bad].all()
+
+
+@pytest.mark.parametrize("n", [500, 2100])
+def test_tau_with_a_subnormal_square_drops_zero_tiles_only(n):
+    import paper_1909_12533_gb300 as sp2
+    X = _decaying(n, 7)
+    X.val[3:9] = 0.0
+    g = sp2.sp2_truncate(X, 1e-155, "frobenius")
+    assert not g[3:9].any() and g.sum() == X.nnzb - 6
+
+
 # ----------------------------------------------------------------- mixed norm (Section 3)
 @pytest.mark.parametrize("part", [64, 128, 4096])
 @pytest.mark.parametrize("tau", [0.0, 1e-6, 1e-3, 0.1])
