@@ -65,20 +65,21 @@ Work carve(void* base, int64_t nnzb, int64_t nseg, int nsb) {
   return w;
 }
 
+// (segment indices R * nsb + C pass 2^31 from 46,341 super-blocks on: 64-bit)
 __global__ void k_nz(const int32_t* __restrict__ brow, const int32_t* __restrict__ bcol, int64_t nnzb, int pt,
                      int nsb, int32_t* nz) {
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (t >= nnzb) return;
   const int R = brow[t] / pt, C = bcol[t] / pt;
-  nz[R * nsb + C] = 1;
-  nz[C * nsb + R] = 1;
+  nz[(int64_t)R * nsb + C] = 1;
+  nz[(int64_t)C * nsb + R] = 1;
 }
 
 __global__ void k_m(const int32_t* __restrict__ nz, int nsb, int32_t* m) {
   const int R = blockIdx.x * blockDim.x + threadIdx.x;
   if (R >= nsb) return;
   int c = 0;
-  for (int C = 0; C < nsb; ++C) c += nz[R * nsb + C];
+  for (int C = 0; C < nsb; ++C) c += nz[(int64_t)R * nsb + C];
   m[R] = c;
 }
 
@@ -119,7 +120,7 @@ __global__ void k_q(const int32_t* __restrict__ brow, const int32_t* __restrict_
   double wt = (I == J) ? 1.0 : 2.0;
   if (mode == 1) {
     const int R = I / pt, C = J / pt;
-    sc = w.scale[R * w.nsb + C];
+    sc = w.scale[(int64_t)R * w.nsb + C];
     if (R != C) wt = 1.0;
   }
   w.q[t] = budget_units(n2[slot ? slot[t] : t], wt, sc);

@@ -130,6 +130,34 @@ def test_tau_with_a_subnormal_square_drops_zero_tiles_only(n):
     assert not g[3:9].any() and g.sum() == X.nnzb - 6
 
 
+def test_more_super_blocks_than_a_32_bit_segment_index_holds():
+    """46,400 super-rows of 32 rows (46,400^2 > 2^31 segments), a block-tridiagonal
+    set with one element a tile: every segment is one tile of weight 1."""
+    import torch
+    import paper_1909_12533_gb300 as sp2
+    nb = 46400
+    brow = np.repeat(np.arange(nb, dtype=np.int32), 2)[:-1]
+    bcol = brow.copy()
+    bcol[1::2] += 1
+    a = np.random.default_rng(46).uniform(0.5, 1.5, brow.size)
+
+    class T:
+        n = 32 * nb - 5
+
+    T.brow = torch.from_numpy(brow).cuda()
+    T.bcol = torch.from_numpy(bcol).cuda()
+    T.val = torch.zeros(brow.size, 32, 32, dtype=torch.float64, device="cuda")
+    T.val[:, 0, 0] = torch.from_numpy(a).cuda()
+    tau = 3.0
+    g = sp2.sp2_truncate(T, tau, "frobinf", 32).cpu().numpy()
+    m = np.full(nb, 3)
+    m[[0, -1]] = 2
+    beta = tau / np.maximum(m[brow], m[bcol])
+    keep = np.ceil((a * a) * (2.0 ** 36 / (beta * beta))) > 2.0 ** 36
+    assert np.array_equal(g, keep.astype(np.int32)) and 0 < g.sum() < g.size
+    sp2.load().sp2_release_memory()      # 26 GB of segment tables
+
+
 # ----------------------------------------------------------------- mixed norm (Section 3)
 @pytest.mark.parametrize("part", [64, 128, 4096])
 @pytest.mark.parametrize("tau", [0.0, 1e-6, 1e-3, 0.1])
