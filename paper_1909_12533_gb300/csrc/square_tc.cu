@@ -1172,7 +1172,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_square_tc(TcArgs a) {
   } else if (warp == 1) {
     if (elect_one()) {
     // ---------------- MMA issuer, one thread.  TMEM is four blocks of 128 columns; a group
-    // accumulator of a segment (a whole super-tile, or 32 of its K steps) takes
+    // accumulator of a segment (a whole super-tile, or seg_ksteps of its K steps) takes
     // a free block on its first product, and the blocks of a segment return to
     // the pool once every epilogue warp has read them (one arrival per warp on
     // the segment slot's tmem_empty barrier; segments are reclaimed in order).
@@ -1430,8 +1430,24 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_square_tc(TcArgs a) {
             if ((written >> gg) & 1u) {        // warp-uniform: groups no product reached are zero
               float g[16];
               tmem_ld16(trow + ((gm >> (8 + 2 * gg)) & 3u) * ST, g);
+              // Integers, exact either way.  With two to four slices nothing bounds a group
+              // sum by 2^31: second slices reach 2^10, and a K loop without segments has
+              // thousands of products of each of a group's pairs, all of one sign on a
+              // diagonal that does not come from dsq or between alike rows.  Such tiles
+              // take the 64-bit conversion.  (Five slices: 256 products a segment of at
+              // most 2^20 + 3 2^18, below 2^29.)
+              float top = 0.0f;
+              if (K != 5) {
 #pragma unroll
-              for (int i = 0; i < 16; ++i) fx[i] += __float2int_rn(g[i]);      // an integer below 2^31: exact
+                for (int i = 0; i < 16; ++i) top = fmaxf(top, fabsf(g[i]));
+              }
+              if (K != 5 && __any_sync(FULLW, top >= 2147483648.0f)) {
+#pragma unroll
+                for (int i = 0; i < 16; ++i) fx[i] += __float2ll_rn(g[i]);
+              } else {
+#pragma unroll
+                for (int i = 0; i < 16; ++i) fx[i] += __float2int_rn(g[i]);
+              }
             }
           }
           if (!first) {

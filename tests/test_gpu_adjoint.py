@@ -237,3 +237,56 @@ def test_autograd_function_second_backward_and_not_converged():
     Dv3, _, _ = Fn.apply(Fv, br, bc, n, nocc, d["homo_ub"], d["lumo_lb"], 0.0,
                          {"stop": "idempotency", "n_max_cap": 3, "allow_not_converged": True})
     assert torch.isfinite(Dv3).all()
+
+
+@pytest.mark.parametrize("n,of_d", [(6400, False), (4096, True)])
+def test_split16_dense_gradient_with_group_sums_above_2_31(n, of_d):
+    # Dense F with known eigenvectors against the Daleckii-Krein form, the default four
+    # slices and K loops without segments.  The recomputed squares of the sweep take
+    # their diagonal from the tensor cores: the sum of the squared second slices,
+    # about n 2^20 / 3, passes 2^31 from n = 6,200 on.  With W = D + diagonal the
+    # two-pass product G X + X G has twice that sum (n = 4,096).  Four slices with
+    # unsegmented FP32 sums, which round above 2^24, give 9.0e-7 and 2.5e-6 here
+    # (tolerance: four times the larger); sums clamped at 2^31 give 2.0e-4 and 1.8e-4.
+    import torch
+    import paper_1909_12533_gb300 as sp2
+    g = torch.Generator(device="cuda")
+    g.manual_seed(n)
+    nocc = n // 2
+    Q = torch.linalg.qr(torch.randn(n, n, dtype=torch.float64, device="cuda", generator=g))[0]
+    lam = torch.cat([torch.linspace(-1.0, -0.6, nocc, dtype=torch.float64, device="cuda"),
+                     torch.linspace(0.6, 1.0, n - nocc, dtype=torch.float64, device="cuda")])
+    F = (Q * lam) @ Q.T
+    F = 0.5 * (F + F.T)
+    if of_d:
+        v = torch.randn(n, dtype=torch.float64, device="cuda", generator=g)
+        W = Q[:, :nocc] @ Q[:, :nocc].T + 0.05 * torch.diag(v)
+    else:
+        W = torch.randn(n, n, dtype=torch.float64, device="cuda", generator=g)
+        W = (W + W.T) / (8 * n) ** 0.5
+    Wt = Q.T @ W @ Q
+    Gt = torch.zeros_like(Wt)
+    Gt[:nocc, nocc:] = Wt[:nocc, nocc:] / (lam[:nocc, None] - lam[None, nocc:])
+    ref = Q @ (Gt + Gt.T) @ Q.T
+    nb = n // 32
+    iu, ju = np.triu_indices(nb)
+
+    class T:
+        pass
+
+    T.n = n
+    T.brow, T.bcol = (torch.from_numpy(x.astype(np.int32)).cuda() for x in (iu, ju))
+    i, j = T.brow.long(), T.bcol.long()
+    T.val = W.view(nb, 32, nb, 32).permute(0, 2, 1, 3)[i, j].contiguous()
+    ctx = sp2.SP2(F, nocc, -0.6, 0.6, 0.0, precision="split16", record_masks=1)
+    ctx.run()
+    assert ctx.code == 0
+    brow, bcol, val = ctx.backward(T)
+    ctx.close()
+    G = torch.zeros(nb, nb, 32, 32, dtype=torch.float64, device="cuda")
+    G[bcol.long(), brow.long()] = val.transpose(1, 2)
+    G[brow.long(), bcol.long()] = val
+    G = G.permute(0, 2, 1, 3).reshape(n, n)
+    err = float((G - ref).norm() / ref.norm())
+    print(f"n = {n}, W of D: {of_d}: ||dF - ref|| / ||ref|| = {err:.3e}")
+    assert err <= 1e-5

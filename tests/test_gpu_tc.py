@@ -190,3 +190,20 @@ def test_split16_diagonal_of_the_square_in_fp64():
         d = float(np.abs(b["D"] - a["D"]).max())
         print(f"dense 512, first square, {k} slices: max |X_1 - X_1(FP64)| = {d:.3e}")
         assert d <= tol
+
+
+@pytest.mark.parametrize("n", [2000, 6001])
+def test_split16_group_sums_above_2_31_of_alike_rows(n):
+    # F = -11^T / n, one delocalised orbital: D = -F, every row alike, so the products
+    # of the second slices add up with one sign and the FP32 sum of their group
+    # (three slice pairs, unit 2^-42) passes 2^31 in the last squares.  It stays below
+    # 2^33: each of its 3 n / 16 additions rounds by at most 2^8 units, and the last
+    # two squares have sums of this size.  (Clamped at 2^31: 2e-7 in every element.)
+    import torch
+    import paper_1909_12533_gb300 as sp2
+    F = torch.full((n, n), -1.0 / n, dtype=torch.float64, device="cuda")
+    D, st = sp2.run(F, 1, -0.9, -0.1, 0.0, precision="split16", slices=4)
+    err = float((D + F).abs().max())
+    print(f"n = {n}: max |D - D_ref| = {err:.3e}, n = {st['n']}")
+    assert st["converged"] and all(p == 1 for p in st["prec_hist"])
+    assert err <= 2 * (3 * n / 16) * 2.0 ** (8 - 42)
