@@ -45,7 +45,8 @@ constexpr int MIXED_POWER_ITERS = 100;        // power steps of the mixed-norm b
 struct Work {
   unsigned long long* q;   // budget units of each tile
   double* scale;           // Frob-Inf: units per squared norm of each segment
-  int32_t* nz;
+  int32_t* nz;             // [nsb x nsb] pairs of super-rows with a tile, and one word behind them:
+                           // set when the tiles are not sorted upper tiles
   int32_t* m;
   int64_t nseg;
   int32_t nsb;
@@ -53,12 +54,14 @@ struct Work {
 
 inline size_t align_up(size_t x) { return (x + 255) & ~size_t(255); }
 
+inline size_t nz_bytes(int nsb) { return ((size_t)nsb * nsb + 1) * 4; }
+
 Work carve(void* base, int64_t nnzb, int64_t nseg, int nsb) {
   char* p = static_cast<char*>(base);
   Work w;
   w.q = reinterpret_cast<unsigned long long*>(p); p += align_up(nnzb * 8);
   w.scale = reinterpret_cast<double*>(p); p += align_up(nseg * 8);
-  w.nz = reinterpret_cast<int32_t*>(p); p += align_up((size_t)nsb * nsb * 4);
+  w.nz = reinterpret_cast<int32_t*>(p); p += align_up(nz_bytes(nsb));
   w.m = reinterpret_cast<int32_t*>(p); p += align_up((size_t)nsb * 4);
   w.nseg = nseg;
   w.nsb = nsb;
@@ -73,6 +76,7 @@ __global__ void k_nz(const int32_t* __restrict__ brow, const int32_t* __restrict
   const int R = brow[t] / pt, C = bcol[t] / pt;
   nz[(int64_t)R * nsb + C] = 1;
   nz[(int64_t)C * nsb + R] = 1;
+  if (bcol[t] < brow[t] || (t > 0 && brow[t - 1] > brow[t])) nz[(int64_t)nsb * nsb] = 1;
 }
 
 __global__ void k_m(const int32_t* __restrict__ nz, int nsb, int32_t* m) {
@@ -142,6 +146,9 @@ __device__ __forceinline__ int digit_of(unsigned long long hi, uint32_t lo, int 
 // segment (R, C), R <= C, of the upper triangle of nsb x nsb super-blocks).
 // The tiles are sorted by row, so the segment's tiles lie in the range of its
 // super-row (all of them in mode 0); the CTAs of the cluster split that range.
+// Tiles in another order, or below the diagonal, are no sp2_bsr, but a selection
+// needs neither: with such a tile every segment reads the whole set, and
+// those with R > C take part.
 // Digits: the 12 bits of sign and exponent first (a tile set spans some 100
 // octaves, so the shared-memory atomics of a warp rarely meet in one bin),
 // 11 bits at a time after that.
@@ -172,7 +179,7 @@ __device__ __forceinline__ int64_t first_row_ge(const int32_t* __restrict__ brow
 }
 
 template <int CTAS, int THREADS>
-__global__ void __cluster_dims__(CTAS, 1, 1) __launch_bounds__(THREADS)
+__global__ void __cluster_dims__(CTAS, 1, 1) __launch_bounds__(THREADS, 1024 / THREADS)
     k_trunc_cluster(const int32_t* __restrict__ brow, const int32_t* __restrict__ bcol,
                     const int32_t* __restrict__ slot, const double* __restrict__ n2,
                     const unsigned long long* __restrict__ q, const int32_t* __restrict__ nz, int64_t nnzb, int nb,
@@ -188,12 +195,17 @@ __global__ void __cluster_dims__(CTAS, 1, 1) __launch_bounds__(THREADS)
   cg::cluster_group cl = cg::this_cluster();
   const int rank = (int)cl.block_rank();
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  int C = 0;
+  int C = 0, row0 = -1;      // the segment's super-column; its first row where the range does not say it
+  auto inside = [&](int64_t t) {
+    return bcol[t] / pt == C && (row0 < 0 || (unsigned)(brow[t] - row0) < (unsigned)pt);
+  };
   if (mode == 1) {
     const int R = (int)blockIdx.y;
     C = (int)(blockIdx.x / CTAS);
-    if (C < R || nz[(int64_t)R * nsb + C] == 0) return;     // the whole cluster
-    if (tid < 2) range[tid] = first_row_ge(brow, nnzb, (R + tid) * pt);
+    const bool has = nz[(int64_t)R * nsb + C] != 0, any_order = nz[(int64_t)nsb * nsb] != 0;
+    if (!has || (C < R && !any_order)) return;     // the whole cluster
+    if (any_order) row0 = R * pt;
+    if (tid < 2) range[tid] = any_order ? tid * nnzb : first_row_ge(brow, nnzb, (R + tid) * pt);
   } else if (tid == 0) {
     range[0] = 0;
     range[1] = nnzb;
@@ -213,7 +225,7 @@ __global__ void __cluster_dims__(CTAS, 1, 1) __launch_bounds__(THREADS)
     unsigned long long s = 0ull;
     uint32_t n = 0u;
     for (int64_t t = c0 + tid; t < c1; t += THREADS)
-      if (bcol[t] / pt == C) {
+      if (inside(t)) {
         s += q[t];
         ++n;
       }
@@ -261,7 +273,7 @@ __global__ void __cluster_dims__(CTAS, 1, 1) __launch_bounds__(THREADS)
           lo = (uint32_t)brow[t] * (uint32_t)nb + (uint32_t)bcol[t];
           if (p > 6) in = (lo >> psh) == pl;
         }
-        if (in && mode == 1) in = bcol[t] / pt == C;
+        if (in && mode == 1) in = inside(t);
         if (in) {
           const uint32_t d = (p < 6 ? (uint32_t)(hi >> sh) : lo >> sh) & dm;
           atomicAdd(&hist[d], q[t]);
@@ -341,7 +353,7 @@ __global__ void __cluster_dims__(CTAS, 1, 1) __launch_bounds__(THREADS)
   const int dsh = depth > 0 ? cl_shift(depth - 1) : 0;
 #pragma unroll 4
   for (int64_t t = c0 + tid; t < c1; t += THREADS) {
-    if (mode == 1 && bcol[t] / pt != C) continue;
+    if (mode == 1 && !inside(t)) continue;
     const unsigned long long hi = __double_as_longlong(n2[slot ? slot[t] : t]);
     bool less, equal;
     if (depth == 0) {
@@ -556,7 +568,7 @@ cudaError_t launch_tile_norms(const double* val, int64_t nnzb, double* n2, cudaS
 size_t trunc_work_bytes(int64_t nnzb, int nb, int64_t part_tiles) {
   const int nsb = (int)((nb + part_tiles - 1) / part_tiles);
   const int64_t nseg = (int64_t)nsb * nsb;
-  return align_up(nnzb * 8) + align_up(nseg * 8) + align_up((size_t)nsb * nsb * 4) + align_up((size_t)nsb * 4) + 1024;
+  return align_up(nnzb * 8) + align_up(nseg * 8) + align_up(nz_bytes(nsb)) + align_up((size_t)nsb * 4) + 1024;
 }
 
 // x: the tiles of X_i (slot indexes n2); n2[slot] = ||X_i tile||_F^2; keep[t] out.
@@ -575,7 +587,7 @@ cudaError_t launch_truncate(const TileSet& x, const double* n2, int nb, double t
   const int md = nseg == 1 ? 0 : 1;   // mode 1 with a single super-block has m = 1: budget tau^2 as in mode 0
   double sc = 0.0;
   if (md == 1) {
-    const cudaError_t e = cudaMemsetAsync(w.nz, 0, (size_t)nsb * nsb * 4, st);
+    const cudaError_t e = cudaMemsetAsync(w.nz, 0, nz_bytes(nsb), st);
     if (e != cudaSuccess) return e;
     { ++g_launches; k_nz<<<grid_for(nnzb, 256), 256, 0, st>>>(x.brow, x.bcol, nnzb, (int)part_tiles, nsb, w.nz); }
     { ++g_launches; k_m<<<grid_for(nsb, 128), 128, 0, st>>>(w.nz, nsb, w.m); }

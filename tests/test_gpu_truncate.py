@@ -158,6 +158,27 @@ def test_more_super_blocks_than_a_32_bit_segment_index_holds():
     sp2.load().sp2_release_memory()      # 26 GB of segment tables
 
 
+@pytest.mark.parametrize("n,mode,part", [(2030, "frobinf", 256), (331, "frobinf", 32), (5900, "frobinf", 3008),
+                                         (2030, "frobenius", 4096)])
+def test_tiles_in_any_order_and_below_the_diagonal(n, mode, part):
+    """The selection does not depend on the order of the tiles, nor on which of the
+    two places (I, J), (J, I) an off-diagonal tile is given at (its norm and its
+    segment's budget are the same): shuffled tiles, tiles stored below the
+    diagonal, and both, in the one-CTA, the cluster and the small select."""
+    import paper_1909_12533_gb300 as sp2
+    X = _decaying(n, 29)
+    o = _oracle_keep(X, 1e-2, mode, part)
+    pt = part // 32 if mode == "frobinf" else 1
+    below = (X.brow // pt + X.bcol // pt) % 3 == 0      # whole segments: each has its own budget
+    perm = np.random.default_rng(3).permutation(X.nnzb)
+    for order, swap in ((perm, False), (np.arange(X.nnzb), True), (perm, True)):
+        s = below & swap
+        Y = BlockSparse(n=n, brow=np.where(s, X.bcol, X.brow)[order], bcol=np.where(s, X.brow, X.bcol)[order],
+                        val=X.val[order])
+        g = sp2.sp2_truncate(Y, 1e-2, mode, part)
+        assert np.array_equal(g, o[order]), (order is perm, swap, np.nonzero(g != o[order]))
+
+
 # ----------------------------------------------------------------- mixed norm (Section 3)
 @pytest.mark.parametrize("part", [64, 128, 4096])
 @pytest.mark.parametrize("tau", [0.0, 1e-6, 1e-3, 0.1])
