@@ -155,11 +155,19 @@ __device__ __forceinline__ int digit_of(unsigned long long hi, uint32_t lo, int 
 // Two sizes: CL_CTAS x 1024 threads for segments of many tiles, one CTA of 256
 // threads for small ones (Frob-Inf with a small partition has thousands, most
 // of them without a tile, which leave at once, and most others with one tile or
-// within their budget, which need no histogram: one truncation of 178,230
-// tiles of a band in 3,000 x 3,000 segments takes 14.9 ms, in 750 x 750 1.7;
-// with a histogram for every pair of super-rows 139.8 and 9.9).
+// within their budget, or with few tiles, which need no histogram: one
+// truncation of 178,230 tiles of a band in 3,000 x 3,000 segments takes 14.9 ms,
+// in 750 x 750 1.4, of 131,328 tiles of a dense matrix in 256 x 256 0.8; with a
+// histogram for every pair of super-rows 139.8, 9.9 and 2.5).
 constexpr int CL_CTAS = 8;
 constexpr int64_t CL_MANY = 4096;   // tiles of a segment (mean) from which the cluster is taken
+// Tiles of a segment up to which the one-CTA select compares them with one
+// another: 131,328 tiles in segments of 16 take 0.56 ms (1.06 with histograms),
+// 8,256 tiles in segments of up to 256 128 us (111).
+constexpr int DIRECT_MAX = 64;
+// Tiles of a super-row up to which that select sums its segment first; the sum
+// reads the range once more (39,765 tiles in six super-rows: 258 us with it, 238).
+constexpr int64_t SUM_FIRST_MAX = 4096;
 constexpr int CL_BINS = 4096;
 constexpr int CL_PASSES = 9;      // 6 over the norm (52, 41, 30, 19, 8, 0), 3 over the index (21, 10, 0)
 constexpr size_t CL_SMEM = (size_t)CL_BINS * 12;
@@ -220,7 +228,7 @@ __global__ void __cluster_dims__(CTAS, 1, 1) __launch_bounds__(THREADS, 1024 / T
   int depth = 0;       // digits fixed in (ph, pl)
   bool all = false;    // every remaining candidate fits
   bool open = true;    // the cut is still to be found
-  if (CTAS == 1) {
+  if (CTAS == 1 && c1 - c0 <= SUM_FIRST_MAX) {
     // the segment's units and tiles: all fit, or the only one does not
     unsigned long long s = 0ull;
     uint32_t n = 0u;
@@ -244,6 +252,34 @@ __global__ void __cluster_dims__(CTAS, 1, 1) __launch_bounds__(THREADS, 1024 / T
     }
     all = s <= rem;
     open = !all && n > 1u;
+    if (open && n <= (uint32_t)DIRECT_MAX) {
+      // few tiles: each thread adds up the units of the tiles that are not behind
+      // its own in the order of the keys
+      unsigned long long* th = hist;                   // squared norms
+      unsigned long long* tq = hist + DIRECT_MAX;      // units
+      uint32_t* tl = cnt + DIRECT_MAX;                 // linear tile indices
+      uint32_t* tt = cnt + 2 * DIRECT_MAX;             // tiles
+      if (tid == 0) s_cnt = 0;
+      __syncthreads();
+      for (int64_t t = c0 + tid; t < c1; t += THREADS)
+        if (inside(t)) {
+          const int k = atomicAdd(&s_cnt, 1);
+          th[k] = (unsigned long long)__double_as_longlong(n2[slot ? slot[t] : t]);
+          tq[k] = q[t];
+          tl[k] = (uint32_t)brow[t] * (uint32_t)nb + (uint32_t)bcol[t];
+          tt[k] = (uint32_t)t;
+        }
+      __syncthreads();
+      if (tid < (int)n) {
+        const unsigned long long hi = th[tid];
+        const uint32_t lo = tl[tid];
+        unsigned long long sum = 0ull;
+        for (uint32_t k = 0; k < n; ++k)
+          if (th[k] < hi || (th[k] == hi && tl[k] <= lo)) sum += tq[k];
+        keep[tt[tid]] = sum <= rem ? 0 : 1;
+      }
+      return;
+    }
     __syncthreads();
   }
   for (int p = 0; open && p < CL_PASSES; ++p) {

@@ -179,6 +179,20 @@ def test_tiles_in_any_order_and_below_the_diagonal(n, mode, part):
         assert np.array_equal(g, o[order]), (order is perm, swap, np.nonzero(g != o[order]))
 
 
+@pytest.mark.parametrize("part,tau", [(64, 0.3), (256, 0.3), (352, 0.3), (384, 0.3), (384, 1e-3)])
+def test_keep_flags_of_segments_around_the_direct_limit(part, tau):
+    """Segments of at most 4, 64, 121 and 144 tiles (the diagonal ones 3, 36, 66 and
+    78): up to 64 tiles are compared with one another, more take histograms; equal
+    norms and zero tiles among them."""
+    import paper_1909_12533_gb300 as sp2
+    X = _decaying(2030, 37, ties=True)
+    X.val[[11, 400, 401, 900]] = 0.0
+    g = sp2.sp2_truncate(X, tau, "frobinf", part)
+    o = _oracle_keep(X, tau, "frobinf", part)
+    assert np.array_equal(g, o), np.nonzero(g != o)
+    assert 0 < g.sum() < X.nnzb
+
+
 # ----------------------------------------------------------------- mixed norm (Section 3)
 @pytest.mark.parametrize("part", [64, 128, 4096])
 @pytest.mark.parametrize("tau", [0.0, 1e-6, 1e-3, 0.1])
