@@ -29,6 +29,20 @@ __global__ void k_bitmap(const int32_t* __restrict__ brow, const int32_t* __rest
   atomicOr(&bits[(int64_t)j * words + (i >> 5)], 1u << (i & 31));
 }
 
+// One warp: wpre of row R (the set bits before each word) and the row's set bits.
+__device__ __forceinline__ int row_prefix(const uint32_t* __restrict__ bits, int words, int64_t R, int32_t* wpre) {
+  const int lane = threadIdx.x & 31;
+  int base = 0;
+  for (int w0 = 0; w0 < words; w0 += 32) {
+    const int w = w0 + lane;
+    const int c = w < words ? __popc(bits[R * words + w]) : 0;
+    const int inc = warp_incl_scan(c);
+    if (w < words) wpre[R * words + w] = base + inc - c;
+    base += __shfl_sync(0xffffffffu, inc, 31);
+  }
+  return base;
+}
+
 // One cluster: wpre[R][w] = set bits of row R before word w, rowptr = exclusive
 // prefix sums of the rows' set bits (one warp per row, then a scan over the
 // rows; a count kernel and a one- or three-launch scan did this before).
@@ -44,17 +58,10 @@ __global__ void __cluster_dims__(SCAN_CTAS, 1, 1) __launch_bounds__(SCAN_THREADS
   const int lane = threadIdx.x & 31;
   int sum = 0;
   for (int R = c0 + (int)(threadIdx.x >> 5); R < c1; R += SCAN_THREADS / 32) {
-    int base = 0;
-    for (int w0 = 0; w0 < words; w0 += 32) {
-      const int w = w0 + lane;
-      const int c = w < words ? __popc(bits[(int64_t)R * words + w]) : 0;
-      const int inc = warp_incl_scan(c);
-      if (w < words) wpre[(int64_t)R * words + w] = base + inc - c;
-      base += __shfl_sync(0xffffffffu, inc, 31);
-    }
+    const int count = row_prefix(bits, words, R, wpre);
     if (lane == 0) {
-      rowptr[R] = base;
-      sum += base;
+      rowptr[R] = count;
+      sum += count;
     }
   }
   int mine;
@@ -75,6 +82,26 @@ __global__ void __cluster_dims__(SCAN_CTAS, 1, 1) __launch_bounds__(SCAN_THREADS
     carry += block;
   }
   if (rank == 0 && threadIdx.x == 0) {
+    rowptr[nb] = all;
+    if (total) *total = all;
+  }
+}
+
+// The same for bitmaps of more than ROWS_CLUSTER_MAX words, which one cluster reads
+// too slowly: the rows over all multiprocessors, then their counts in one cluster.
+__global__ void __launch_bounds__(256) k_row_counts(const uint32_t* __restrict__ bits, int nb, int words,
+                                                    int32_t* wpre, int32_t* rowptr) {
+  const int64_t R = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+  if (R >= nb) return;
+  const int count = row_prefix(bits, words, R, wpre);
+  if ((threadIdx.x & 31) == 0) rowptr[R] = count;
+}
+
+__global__ void __cluster_dims__(SCAN_CTAS, 1, 1) __launch_bounds__(SCAN_THREADS)
+    k_row_offsets(int nb, int32_t* rowptr, int32_t* total) {
+  const int all = cluster_scan(
+      nb, [&](int64_t R) { return rowptr[R]; }, [&](int64_t R, int, int ex) { rowptr[R] = ex; });
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
     rowptr[nb] = all;
     if (total) *total = all;
   }
@@ -278,6 +305,11 @@ __global__ void k_check_finite(const double* __restrict__ val, int64_t count, in
 
 inline unsigned grid_for(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
 
+// Words of a bitmap up to which one cluster scans it; above, two launches.  One
+// cluster -> two launches: 53,300 words 10.1 -> 10.3 us, 126,000 11.8 -> 10.3,
+// 1.1 million (N = 192,000) 51 -> 12, 134 million (65,535 tile rows) 6,900 -> 174.
+constexpr int64_t ROWS_CLUSTER_MAX = 1 << 16;
+
 }  // namespace
 
 size_t scan_tmp_bytes(int64_t n) {
@@ -312,8 +344,15 @@ cudaError_t launch_bitmap(const TileSet& s, int nb, FullPattern& fp, cudaStream_
 
 cudaError_t launch_rows_scan(const uint32_t* bits, int nb, int words, int32_t* wpre, int32_t* rowptr, int32_t* total,
                              cudaStream_t st) {
+  if ((int64_t)nb * words <= ROWS_CLUSTER_MAX) {
+    ++g_launches;
+    k_rows_scan<<<SCAN_CTAS, SCAN_THREADS, 0, st>>>(bits, nb, words, wpre, rowptr, total);
+    return cudaGetLastError();
+  }
   ++g_launches;
-  k_rows_scan<<<SCAN_CTAS, SCAN_THREADS, 0, st>>>(bits, nb, words, wpre, rowptr, total);
+  k_row_counts<<<grid_for((int64_t)nb * 32, 256), 256, 0, st>>>(bits, nb, words, wpre, rowptr);
+  ++g_launches;
+  k_row_offsets<<<SCAN_CTAS, SCAN_THREADS, 0, st>>>(nb, rowptr, total);
   return cudaGetLastError();
 }
 

@@ -542,6 +542,58 @@ __global__ void __cluster_dims__(SCAN_CTAS, 1, 1) __launch_bounds__(SCAN_THREADS
   }
 }
 
+// The same for more than SUPER_CLUSTER_MAX words: one warp per super-row over all
+// multiprocessors writes its bitmap and, in its first offset, its set bits; one
+// cluster scans those; the warps then write the offsets.
+__global__ void __launch_bounds__(256) k_super_counts(const uint32_t* __restrict__ bits, int nb, int words, int nsr,
+                                                      uint32_t* sb, int32_t* spos) {
+  const int64_t R = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
+  if (R >= nsr) return;
+  int c = 0;
+  for (int w = lane; w < words; w += 32) {
+    uint32_t m = 0;
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+      if (4 * R + a < nb) m |= bits[(4 * R + a) * words + w];
+    sb[R * words + w] = m;
+    c += __popc(m);
+  }
+  c = __reduce_add_sync(0xffffffffu, c);
+  if (lane == 0) spos[R * words] = c;
+}
+
+__global__ void __cluster_dims__(SCAN_CTAS, 1, 1) __launch_bounds__(SCAN_THREADS)
+    k_super_offsets(int words, int nsr, int32_t* spos, int32_t* total) {
+  const int all = cluster_scan(
+      nsr, [&](int64_t R) { return spos[R * words]; }, [&](int64_t R, int, int ex) { spos[R * words] = ex; });
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    spos[(int64_t)nsr * words] = all;
+    if (total) *total = all;
+  }
+}
+
+__global__ void __launch_bounds__(256) k_super_positions(const uint32_t* __restrict__ sb, int words, int nsr,
+                                                         int32_t* spos) {
+  const int64_t R = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
+  if (R >= nsr) return;
+  int base = spos[R * words];
+  __syncwarp();      // every lane has it before lane 0 writes that word again (the same value)
+  for (int w0 = 0; w0 < words; w0 += 32) {
+    const int w = w0 + lane;
+    const int c = w < words ? __popc(sb[R * words + w]) : 0;
+    int inc = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, inc, o);
+      if (lane >= o) inc += v;
+    }
+    if (w < words) spos[R * words + w] = base + inc - c;
+    base += __shfl_sync(0xffffffffu, inc, 31);
+  }
+}
+
 // Launch order of the super-tiles: blocks of RB super-rows x CB super-columns,
 // row-major inside a block, blocks row-major.  CTAs that run at the same time
 // then share A panels (same super-row) and B panels (same super-column), so the
@@ -1716,10 +1768,25 @@ cudaError_t launch_upper_bits(const TileSet& x, int nb, int words, uint32_t* bit
   return cudaGetLastError();
 }
 
+// Words of the super-row bitmaps up to which one cluster makes them; above, three
+// launches.  One cluster -> three launches: 31,500 words 10.3 -> 14.5 us, 49,375
+// 16.5 -> 14.4, 282,000 (N = 192,000) 53 -> 17, 34 million (65,535 tile rows) 5,700 -> 173.
+constexpr int64_t SUPER_CLUSTER_MAX = 1 << 15;
+
 cudaError_t launch_super_scan(const FullPattern& fp, int nb, int nsr, uint32_t* sb, int32_t* spos, int32_t* total,
                               cudaStream_t st) {
+  if ((int64_t)nsr * fp.words <= SUPER_CLUSTER_MAX) {
+    ++g_launches;
+    k_super_scan<<<SCAN_CTAS, SCAN_THREADS, 0, st>>>(fp.bits, nb, fp.words, nsr, sb, spos, total);
+    return cudaGetLastError();
+  }
+  const unsigned g = grid_for((int64_t)nsr * 32, 256);
   ++g_launches;
-  k_super_scan<<<SCAN_CTAS, SCAN_THREADS, 0, st>>>(fp.bits, nb, fp.words, nsr, sb, spos, total);
+  k_super_counts<<<g, 256, 0, st>>>(fp.bits, nb, fp.words, nsr, sb, spos);
+  ++g_launches;
+  k_super_offsets<<<SCAN_CTAS, SCAN_THREADS, 0, st>>>(fp.words, nsr, spos, total);
+  ++g_launches;
+  k_super_positions<<<g, 256, 0, st>>>(sb, fp.words, nsr, spos);
   return cudaGetLastError();
 }
 

@@ -68,6 +68,42 @@ def test_parity_around_the_split_tile_limit(n):
     assert np.linalg.norm(dF - G) <= 1e-10 * np.linalg.norm(G)
 
 
+@pytest.mark.parametrize("precision,tol", [("fp64", 1e-10), ("split16", 1e-6)])
+@pytest.mark.parametrize("nb", [1500, 2502])
+def test_many_tile_rows(nb, precision, tol):
+    # 1,500 tile rows: the row offsets of a bitmap of 70,500 words come from two
+    # launches; 2,502: so do the super-row bitmaps (49,454 words).  F is block
+    # diagonal, dense blocks of three tile rows (four kinds, the last one ragged), so
+    # D is block diagonal with the projectors of the blocks.
+    import paper_1909_12533_gb300 as sp2
+    n = 32 * nb - 7
+    nblk = nb // 3
+    kinds = [dense_gapped(96, 30 + 5 * k, (-2.0, -0.5), (0.5, 2.0), seed=900 + k) for k in range(4)]
+    kinds.append(dense_gapped(89, 41, (-2.0, -0.5), (0.5, 2.0), seed=904))
+    which = np.arange(nblk) % 4
+    which[-1] = 4
+    tiles, proj = [], []
+    for d in kinds:
+        lam, V = np.linalg.eigh(d["F"])
+        V = V[:, lam < 0]
+        tiles.append(from_dense(d["F"], keep_zero_tiles=True))
+        proj.append(from_dense(V @ V.T, keep_zero_tiles=True).val)
+    base = 3 * np.arange(nblk, dtype=np.int32)[:, None]
+    brow, bcol = (base + t.astype(np.int32) for t in (tiles[0].brow, tiles[0].bcol))
+    order = np.lexsort((bcol.ravel(), brow.ravel()))
+    F = BlockSparse(n=n, brow=brow.ravel()[order], bcol=bcol.ravel()[order],
+                    val=np.concatenate([tiles[k].val for k in which])[order])
+    nocc = int(sum(kinds[k]["nocc"] for k in which))
+    ctx = sp2.SP2(F, nocc, -0.5, 0.5, 0.0, stop="idempotency", precision=precision)
+    st = ctx.run()
+    gb, gc, gv = ctx.D_host()
+    ctx.close()
+    assert st["converged"] and set(st["nnzb_hist"]) == {6 * nblk}
+    assert np.array_equal(gb, F.brow) and np.array_equal(gc, F.bcol)
+    ref = np.concatenate([proj[k] for k in which])[order]
+    assert np.linalg.norm(gv - ref) <= tol, np.linalg.norm(gv - ref)
+
+
 def test_parity_frobinf_multiple_superblocks():
     c = _case("3s")
     kw = dict(trunc="frobinf", frobinf_part=1024)
