@@ -186,6 +186,39 @@ __device__ __forceinline__ int64_t first_row_ge(const int32_t* __restrict__ brow
   return lo;
 }
 
+// Adds the units q of the lanes with `in` to their bins d; the whole warp calls it.
+// Up to four bins that four or more lanes share take one addition each: the tiles
+// of a periodic system have equal norms, and then all additions of a pass meet in
+// a few bins.  One truncation without it, with it: 119,990 equal tiles 3.6 ms,
+// 0.54; 888,825 equal tiles 27.7, 3.2; 178,230 tiles of random norms 0.60 both.
+__device__ __forceinline__ void hist_add(unsigned long long* hist, uint32_t* cnt, bool in, uint32_t d,
+                                         unsigned long long q) {
+  constexpr unsigned FULLW = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  unsigned left = __ballot_sync(FULLW, in);
+  bool alone = in;
+  for (int r = 0; r < 4 && left != 0u; ++r) {
+    const int lead = __ffs(left) - 1;
+    const uint32_t d0 = __shfl_sync(FULLW, d, lead);      // every lane takes part
+    const bool same = in && d == d0;
+    const unsigned peers = __ballot_sync(FULLW, same);
+    left &= ~peers;
+    if (same && __popc(peers) >= 4) {
+      const unsigned lo = __reduce_add_sync(peers, (unsigned)q & 0x7FFFFu);      // q <= 2^37: both sums fit
+      const unsigned hi = __reduce_add_sync(peers, (unsigned)(q >> 19));
+      if (lane == lead) {
+        atomicAdd(&hist[d], ((unsigned long long)hi << 19) + lo);
+        atomicAdd(&cnt[d], (uint32_t)__popc(peers));
+      }
+      alone = false;
+    }
+  }
+  if (alone) {
+    atomicAdd(&hist[d], q);
+    atomicAdd(&cnt[d], 1u);
+  }
+}
+
 template <int CTAS, int THREADS>
 __global__ void __cluster_dims__(CTAS, 1, 1) __launch_bounds__(THREADS, 1024 / THREADS)
     k_trunc_cluster(const int32_t* __restrict__ brow, const int32_t* __restrict__ bcol,
@@ -290,7 +323,7 @@ __global__ void __cluster_dims__(CTAS, 1, 1) __launch_bounds__(THREADS, 1024 / T
     __syncthreads();
     const int sh = cl_shift(p), psh = p > 0 ? cl_shift(p - 1) : 0;
     const uint32_t dm = p == 0 ? 0xFFFu : p == 5 ? 0xFFu : p == 8 ? 0x3FFu : 0x7FFu;
-    for (int64_t t0 = c0 + tid; t0 < c1; t0 += MLP * THREADS) {
+    for (int64_t t0 = c0 + tid; t0 - lane < c1; t0 += MLP * THREADS) {      // whole warps
       unsigned long long h[MLP];
 #pragma unroll
       for (int u = 0; u < MLP; ++u) {
@@ -310,11 +343,7 @@ __global__ void __cluster_dims__(CTAS, 1, 1) __launch_bounds__(THREADS, 1024 / T
           if (p > 6) in = (lo >> psh) == pl;
         }
         if (in && mode == 1) in = inside(t);
-        if (in) {
-          const uint32_t d = (p < 6 ? (uint32_t)(hi >> sh) : lo >> sh) & dm;
-          atomicAdd(&hist[d], q[t]);
-          atomicAdd(&cnt[d], 1u);
-        }
+        hist_add(hist, cnt, in, (p < 6 ? (uint32_t)(hi >> sh) : lo >> sh) & dm, in ? q[t] : 0ull);
       }
     }
     cl.sync();

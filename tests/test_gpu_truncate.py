@@ -193,6 +193,26 @@ def test_keep_flags_of_segments_around_the_direct_limit(part, tau):
     assert 0 < g.sum() < X.nnzb
 
 
+@pytest.mark.parametrize("mode,part", [("frobenius", 4096), ("frobinf", 704), ("frobinf", 1056)])
+@pytest.mark.parametrize("classes", [1, 2, 6])
+def test_many_tiles_of_equal_norm(mode, part, classes):
+    """All norms are equal, or one of a few that alternate along the rows (what a
+    periodic system has): the lanes of a warp share their bins, and the cut lies
+    among equal norms, so the index decides."""
+    import paper_1909_12533_gb300 as sp2
+    n = 2100
+    nb = (n + 31) // 32
+    i, j = np.triu_indices(nb)
+    val = np.zeros((i.size, 32, 32))
+    val[:, 0, 0] = 1.0 + 0.25 * ((j - i) % classes)
+    X = BlockSparse(n=n, brow=i.astype(np.int32), bcol=j.astype(np.int32), val=val)
+    for tau in (3.0, 31.0, 61.0):
+        g = sp2.sp2_truncate(X, tau, mode, part)
+        o = _oracle_keep(X, tau, mode, part)
+        assert np.array_equal(g, o), (tau, np.nonzero(g != o))
+        assert 0 < g.sum() < g.size
+
+
 # ----------------------------------------------------------------- mixed norm (Section 3)
 @pytest.mark.parametrize("part", [64, 128, 4096])
 @pytest.mark.parametrize("tau", [0.0, 1e-6, 1e-3, 0.1])
