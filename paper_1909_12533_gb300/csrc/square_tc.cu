@@ -1472,35 +1472,38 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_square_tc(TcArgs a) {
           const int row0 = bt * 32 + hc * 16;
           long long fx[16];
           long long* sp = scr + row0 * ST;
-#pragma unroll
-          for (int i = 0; i < 16; ++i) fx[i] = 0;
           const uint32_t trow = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)row0;
+          // The group sums are integers.  With two to four slices nothing bounds them by
+          // 2^31: second slices reach 2^10, and a K loop without segments has thousands
+          // of products of each of a group's pairs, all of one sign on a diagonal that
+          // does not come from dsq or between alike rows.  A chunk with such a sum is
+          // read again with the 64-bit conversion (one test a chunk costs nothing that
+          // shows; a test before the conversion of each group cost 0.4% to 0.9% of a run).
+          // Five slices: 256 products a segment of at most 2^20 + 3 2^18, below 2^29.
+          float top = 0.0f;
+          for (bool wide = false;; wide = true) {
+#pragma unroll
+            for (int i = 0; i < 16; ++i) fx[i] = 0;
 #pragma unroll 1
-          for (int gg = 0; gg <= ghi - glo; ++gg) {   // relative groups of the window, coarsest first
+            for (int gg = 0; gg <= ghi - glo; ++gg) {   // relative groups of the window, coarsest first
 #pragma unroll
-            for (int i = 0; i < 16; ++i) fx[i] *= 1ll << W;
-            if ((written >> gg) & 1u) {        // warp-uniform: groups no product reached are zero
-              float g[16];
-              tmem_ld16(trow + ((gm >> (8 + 2 * gg)) & 3u) * ST, g);
-              // Integers, exact either way.  With two to four slices nothing bounds a group
-              // sum by 2^31: second slices reach 2^10, and a K loop without segments has
-              // thousands of products of each of a group's pairs, all of one sign on a
-              // diagonal that does not come from dsq or between alike rows.  Such tiles
-              // take the 64-bit conversion.  (Five slices: 256 products a segment of at
-              // most 2^20 + 3 2^18, below 2^29.)
-              float top = 0.0f;
-              if (K != 5) {
+              for (int i = 0; i < 16; ++i) fx[i] *= 1ll << W;
+              if ((written >> gg) & 1u) {        // warp-uniform: groups no product reached are zero
+                float g[16];
+                tmem_ld16(trow + ((gm >> (8 + 2 * gg)) & 3u) * ST, g);
+                if (K != 5 && wide) {
 #pragma unroll
-                for (int i = 0; i < 16; ++i) top = fmaxf(top, fabsf(g[i]));
-              }
-              if (K != 5 && __any_sync(FULLW, top >= 2147483648.0f)) {
+                  for (int i = 0; i < 16; ++i) fx[i] += __float2ll_rn(g[i]);
+                } else {
 #pragma unroll
-                for (int i = 0; i < 16; ++i) fx[i] += __float2ll_rn(g[i]);
-              } else {
-#pragma unroll
-                for (int i = 0; i < 16; ++i) fx[i] += __float2int_rn(g[i]);
+                  for (int i = 0; i < 16; ++i) {
+                    if (K != 5) top = fmaxf(top, fabsf(g[i]));
+                    fx[i] += __float2int_rn(g[i]);
+                  }
+                }
               }
             }
+            if (K == 5 || wide || !__any_sync(FULLW, top >= 2147483648.0f)) break;
           }
           if (!first) {
 #pragma unroll
