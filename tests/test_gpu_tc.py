@@ -141,10 +141,11 @@ def test_split16_fp64_tail_reaches_idempotency_tolerance():
     assert all(p == 1 for p in g0["stats"]["prec_hist"])
 
 
-@pytest.mark.parametrize("key,extra", [(1, {}), ("2s", {}), ("3s", {}), ("4s", {}),
-                                       ("5s", {"acc_flush_min": 1}), ("2s", {"storage": "general"})])
-def test_split_supply_gives_the_same_result(key, extra):
-    # both values of the parameter are accepted and give the same bits
+@pytest.mark.parametrize("key,extra", [("3s", {}), ("5s", {"acc_flush_min": 1})])
+def test_split16_runs_repeat_bit_for_bit(key, extra):
+    # the super-tiles are taken from a work counter and the sums meet in a fixed
+    # order: two runs give the same bits.  split_supply is accepted with both its
+    # values and has no effect
     c = make_config(key)
     kw = dict(stop=c["stop"], precision="split16", slices=4, **extra)
     a = run_gpu(c["F"], c["nocc"], c["homo_ub"], c["lumo_lb"], c["tau"], split_supply=0, **kw)
@@ -192,17 +193,18 @@ def test_split16_diagonal_of_the_square_in_fp64():
         assert d <= tol
 
 
-@pytest.mark.parametrize("n", [2000, 6001])
-def test_split16_group_sums_above_2_31_of_alike_rows(n):
+@pytest.mark.parametrize("n,flush", [(2000, 512), (2000, 1), (6001, 512), (6001, 0)])
+def test_split16_group_sums_above_2_31_of_alike_rows(n, flush):
     # F = -11^T / n, one delocalised orbital: D = -F, every row alike, so the products
     # of the second slices add up with one sign and the FP32 sum of their group
     # (three slice pairs, unit 2^-42) passes 2^31 in the last squares.  It stays below
     # 2^33: each of its 3 n / 16 additions rounds by at most 2^8 units, and the last
     # two squares have sums of this size.  (Clamped at 2^31: 2e-7 in every element.)
+    # With flush = 1 the K loop has segments of 16 K tiles, whose sums stay below 2^31.
     import torch
     import paper_1909_12533_gb300 as sp2
     F = torch.full((n, n), -1.0 / n, dtype=torch.float64, device="cuda")
-    D, st = sp2.run(F, 1, -0.9, -0.1, 0.0, precision="split16", slices=4)
+    D, st = sp2.run(F, 1, -0.9, -0.1, 0.0, precision="split16", slices=4, acc_flush_min=flush)
     err = float((D + F).abs().max())
     print(f"n = {n}: max |D - D_ref| = {err:.3e}, n = {st['n']}")
     assert st["converged"] and all(p == 1 for p in st["prec_hist"])
