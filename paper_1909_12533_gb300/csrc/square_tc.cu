@@ -286,6 +286,16 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
   for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+__device__ __forceinline__ void tmem_ld4(uint32_t taddr, float* v) {
+  uint32_t r[4];
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(taddr));
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int i = 0; i < 4; ++i) v[i] = __uint_as_float(r[i]);
+}
+
 // ------------------------------------------------------------------ slicing
 constexpr int PANEL_BYTES = 4 * SLICE_BYTES;   // one slice of the 4 tiles of a record
 
@@ -1467,43 +1477,38 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_square_tc(TcArgs a) {
         tc_fence_after();
         const uint32_t gm = gmap[q];
         const uint32_t written = gm & 0xFu;
+        // The group sums are integers, converted by the 32-bit instruction, which
+        // saturates.  With two to four slices nothing bounds them by 2^31: second
+        // slices reach 2^10, and a K loop without segments has thousands of products
+        // of each of a group's pairs, all of one sign on a diagonal that does not come
+        // from dsq or between alike rows.  A warp that met such a sum adds what the
+        // conversion lost afterwards; the vote on that stands where the warp has to
+        // meet anyway.  Squares of the water-like N = 192,000 case: 1,327 ms without a
+        // test (and wrong sums), 1,331 so, 1,337 with a vote after each 16 rows, and a
+        // vote before each group's conversion cost whole runs 0.4% to 0.9%.  Five
+        // slices: 256 products a segment of at most 2^20 + 3 2^18, below 2^29.
+        float top = 0.0f;
 #pragma unroll 1
         for (int hc = 0; hc < 2 && oi >= 0; ++hc) {       // 16 rows at a time
           const int row0 = bt * 32 + hc * 16;
           long long fx[16];
           long long* sp = scr + row0 * ST;
+#pragma unroll
+          for (int i = 0; i < 16; ++i) fx[i] = 0;
           const uint32_t trow = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)row0;
-          // The group sums are integers.  With two to four slices nothing bounds them by
-          // 2^31: second slices reach 2^10, and a K loop without segments has thousands
-          // of products of each of a group's pairs, all of one sign on a diagonal that
-          // does not come from dsq or between alike rows.  A chunk with such a sum is
-          // read again with the 64-bit conversion (one test a chunk costs nothing that
-          // shows; a test before the conversion of each group cost 0.4% to 0.9% of a run).
-          // Five slices: 256 products a segment of at most 2^20 + 3 2^18, below 2^29.
-          float top = 0.0f;
-          for (bool wide = false;; wide = true) {
-#pragma unroll
-            for (int i = 0; i < 16; ++i) fx[i] = 0;
 #pragma unroll 1
-            for (int gg = 0; gg <= ghi - glo; ++gg) {   // relative groups of the window, coarsest first
+          for (int gg = 0; gg <= ghi - glo; ++gg) {   // relative groups of the window, coarsest first
 #pragma unroll
-              for (int i = 0; i < 16; ++i) fx[i] *= 1ll << W;
-              if ((written >> gg) & 1u) {        // warp-uniform: groups no product reached are zero
-                float g[16];
-                tmem_ld16(trow + ((gm >> (8 + 2 * gg)) & 3u) * ST, g);
-                if (K != 5 && wide) {
+            for (int i = 0; i < 16; ++i) fx[i] *= 1ll << W;
+            if ((written >> gg) & 1u) {        // warp-uniform: groups no product reached are zero
+              float g[16];
+              tmem_ld16(trow + ((gm >> (8 + 2 * gg)) & 3u) * ST, g);
 #pragma unroll
-                  for (int i = 0; i < 16; ++i) fx[i] += __float2ll_rn(g[i]);
-                } else {
-#pragma unroll
-                  for (int i = 0; i < 16; ++i) {
-                    if (K != 5) top = fmaxf(top, fabsf(g[i]));
-                    fx[i] += __float2int_rn(g[i]);
-                  }
-                }
+              for (int i = 0; i < 16; ++i) {
+                if (K != 5) top = fmaxf(top, fabsf(g[i]));
+                fx[i] += __float2int_rn(g[i]);
               }
             }
-            if (K == 5 || wide || !__any_sync(FULLW, top >= 2147483648.0f)) break;
           }
           if (!first) {
 #pragma unroll
@@ -1512,9 +1517,27 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_square_tc(TcArgs a) {
 #pragma unroll
           for (int i = 0; i < 16; ++i) st_staging(sp + i * ST, fx[i], pol);
         }
-        // this warp's TMEM reads of the segment are complete
+        // this warp's TMEM reads of the segment are complete (the vote is also the
+        // warp's barrier)
         tc_fence_before();
-        __syncwarp();
+        if (__any_sync(FULLW, K != 5 && top >= 2147483648.0f)) {
+#pragma unroll 1
+          for (int u = 0; u < 8 * (ghi - glo + 1); ++u) {       // 4 rows of a group at a time
+            const int gg = u >> 3, row0 = bt * 32 + (u & 7) * 4;
+            if (!((written >> gg) & 1u)) continue;
+            float g[4];
+            tmem_ld4(tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)row0 + ((gm >> (8 + 2 * gg)) & 3u) * ST, g);
+            long long* sp = scr + row0 * ST;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              const long long lost = __float2ll_rn(g[i]) - __float2int_rn(g[i]);
+              if (lost != 0)
+                st_staging(sp + i * ST, ld_staging(sp + i * ST, pol) + lost * (1ll << (W * (ghi - glo - gg))), pol);
+            }
+          }
+          tc_fence_before();
+          __syncwarp();
+        }
         if (lane == 0) mbar_arrive(&tmem_empty[q]);
         ++seg;
         if (gm & SEG_LAST) break;
