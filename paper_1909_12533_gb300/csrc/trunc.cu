@@ -99,17 +99,20 @@ __global__ void k_seg_scale(Work w, double tau) {
 }
 
 // budget units of a tile of squared norm v and weight wt (1: stored once, 2: mirrored),
-// at most Q_CAP, which no budget holds: also for a NaN (a tile with a NaN, a
-// norm that was never computed), so that the sums of a selection stay below
-// 2^64 (2^27 tiles are a terabyte) and exactly one bin holds its cut.  A NaN
+// rounded up, at most Q_CAP, which no budget holds: also for a NaN (a tile with a
+// NaN, a norm that was never computed), so that the sums of a selection stay
+// below 2^64 (2^27 tiles are a terabyte) and exactly one bin holds its cut.  A NaN
 // converted to an integer would be 2^63 units, a wrapped sum would let several
 // CTAs of a cluster name a cut, and one could leave while another still reads
 // its shared memory.  A zero tile has no units, whatever the scale (infinite
-// for a tau whose square is subnormal).
+// for a tau whose square is subnormal).  The comparisons are made on the bit
+// patterns (those of 2^37 and above, of NaN and of negative values are not below
+// that of 2^37): the FP64 pipe compares two lanes a cycle.
 __device__ __forceinline__ unsigned long long budget_units(double v, double wt, double sc) {
-  if (v == 0.0) return 0ull;
-  const double x = (wt * v) * sc;
-  return sc != 0.0 && x < (double)Q_CAP ? (unsigned long long)ceil(x) : Q_CAP;
+  const unsigned long long x = (unsigned long long)__double_as_longlong((wt * v) * sc);
+  if (((unsigned long long)__double_as_longlong(v) << 1) == 0ull) return 0ull;
+  if (((unsigned long long)__double_as_longlong(sc) << 1) == 0ull || x >= (1023ull + 37ull) << 52) return Q_CAP;
+  return __double2ull_ru(__longlong_as_double((long long)x));
 }
 
 // mode 0: one segment, scale sc; mode 1: the segment's scale.  Its own launch
@@ -165,9 +168,9 @@ constexpr int64_t CL_MANY = 4096;   // tiles of a segment (mean) from which the 
 // another: 131,328 tiles in segments of 16 take 0.56 ms (1.06 with histograms),
 // 8,256 tiles in segments of up to 256 128 us (111).
 constexpr int DIRECT_MAX = 64;
-// Tiles of a super-row up to which that select sums its segment first; the sum
-// reads the range once more (39,765 tiles in six super-rows: 258 us with it, 238).
-constexpr int64_t SUM_FIRST_MAX = 4096;
+// Mean tiles of a segment up to which that select sums its segment first; the sum
+// reads the range once more (25,050 tiles in 55 segments: 152 us with it, 146).
+constexpr int64_t SUM_FIRST_MAX = 256;
 constexpr int CL_BINS = 4096;
 constexpr int CL_PASSES = 9;      // 6 over the norm (52, 41, 30, 19, 8, 0), 3 over the index (21, 10, 0)
 constexpr size_t CL_SMEM = (size_t)CL_BINS * 12;
@@ -186,24 +189,24 @@ __device__ __forceinline__ int64_t first_row_ge(const int32_t* __restrict__ brow
   return lo;
 }
 
-// Adds the units q of the lanes with `in` to their bins d; the whole warp calls it.
-// Up to four bins that four or more lanes share take one addition each: the tiles
-// of a periodic system have equal norms, and then all additions of a pass meet in
-// a few bins.  One truncation without it, with it: 119,990 equal tiles 3.6 ms,
-// 0.54; 888,825 equal tiles 27.7, 3.2; 178,230 tiles of random norms 0.60 both.
-__device__ __forceinline__ void hist_add(unsigned long long* hist, uint32_t* cnt, bool in, uint32_t d,
-                                         unsigned long long q) {
-  constexpr unsigned FULLW = 0xffffffffu;
+// Adds a candidate's units q to its bin d.  Up to four bins that `share` or more of
+// the candidates in the warp (the lanes that call this together) have take one
+// addition each; the search ends at the first bin that fewer have.  The tiles of
+// a periodic system have equal norms, and then all additions of a pass meet in a
+// few bins.  One truncation without it, with it: 119,990 equal tiles 3.6 ms, 0.54;
+// 888,825 equal tiles 27.7, 3.2; 178,230 tiles of random norms 0.537, 0.539.
+__device__ __forceinline__ void hist_add(unsigned long long* hist, uint32_t* cnt, uint32_t d, unsigned long long q, int share) {
+  const unsigned act = __activemask();
   const int lane = threadIdx.x & 31;
-  unsigned left = __ballot_sync(FULLW, in);
-  bool alone = in;
+  unsigned left = act;
+  bool alone = true;
   for (int r = 0; r < 4 && left != 0u; ++r) {
     const int lead = __ffs(left) - 1;
-    const uint32_t d0 = __shfl_sync(FULLW, d, lead);      // every lane takes part
-    const bool same = in && d == d0;
-    const unsigned peers = __ballot_sync(FULLW, same);
+    const uint32_t d0 = __shfl_sync(act, d, lead);
+    const unsigned peers = __ballot_sync(act, d == d0);
+    if (__popc(peers) < share) break;
     left &= ~peers;
-    if (same && __popc(peers) >= 4) {
+    if (d == d0) {
       const unsigned lo = __reduce_add_sync(peers, (unsigned)q & 0x7FFFFu);      // q <= 2^37: both sums fit
       const unsigned hi = __reduce_add_sync(peers, (unsigned)(q >> 19));
       if (lane == lead) {
@@ -224,7 +227,7 @@ __global__ void __cluster_dims__(CTAS, 1, 1) __launch_bounds__(THREADS, 1024 / T
     k_trunc_cluster(const int32_t* __restrict__ brow, const int32_t* __restrict__ bcol,
                     const int32_t* __restrict__ slot, const double* __restrict__ n2,
                     const unsigned long long* __restrict__ q, const int32_t* __restrict__ nz, int64_t nnzb, int nb,
-                    int mode, int pt, int nsb, int32_t* keep) {
+                    int mode, int pt, int nsb, int sum_first, int32_t* keep) {
   extern __shared__ __align__(16) unsigned char cl_smem[];
   unsigned long long* hist = reinterpret_cast<unsigned long long*>(cl_smem);   // [CL_BINS] units
   uint32_t* cnt = reinterpret_cast<uint32_t*>(hist + CL_BINS);                 // [CL_BINS] candidates
@@ -261,7 +264,7 @@ __global__ void __cluster_dims__(CTAS, 1, 1) __launch_bounds__(THREADS, 1024 / T
   int depth = 0;       // digits fixed in (ph, pl)
   bool all = false;    // every remaining candidate fits
   bool open = true;    // the cut is still to be found
-  if (CTAS == 1 && c1 - c0 <= SUM_FIRST_MAX) {
+  if (CTAS == 1 && sum_first) {
     // the segment's units and tiles: all fit, or the only one does not
     unsigned long long s = 0ull;
     uint32_t n = 0u;
@@ -323,7 +326,7 @@ __global__ void __cluster_dims__(CTAS, 1, 1) __launch_bounds__(THREADS, 1024 / T
     __syncthreads();
     const int sh = cl_shift(p), psh = p > 0 ? cl_shift(p - 1) : 0;
     const uint32_t dm = p == 0 ? 0xFFFu : p == 5 ? 0xFFu : p == 8 ? 0x3FFu : 0x7FFu;
-    for (int64_t t0 = c0 + tid; t0 - lane < c1; t0 += MLP * THREADS) {      // whole warps
+    for (int64_t t0 = c0 + tid; t0 < c1; t0 += MLP * THREADS) {
       unsigned long long h[MLP];
 #pragma unroll
       for (int u = 0; u < MLP; ++u) {
@@ -343,7 +346,7 @@ __global__ void __cluster_dims__(CTAS, 1, 1) __launch_bounds__(THREADS, 1024 / T
           if (p > 6) in = (lo >> psh) == pl;
         }
         if (in && mode == 1) in = inside(t);
-        hist_add(hist, cnt, in, (p < 6 ? (uint32_t)(hi >> sh) : lo >> sh) & dm, in ? q[t] : 0ull);
+        if (in) hist_add(hist, cnt, (p < 6 ? (uint32_t)(hi >> sh) : lo >> sh) & dm, q[t], p == 0 ? 8 : 4);
       }
     }
     cl.sync();
@@ -669,7 +672,8 @@ cudaError_t launch_truncate(const TileSet& x, const double* n2, int nb, double t
     if (e != cudaSuccess) return e;
     ++g_launches;
     kernel<<<dim3(side * ctas, side), threads, CL_SMEM, st>>>(x.brow, x.bcol, x.slot, n2, w.q, w.nz, nnzb, nb, md,
-                                                               (int)part_tiles, nsb, keep);
+                                                               (int)part_tiles, nsb,
+                                                               nnzb <= SUM_FIRST_MAX * nclus ? 1 : 0, keep);
     return cudaGetLastError();
   };
   return nnzb >= CL_MANY * nclus || nclus == 1 ? launch(k_trunc_cluster<CL_CTAS, 1024>, CL_CTAS, 1024)
